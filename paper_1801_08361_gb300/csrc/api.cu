@@ -364,7 +364,7 @@ relo_status run_pass(const RansacPass& p, cudaStream_t s, int* launches, cudaEve
   }
   if (p.n > 0) {
     RELO_CUDA(launch_compact(p.d_jobs, p.n, p.chunks, s));
-    RELO_CUDA(launch_hypotheses(p.d_jobs, p.n, p.hyps, p.d_counter, s, sched));
+    RELO_CUDA(launch_hypotheses(p.d_jobs, p.n, p.hyps, p.d_counter, s, sched, p.R * p.B));
     L += 4;
   }
   RELO_CUDA(record(ev_hyp, s, external));
@@ -373,7 +373,7 @@ relo_status run_pass(const RansacPass& p, cudaStream_t s, int* launches, cudaEve
     RELO_CUDA(launch_round(p.d_jobs, p.n, r, p.d_alive_prefix + (size_t)r * (p.n + 1), p.tot_alive[r],
                            p.max_alive[r], p.d_surv_prefix + (size_t)r * (p.n + 1), p.tot_surv[r], p.max_surv[r],
                            p.B, s, sched));
-    L += 5;
+    L += round_launches(p.n, p.max_alive[r], p.B);
   }
   if (p.n > 0) {
     RELO_CUDA(launch_finalise(p.d_jobs, p.n, s));
@@ -388,7 +388,7 @@ int pass_launches(const RansacPass& p, const Schedule& sched = Schedule()) {
   if (sched.persistent && p.d_items && p.n > 0) return 4;
   int L = p.n > 0 ? 5 : 0;
   for (int r = 0; r < p.R; ++r)
-    if (p.tot_alive[r] > 0) L += 5;
+    if (p.tot_alive[r] > 0) L += round_launches(p.n, p.max_alive[r], p.B);
   return L;
 }
 
@@ -1415,6 +1415,7 @@ relo_status relo_ransac_round(const relo_forest* f, const uint16_t* depth, const
   RELO_CUDA(cudaMemcpyAsync(s.d_surv, sp, sizeof(sp), cudaMemcpyHostToDevice, cs));
   RELO_CUDA(cudaMemsetAsync(j.err, 0, sizeof(int32_t), cs));
   RELO_CUDA(launch_compact(s.d_job, 1, s.chunks, cs));
+  RELO_CUDA(launch_draw(s.d_job, 1, round, s.d_alive, cs));
   RELO_CUDA(launch_round(s.d_job, 1, round, s.d_alive, n_alive, n_alive, s.d_surv, (n_alive + 1) / 2,
                          (n_alive + 1) / 2, p->batch, cs));
   return RELO_OK;

@@ -80,6 +80,119 @@ __device__ __forceinline__ void cam_point_d(int u, int v, int d, double fx, doub
 }
 
 // ---------------------------------------------------------------------------------------------
+// horn_pose (relo_internal.cuh) by 16 lanes, two solves per warp: lane 4 i + j of a half-warp holds
+// entries (i, j) of A and V.  The FP64 pipe takes many cycles per warp instruction however few lanes
+// are active, so one thread's solve (about 700 FP64 instructions a sweep) is bound by that pipe's
+// latency: 84-105 us whether one hypothesis or two thousand are re-fitted.  Sharing the entries among
+// lanes leaves about 200 a sweep, most of them the two rotations' angles, which both halves of the
+// columns take at once.  Every entry goes through horn_pose's operations in its order and rounding,
+// so both forms give the same bits.  Used where a launch has at most kGroupSolves solves; beyond,
+// the 32 solves a warp of the other form advances per instruction win.
+// ---------------------------------------------------------------------------------------------
+#ifndef RELO_GROUP_SOLVES
+#define RELO_GROUP_SOLVES 2048
+#endif
+constexpr int kGroupSolves = RELO_GROUP_SOLVES;
+constexpr int kSolvesPerWarp = 2;
+
+__device__ __forceinline__ double group_get(double v, int from) { return __shfl_sync(0xffffffffu, v, from, 16); }
+
+// S: the cross-covariance's entry `lane & 15` (0..8) in lanes 0..8 of the group; cbar, wbar: all
+// lanes.  active: the group has a solve (the warp's other group may not).  Lane 0 of the group
+// writes out.  All 32 lanes call it together.
+__device__ __forceinline__ void horn_pose_group(double S_lane, const double cbar[3], const double wbar[3], bool active,
+                                                double* out) {
+  const int l = threadIdx.x & 15, i = l >> 2, j = l & 3;
+  double S[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) S[k] = group_get(S_lane, k);
+  const double Sxx = S[0], Sxy = S[1], Sxz = S[2], Syx = S[3], Syy = S[4], Syz = S[5], Szx = S[6], Szy = S[7],
+               Szz = S[8];
+  double A, V = i == j ? 1.0 : 0.0;
+  {
+    const int u = min(i, j), v = max(i, j);
+    double x = Syz, y = -Szy;                                   // (0, 1)
+    if (u == 0 && v == 2) x = Szx, y = -Sxz;
+    if (u == 0 && v == 3) x = Sxy, y = -Syx;
+    if (u == 1 && v == 2) x = Sxy, y = Syx;
+    if (u == 1 && v == 3) x = Szx, y = Sxz;
+    if (u == 2 && v == 3) x = Syz, y = Szy;
+    if (u == v) {
+      x = u < 2 ? Sxx : -Sxx;
+      y = (u == 0 || u == 2) ? Syy : -Syy;
+    }
+    A = __dadd_rn(x, y);
+    if (u == v) A = __dadd_rn(A, (u == 0 || u == 3) ? Szz : -Szz);
+  }
+  bool busy = active;
+  for (int sweep = 0; sweep < 30; ++sweep) {
+    double off = 0.0, diag = 0.0;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) {
+      const double d = group_get(A, 5 * p);
+      diag = __fma_rn(d, d, diag);
+#pragma unroll
+      for (int q = p + 1; q < 4; ++q) {
+        const double o = group_get(A, 4 * p + q);
+        off = __fma_rn(o, o, off);
+      }
+    }
+    if (off <= 1e-30 * (diag + 1e-300)) busy = false;
+    if (!__any_sync(0xffffffffu, busy)) break;
+#pragma unroll
+    for (int st = 0; st < 3; ++st) {
+      // stage st rotates the pairs (0, st + 1) and the two other indices, in that order
+      const int flip = st + 1;
+      const int jp = j ^ flip, ip = i ^ flip;                   // partners
+      const bool j_first = j < jp, i_first = i < ip;            // first index of its pair
+      const bool j0 = j == 0 || j == flip, i0 = i == 0 || i == flip;  // in pair (0, flip)
+      // angle of the pair holding j: p = min(j, jp), q = max(j, jp)
+      const int p = min(j, jp), q = max(j, jp);
+      const double apq = group_get(A, 4 * p + q), aqq = group_get(A, 5 * q), app = group_get(A, 5 * p);
+      double c = 1.0, s = 0.0;
+      if (fabs(apq) >= 1e-300) {
+        const double theta = __ddiv_rn(__dsub_rn(aqq, app), 2.0 * apq);
+        const double t = __ddiv_rn(theta >= 0.0 ? 1.0 : -1.0, __dadd_rn(fabs(theta), __dsqrt_rn(__fma_rn(theta, theta, 1.0))));
+        c = rsqrt(__fma_rn(t, t, 1.0));
+        s = __dmul_rn(t, c);
+      }
+      const double ci = group_get(c, i), si = group_get(s, i);  // lane i (row 0) holds column i's angle
+      // x' = c x - s y for the pair's first index, y' = s x + c y for its second
+      auto rotate = [](double mine, double other, bool first, double cc, double ss) {
+        const double x = first ? mine : other, y = first ? other : mine;
+        return __fma_rn(first ? cc : ss, x, __dmul_rn(first ? -ss : cc, y));
+      };
+      // horn_pose rotates pair 0's columns, its rows, then pair 1's columns and rows: entries in
+      // pair 0's rows and pair 1's columns see the row rotation first, all others the column's
+      const bool row_first = i0 && !j0;
+      double other = group_get(A, row_first ? 4 * ip + j : 4 * i + jp);
+      double B = rotate(A, other, row_first ? i_first : j_first, row_first ? ci : c, row_first ? si : s);
+      other = group_get(B, row_first ? 4 * i + jp : 4 * ip + j);
+      B = rotate(B, other, row_first ? j_first : i_first, row_first ? c : ci, row_first ? s : si);
+      other = group_get(V, 4 * i + jp);
+      const double U = rotate(V, other, j_first, c, s);
+      if (busy) {
+        A = B;
+        V = U;
+      }
+    }
+  }
+  double best_d = group_get(A, 0);
+  int bk = 0;
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    const double d = group_get(A, 5 * k);
+    if (d > best_d) {
+      best_d = d;
+      bk = k;
+    }
+  }
+  const double w = group_get(V, bk), x = group_get(V, 4 + bk), y = group_get(V, 8 + bk), z = group_get(V, 12 + bk);
+  if (!active || l != 0) return;
+  quaternion_pose(w, x, y, z, cbar, wbar, out);
+}
+
+// ---------------------------------------------------------------------------------------------
 // Valid-pixel table
 // ---------------------------------------------------------------------------------------------
 constexpr int kCompactThreads = 256;
@@ -413,7 +526,35 @@ __global__ void __launch_bounds__(kSearchWarps * 32, RELO_SEARCH_MIN_BLOCKS)
   }
 }
 
-// FP64 Kabsch (Horn) of each hypothesis's kept try; also initialises the round state.
+// (first mode, mode count) of an entry's leaf in tree t: its modes are f.modes[first ..
+// first + count) in units of kModeFloats; count 0 for a leaf id outside the forest.
+__device__ __forceinline__ int2 tree_modes(const RansacJob& job, int idx, const TableEntry& e, int t, int L) {
+  const ForestView& f = job.forest;
+  const int leaf = entry_leaf(job, idx, e, t);
+  if (leaf >= L || !RELO_CHECK(t >= 0 && t < f.T)) return make_int2(0, 0);
+  const int node = t * L + leaf;
+  return make_int2(node * f.M, min((int)__ldg(&f.n_modes[node]), f.M));
+}
+
+// Draws pixel i of round r (a position in the valid table) and writes its record (camera point and
+// where its modes are), which every hypothesis then reads.
+__device__ __forceinline__ void draw_pixel(const RansacJob& job, int r, int i, int n_valid) {
+  const float ifx = (float)(1.0 / job.fx), ify = (float)(1.0 / job.fy), cx = (float)job.cx, cy = (float)job.cy;
+  const int T = job.forest.T, L = 1 << job.forest.D;
+  const uint4 x = philox4x32_10(make_uint4(2u, (uint32_t)r, (uint32_t)i, 0u), job.key0, job.key1);
+  const int idx = (int)uniform_below(x.x, (uint32_t)n_valid);
+  job.drawn[(size_t)r * job.B + i] = idx;
+  const TableEntry e = load_entry(job, idx);
+  const float3 c = cam_point_f(e.u, e.v, e.depth, ifx, ify, cx, cy);
+  int4* rec = job.pix + ((size_t)r * job.B + i) * job.hs;
+  rec[0] = make_int4(__float_as_int(c.x), __float_as_int(c.y), __float_as_int(c.z), 0);
+  for (int t = 0; t < T; t += 2) {
+    const int2 a = tree_modes(job, idx, e, t, L);
+    const int2 b = t + 1 < T ? tree_modes(job, idx, e, t + 1, L) : make_int2(0, 0);
+    rec[1 + t / 2] = make_int4(a.x, a.y, b.x, b.y);
+  }
+}
+
 // FP64 Kabsch of hypothesis h's kept try; also initialises its round state.
 __device__ __forceinline__ void fit_one(const RansacJob& job, int h) {
   double* pose = job.poses + 12 * (size_t)h;
@@ -429,14 +570,15 @@ __device__ __forceinline__ void fit_one(const RansacJob& job, int h) {
       wp[k][1] = m.y;
       wp[k][2] = m.z;
       for (int a = 0; a < 3; ++a) {
-        cb[a] += cp[k][a] / 3.0;
-        wb[a] += wp[k][a] / 3.0;
+        cb[a] = __dadd_rn(cb[a], __ddiv_rn(cp[k][a], 3.0));
+        wb[a] = __dadd_rn(wb[a], __ddiv_rn(wp[k][a], 3.0));
       }
     }
     double S[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
     for (int k = 0; k < 3; ++k)
       for (int a = 0; a < 3; ++a)
-        for (int b = 0; b < 3; ++b) S[3 * a + b] += (cp[k][a] - cb[a]) * (wp[k][b] - wb[b]);
+        for (int b = 0; b < 3; ++b)
+          S[3 * a + b] = __fma_rn(__dsub_rn(cp[k][a], cb[a]), __dsub_rn(wp[k][b], wb[b]), S[3 * a + b]);
     horn_pose(S, cb, wb, pose);
   } else {
     for (int q = 0; q < 12; ++q) pose[q] = (q % 5 == 0) ? 1.0 : 0.0;
@@ -446,23 +588,92 @@ __device__ __forceinline__ void fit_one(const RansacJob& job, int h) {
   job.inliers[h] = 0;
 }
 
-__global__ void __launch_bounds__(128) fit_kernel(const RansacJob* __restrict__ jobs, int n_jobs, int total) {
-  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
-  if (gid >= total) return;
+// fit_one of two hypotheses by a warp (hypothesis h by the group of 16 lanes; h < 0: none).
+__device__ __forceinline__ void fit_group(const RansacJob& job, int h) {
+  const int l = threadIdx.x & 15;
+  const bool ok = h >= 0 && job.hyp_ok[h] != 0;
+  double cb[3] = {0, 0, 0}, wb[3] = {0, 0, 0}, S = 0.0;
+  if (ok) {
+    // every lane takes the three points (the loads are broadcasts); lane 3 a + b sums S(a, b)
+    const Corr c = draw_try(job, h, job.tries[h], *job.n_valid);
+    const int L = 1 << job.forest.D;
+    double cp[3][3], wp[3][3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      cam_point_d(c.e[k].u, c.e[k].v, c.e[k].depth, job.fx, job.fy, job.cx, job.cy, cp[k]);
+      const float4 m = job.forest.top[(size_t)c.tree[k] * L + c.leaf[k]];
+      wp[k][0] = m.x;
+      wp[k][1] = m.y;
+      wp[k][2] = m.z;
+#pragma unroll
+      for (int a = 0; a < 3; ++a) {
+        cb[a] = __dadd_rn(cb[a], __ddiv_rn(cp[k][a], 3.0));
+        wb[a] = __dadd_rn(wb[a], __ddiv_rn(wp[k][a], 3.0));
+      }
+    }
+    const int a = min(l / 3, 2), b = l - 3 * (l / 3);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double ca = a == 0 ? cp[k][0] : a == 1 ? cp[k][1] : cp[k][2], ma = a == 0 ? cb[0] : a == 1 ? cb[1] : cb[2];
+      const double wv = b == 0 ? wp[k][0] : b == 1 ? wp[k][1] : wp[k][2], mb = b == 0 ? wb[0] : b == 1 ? wb[1] : wb[2];
+      S = __fma_rn(__dsub_rn(ca, ma), __dsub_rn(wv, mb), S);
+    }
+  }
+  __syncwarp();
+  horn_pose_group(S, cb, wb, ok, h >= 0 ? job.poses + 12 * (size_t)h : nullptr);
+  if (h < 0) return;
+  if (!ok && l < 12) job.poses[12 * (size_t)h + l] = (l % 5 == 0) ? 1.0 : 0.0;
+  if (l == 0) {
+    job.energy[h] = ok ? 0.0 : (double)INFINITY;
+    job.alive_a[h] = h;
+    job.inliers[h] = 0;
+  }
+}
+
+__device__ __forceinline__ int hypothesis_job(const RansacJob* __restrict__ jobs, int n_jobs, int gid) {
   int lo = 0, hi = n_jobs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
     if (jobs[mid].hyp_begin <= gid) lo = mid;
     else hi = mid - 1;
   }
-  const RansacJob& job = jobs[lo];
+  return lo;
+}
+
+// The kept tries' poses, and the draws of every round (both need only the table and the search's
+// result, and a round's draws are the same whoever is alive): CTAs below fit_blocks take the fits,
+// draw_blocks CTAs per job after them the job's drawn pixels.  kGroup: two hypotheses per warp
+// (fit_group) instead of 32.
+constexpr int kFitThreads = 128;
+template <bool kGroup>
+__global__ void __launch_bounds__(kFitThreads) fit_kernel(const RansacJob* __restrict__ jobs, int n_jobs, int total,
+                                                          int fit_blocks, int draw_blocks) {
+  if ((int)blockIdx.x >= fit_blocks) {
+    const int q = (int)blockIdx.x - fit_blocks, jid = q / draw_blocks;
+    const RansacJob& job = jobs[jid];
+    if (job_skipped(job.skip)) return;
+    const int i = (q - jid * draw_blocks) * kFitThreads + threadIdx.x;
+    if (i < job.n_rounds * job.B && *job.n_valid > 0) draw_pixel(job, i / job.B, i % job.B, *job.n_valid);
+    return;
+  }
+  if (kGroup) {
+    const int gid = ((int)blockIdx.x * kFitThreads + (int)threadIdx.x) >> 4;
+    // the groups of a warp may serve different jobs; an idle group takes part with h = -1
+    const RansacJob& job = jobs[hypothesis_job(jobs, n_jobs, min(gid, total - 1))];
+    const int h = gid - job.hyp_begin;
+    fit_group(job, gid < total && h < job.K && !job_skipped(job.skip) ? h : -1);
+    return;
+  }
+  const int gid = blockIdx.x * blockDim.x + threadIdx.x;
+  if (gid >= total) return;
+  const RansacJob& job = jobs[hypothesis_job(jobs, n_jobs, gid)];
   const int h = gid - job.hyp_begin;
   if (h >= job.K || job_skipped(job.skip)) return;
   fit_one(job, h);
 }
 
 cudaError_t launch_hypotheses(const RansacJob* jobs, int n_jobs, int total_hyps, int32_t* counter, cudaStream_t s,
-                              const Schedule& sched) {
+                              const Schedule& sched, int max_draws) {
   if (total_hyps <= 0) return cudaSuccess;
   static PerDevice resident;  // resident search CTAs per SM on each device
   int sms = 0, per_sm = 0;
@@ -480,7 +691,12 @@ cudaError_t launch_hypotheses(const RansacJob* jobs, int n_jobs, int total_hyps,
   if (e != cudaSuccess) return e;
   const int grid = std::min(sms * ctas, (total_hyps + kSearchWarps - 1) / kSearchWarps);
   search_kernel<<<grid, kSearchWarps * 32, 0, s>>>(jobs, n_jobs, total_hyps, counter);
-  fit_kernel<<<(total_hyps + 127) / 128, 128, 0, s>>>(jobs, n_jobs, total_hyps);
+  const bool group = total_hyps <= kGroupSolves;
+  const int per_block = group ? kSolvesPerWarp * kFitThreads / 32 : kFitThreads;
+  const int fit_blocks = (total_hyps + per_block - 1) / per_block, draw_blocks = (max_draws + kFitThreads - 1) / kFitThreads;
+  const unsigned fit_grid = (unsigned)fit_blocks + (unsigned)draw_blocks * (unsigned)n_jobs;
+  if (group) fit_kernel<true><<<fit_grid, kFitThreads, 0, s>>>(jobs, n_jobs, total_hyps, fit_blocks, draw_blocks);
+  else fit_kernel<false><<<fit_grid, kFitThreads, 0, s>>>(jobs, n_jobs, total_hyps, fit_blocks, draw_blocks);
   return cudaGetLastError();
 }
 
@@ -490,18 +706,7 @@ cudaError_t launch_hypotheses(const RansacJob* jobs, int n_jobs, int total_hyps,
 __device__ __forceinline__ const int32_t* alive_in(const RansacJob& j, int r) { return (r & 1) ? j.alive_b : j.alive_a; }
 __device__ __forceinline__ int32_t* alive_out(const RansacJob& j, int r) { return (r & 1) ? j.alive_a : j.alive_b; }
 
-// (first mode, mode count) of an entry's leaf in tree t: its modes are f.modes[first ..
-// first + count) in units of kModeFloats; count 0 for a leaf id outside the forest.
-__device__ __forceinline__ int2 tree_modes(const RansacJob& job, int idx, const TableEntry& e, int t, int L) {
-  const ForestView& f = job.forest;
-  const int leaf = entry_leaf(job, idx, e, t);
-  if (leaf >= L || !RELO_CHECK(t >= 0 && t < f.T)) return make_int2(0, 0);
-  const int node = t * L + leaf;
-  return make_int2(node * f.M, min((int)__ldg(&f.n_modes[node]), f.M));
-}
-
-// Draw round r's B pixels (positions in the valid table), one CTA per job, and write each drawn
-// pixel's record (camera point and where its modes are), which every hypothesis then reads.
+// Draw round r's B pixels, one CTA per job.
 __device__ __forceinline__ void draw_block(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ alive_prefix,
                                            int r, int jid) {
   if (alive_prefix[jid + 1] - alive_prefix[jid] == 0) return;
@@ -509,22 +714,7 @@ __device__ __forceinline__ void draw_block(const RansacJob* __restrict__ jobs, c
   if (job_skipped(job.skip)) return;
   const int n_valid = *job.n_valid;
   if (n_valid == 0) return;
-  const float ifx = (float)(1.0 / job.fx), ify = (float)(1.0 / job.fy), cx = (float)job.cx, cy = (float)job.cy;
-  const int T = job.forest.T, L = 1 << job.forest.D;
-  for (int i = threadIdx.x; i < job.B; i += blockDim.x) {
-    const uint4 x = philox4x32_10(make_uint4(2u, (uint32_t)r, (uint32_t)i, 0u), job.key0, job.key1);
-    const int idx = (int)uniform_below(x.x, (uint32_t)n_valid);
-    job.drawn[(size_t)r * job.B + i] = idx;
-    const TableEntry e = load_entry(job, idx);
-    const float3 c = cam_point_f(e.u, e.v, e.depth, ifx, ify, cx, cy);
-    int4* rec = job.pix + ((size_t)r * job.B + i) * job.hs;
-    rec[0] = make_int4(__float_as_int(c.x), __float_as_int(c.y), __float_as_int(c.z), 0);
-    for (int t = 0; t < T; t += 2) {
-      const int2 a = tree_modes(job, idx, e, t, L);
-      const int2 b = t + 1 < T ? tree_modes(job, idx, e, t + 1, L) : make_int2(0, 0);
-      rec[1 + t / 2] = make_int4(a.x, a.y, b.x, b.y);
-    }
-  }
+  for (int i = threadIdx.x; i < job.B; i += blockDim.x) draw_pixel(job, r, i, n_valid);
 }
 
 __global__ void draw_kernel(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ alive_prefix, int r) {
@@ -532,34 +722,49 @@ __global__ void draw_kernel(const RansacJob* __restrict__ jobs, const int32_t* _
 }
 
 // A pixel's modes, staged by its warp in shared memory: the warp copies every mode of the pixel's
-// leaves (trees in order, modes in order) with parallel loads, then every lane scores them from
-// there, instead of each mode being a dependent global load in turn.
-constexpr int kStageModes = 64;  // modes per warp slot; a pixel with more is scored from global memory
+// leaves (trees in order, modes in order), then every lane scores them from there, instead of each
+// mode being a dependent global load in turn.  A pixel's staging is two dependent L2 round trips
+// (its record's mode ranges, then the modes), which is what bound the round kernels: the copies are
+// asynchronous into two slots per warp, so that the next pixel's modes arrive while this one is
+// scored, and the ranges are read a pixel earlier still.
+constexpr int kStageModes = 60;  // modes per warp slot (two slots of 8 warps fit 48 KB); a pixel with
+                                 // more is scored from global memory
 
 struct ModeSlot {
   float4 m[kStageModes * 3];
 };
+struct ModeSlots {
+  ModeSlot s[2];
+};
 
-// Copies the modes of record rec into slot (all lanes of the warp take part); returns their
-// number, or -1 if they do not fit (then nothing is staged).
-__device__ __forceinline__ int stage_modes(const RansacJob& job, const int4* __restrict__ rec, ModeSlot& slot,
-                                           int lane) {
+__device__ __forceinline__ void copy_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void copy_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+
+// (first mode, mode count) of a pixel record's leaf in tree `lane` (lanes below T; 0 elsewhere).
+__device__ __forceinline__ int2 mode_range(const int4* __restrict__ rec, int T, int lane) {
+  return lane < T ? __ldg(reinterpret_cast<const int2*>(rec + 1) + lane) : make_int2(0, 0);
+}
+
+// Starts the copies of the modes of a pixel with ranges `range` into slot (all lanes of the warp
+// take part); returns their number, or -1 if they do not fit (then nothing is staged).
+__device__ __forceinline__ int stage_modes(const RansacJob& job, int2 range, ModeSlot& slot, int lane) {
   const ForestView& f = job.forest;
-  int total = 0;
-  for (int t = 0; t < f.T; ++t) {
-    const int4 w = __ldg(&rec[1 + t / 2]);
-    total += (t & 1) ? w.w : w.y;
-  }
+  const int total = warp_sum_i(range.y);
   if (total > kStageModes) return -1;
   int off = 0;
   for (int t = 0; t < f.T; ++t) {
-    const int4 w = __ldg(&rec[1 + t / 2]);
-    const int first = (t & 1) ? w.z : w.x, nm = (t & 1) ? w.w : w.y;
+    const int first = __shfl_sync(0xffffffffu, range.x, t), nm = __shfl_sync(0xffffffffu, range.y, t);
     const float4* src = reinterpret_cast<const float4*>(f.modes + (size_t)first * kModeFloats);
-    for (int i = lane; i < 3 * nm; i += 32) slot.m[3 * off + i] = __ldg(&src[i]);
+    for (int i = lane; i < 3 * nm; i += 32) copy_async16(&slot.m[3 * off + i], src + i);
     off += nm;
   }
-  __syncwarp();
   return total;
 }
 
@@ -573,23 +778,10 @@ __device__ __forceinline__ float mode_score(float4 a, float4 b, float4 c, float3
 }
 
 // Best mode of a drawn pixel (its record) under x = P c, over trees then modes in order (the first
-// of equal scores wins): its score (-inf if none) and mean.  n_staged >= 0: the modes are in slot
-// (same order); otherwise they are read from global memory (every lane reads the same mode, so
-// each load is one broadcast).
-__device__ __forceinline__ float record_best(const RansacJob& job, const int4* __restrict__ rec, const ModeSlot& slot,
-                                             int n_staged, float3 x, float3* mu_best) {
+// of equal scores wins), read from global memory: its score (-inf if none) and mean.
+__device__ __forceinline__ float record_best_global(const RansacJob& job, const int4* __restrict__ rec, float3 x,
+                                                    float3* mu_best) {
   float best = -INFINITY;
-  if (n_staged >= 0) {
-    for (int k = 0; k < n_staged; ++k) {
-      const float4 a = slot.m[3 * k], b = slot.m[3 * k + 1], c = slot.m[3 * k + 2];
-      const float sc = mode_score(a, b, c, x);
-      if (sc > best) {
-        best = sc;
-        if (mu_best) *mu_best = make_float3(a.x, a.y, a.z);
-      }
-    }
-    return best;
-  }
   const ForestView& f = job.forest;
   for (int t = 0; t < f.T; ++t) {
     const int4 w = __ldg(&rec[1 + t / 2]);
@@ -612,23 +804,23 @@ __device__ __forceinline__ float3 record_point(const int4* __restrict__ rec) {
   return make_float3(__int_as_float(w.x), __int_as_float(w.y), __int_as_float(w.z));
 }
 
-// record_best over staged modes with the whole warp on one point x (every lane passes the same x):
-// lane l scores modes l, l + 32, ..., then the warp keeps the largest score and, among equal ones,
-// the lowest index -- the mode that the scan in order with a strict comparison keeps (a NaN score
-// never wins in either).  Returns the score (-inf if none) and, in every lane, the mode's mean.
-__device__ __forceinline__ float warp_best_staged(const ModeSlot& slot, int n_staged, float3 x, int lane,
-                                                  float3* mu_best) {
+// record_best over staged modes by a group of 1 << g lanes (aligned; every lane of it passes the
+// same x): lane `sub` of the group scores modes sub, sub + (1 << g), ..., then the group keeps the
+// largest score and, among equal ones, the lowest index -- the mode that the scan in order with a
+// strict comparison keeps (a NaN score never wins in either).  Returns the score (-inf if none) and,
+// in every lane of the group, the mode's mean.
+__device__ __forceinline__ float group_best_staged(const ModeSlot& slot, int n_staged, float3 x, int sub, int g,
+                                                   float3* mu_best) {
   float best = -INFINITY;
   int bi = -1;
-  for (int k = lane; k < n_staged; k += 32) {
+  for (int k = sub; k < n_staged; k += 1 << g) {
     const float sc = mode_score(slot.m[3 * k], slot.m[3 * k + 1], slot.m[3 * k + 2], x);
     if (sc > best) {
       best = sc;
       bi = k;
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
+  for (int o = 1 << g >> 1; o > 0; o >>= 1) {
     const float ob = __shfl_xor_sync(0xffffffffu, best, o);
     const int oi = __shfl_xor_sync(0xffffffffu, bi, o);
     if (ob > best || (ob == best && oi >= 0 && (bi < 0 || oi < bi))) {
@@ -636,75 +828,120 @@ __device__ __forceinline__ float warp_best_staged(const ModeSlot& slot, int n_st
       bi = oi;
     }
   }
-  if (bi >= 0) {
+  if (mu_best && bi >= 0) {
     const float4 a = slot.m[3 * bi];
     *mu_best = make_float3(a.x, a.y, a.z);
   }
   return best;
 }
 
-// Chunks with at most this many hypotheses score each staged pixel with the whole warp per
-// hypothesis (warp_best_staged) instead of one lane per hypothesis scanning every mode: the last
-// rounds, where a job keeps one or two survivors and the lanes of a chunk would mostly idle.
-// Measured on the house batch: faster for 1 and 2 hypotheses (re-fit sums 457 -> 309 us in the
-// last round), slower from 4 (the warp pass's shuffle reductions are a dependent chain, while the
-// per-lane scan overlaps its independent mode scores).  Both give the same scores and modes.
-#ifndef RELO_FEW_HYPS
-#define RELO_FEW_HYPS 2
-#endif
-constexpr int kFewHyps = RELO_FEW_HYPS;
+// Lanes per hypothesis of a chunk with n of them, as a power of two: a chunk of 32 gives each lane
+// one hypothesis; the last rounds, where a job keeps few survivors, share a hypothesis's modes among
+// the lanes that would otherwise idle.
+__host__ __device__ __forceinline__ int group_log2(int n) { return n > 16 ? 0 : n > 8 ? 1 : n > 4 ? 2 : n > 2 ? 3 : n > 1 ? 4 : 5; }
 
-// Round kernels: a CTA takes 32 hypotheses of one job (one per lane) and its warps split the
-// pixels, each warp walking every kRoundWarps-th pixel; per-warp partial sums are combined in
-// warp order, so the result does not depend on scheduling.
+// Round kernels: a CTA takes up to 32 hypotheses of one job and its warps split the pixels, each
+// warp walking every kRoundWarps-th pixel; per-warp partial sums are combined in warp order, so the
+// result does not depend on scheduling.
 constexpr int kRoundWarps = 8;
 
-// Energies of round r for hypotheses chunk * 32 .. + 31 of job jid.
+// Calls score(i, point, slot, n_staged) for pixels i = first, first + step, ... below end in turn,
+// with the pixel's modes staged (n_staged as stage_modes) and the next one's on their way.  rec0:
+// record of pixel 0, hs: its int4 words.
+template <class F>
+__device__ __forceinline__ void for_staged_pixels(const RansacJob& job, const int4* __restrict__ rec0, int hs, int first,
+                                                  int end, int step, ModeSlots& slots, int lane, F&& score) {
+  const int T = job.forest.T;
+  if (first >= end) return;
+  const int4* rec = rec0 + (size_t)first * hs;
+  int4 point = __ldg(rec);
+  int n_staged = stage_modes(job, mode_range(rec, T, lane), slots.s[0], lane);
+  copy_commit();
+  int2 range = make_int2(0, 0);
+  int4 next_point = point;
+  if (first + step < end) {
+    rec = rec0 + (size_t)(first + step) * hs;
+    next_point = __ldg(rec);
+    range = mode_range(rec, T, lane);
+  }
+  int which = 0;
+  for (int i = first; i < end; i += step, which ^= 1) {
+    int next_staged = 0;
+    const int4 c = point;
+    __syncwarp();  // the other slot's pixel is scored
+    if (i + step < end) next_staged = stage_modes(job, range, slots.s[which ^ 1], lane);
+    copy_commit();
+    point = next_point;
+    if (i + 2 * step < end) {
+      rec = rec0 + (size_t)(i + 2 * step) * hs;
+      next_point = __ldg(rec);
+      range = mode_range(rec, T, lane);
+    }
+    copy_wait<1>();
+    __syncwarp();  // every lane's copies of pixel i have landed
+    score(i, make_float3(__int_as_float(c.x), __int_as_float(c.y), __int_as_float(c.z)), slots.s[which], n_staged);
+    n_staged = next_staged;
+  }
+  copy_wait<0>();
+}
+
+// Whether a split launch's energies of the job go through its score buffer: the per-pixel scores
+// take the re-fit sums' buffer, whose 128 ceil(R B / 64) bytes per hypothesis hold 4 B for R >= 2
+// rounds (a job of two hypotheses has one).
+__device__ __forceinline__ bool split_scores(const RansacJob& job, int n_split) { return n_split > 1 && job.K > 2; }
+
+// Energies of round r for hypotheses chunk * 32 .. + 31 of job jid.  n_split > 1: only the pixels of
+// part `split`, whose scores go to the job's score buffer [pixel][alive hypothesis] instead, for
+// sum_scores to add in the same order.
 __device__ __forceinline__ void energy_block(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ alive_prefix,
-                                             int r, int chunk, int jid, ModeSlot* slots, float (*part)[32]) {
+                                             int r, int chunk, int jid, int split, int n_split, ModeSlots* slots,
+                                             float (*part)[32]) {
   const int n_alive = alive_prefix[jid + 1] - alive_prefix[jid];
   if (chunk * 32 >= n_alive) return;
   const RansacJob& job = jobs[jid];
   if (job_skipped(job.skip) || *job.n_valid == 0) return;
+  const bool to_scores = split_scores(job, n_split);
+  if (!to_scores && split > 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int a = chunk * 32 + lane;
+  const int n_here = min(32, n_alive - chunk * 32);
+  const int g = group_log2(n_here), sub = lane & ((1 << g) - 1);
+  const int a = chunk * 32 + (lane >> g);
   const int h = a < n_alive ? alive_in(job, r)[a] : 0;
-  const bool valid = a < n_alive && job.hyp_ok[h];
   const PoseF P = pose_to_float(job.poses + 12 * (size_t)h);
   float sum = 0.f;
-  const int4* recs = job.pix + (size_t)r * job.B * job.hs;
-  const int n_here = min(32, n_alive - chunk * 32);
-  for (int i = warp; i < job.B; i += kRoundWarps) {
-    const int4* rec = recs + (size_t)i * job.hs;
-    __syncwarp();  // the slot's previous pixel is scored
-    const int n_staged = stage_modes(job, rec, slots[warp], lane);
-    const float3 x = apply(P, record_point(rec));
-    if (n_here <= kFewHyps && n_staged >= 0) {
-      for (int j = 0; j < n_here; ++j) {
-        const float3 xj = make_float3(__shfl_sync(0xffffffffu, x.x, j), __shfl_sync(0xffffffffu, x.y, j),
-                                      __shfl_sync(0xffffffffu, x.z, j));
-        float3 mu;
-        const float best = warp_best_staged(slots[warp], n_staged, xj, lane, &mu);
-        if (lane == j) sum += fminf(kLogEps, -best);
-      }
-    } else {
-      const float best = record_best(job, rec, slots[warp], n_staged, x, nullptr);
-      sum += fminf(kLogEps, -best);
-    }
-  }
-  part[warp][lane] = sum;
+  const int rows = (job.B + kRoundWarps - 1) / kRoundWarps, per = (rows + n_split - 1) / n_split;
+  const int row0 = to_scores ? split * per : 0, row1 = to_scores ? min(rows, row0 + per) : rows;
+  float* scores = reinterpret_cast<float*>(job.refit);
+  for_staged_pixels(job, job.pix + (size_t)r * job.B * job.hs, job.hs, row0 * kRoundWarps + warp,
+                    min(row1 * kRoundWarps, job.B), kRoundWarps, slots[warp], lane,
+                    [&](int i, float3 c, const ModeSlot& slot, int n_staged) {
+                      const float3 x = apply(P, c);
+                      const float best =
+                          n_staged >= 0 ? group_best_staged(slot, n_staged, x, sub, g, nullptr)
+                                        : record_best_global(job, job.pix + ((size_t)r * job.B + i) * job.hs, x, nullptr);
+                      const float e = fminf(kLogEps, -best);
+                      if (to_scores) {
+                        if (sub == 0 && a < n_alive) scores[(size_t)i * n_alive + a] = e;
+                      } else {
+                        sum += e;
+                      }
+                    });
+  if (to_scores) return;
+  if (sub == 0) part[warp][lane >> g] = sum;
   __syncthreads();
-  if (warp == 0 && valid) {
-    float e = 0.f;
+  if (warp == 0 && chunk * 32 + lane < n_alive) {
+    const int hl = alive_in(job, r)[chunk * 32 + lane];
+    if (job.hyp_ok[hl]) {
+      float e = 0.f;
 #pragma unroll
-    for (int w = 0; w < kRoundWarps; ++w) e += part[w][lane];
-    job.energy[h] += (double)e;
+      for (int w = 0; w < kRoundWarps; ++w) e += part[w][lane];
+      job.energy[hl] += (double)e;
+    }
   }
 }
 
-// Energies of round r: grid (hypothesis chunks, jobs).
-// CTAs per SM the compiler must fit for the energies, when set (otherwise the compiler's choice:
-// 64 registers, four CTAs per SM)
+// Energies of round r: grid (hypothesis chunks, jobs, pixel splits).
+// CTAs per SM the compiler must fit for the energies, when set (otherwise the compiler's choice)
 #ifdef RELO_ENERGY_MIN_BLOCKS
 #define RELO_ENERGY_BOUNDS __launch_bounds__(kRoundWarps * 32, RELO_ENERGY_MIN_BLOCKS)
 #else
@@ -712,10 +949,35 @@ __device__ __forceinline__ void energy_block(const RansacJob* __restrict__ jobs,
 #endif
 __global__ void RELO_ENERGY_BOUNDS energy_kernel(const RansacJob* __restrict__ jobs,
                                                                   const int32_t* __restrict__ alive_prefix, int r) {
-  __shared__ ModeSlot slots[kRoundWarps];
+  __shared__ ModeSlots slots[kRoundWarps];
   __shared__ float part[kRoundWarps][32];
-  energy_block(jobs, alive_prefix, r, blockIdx.x, blockIdx.y, slots, part);
+  energy_block(jobs, alive_prefix, r, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, slots, part);
 }
+
+// The energies of a split round from its per-pixel scores: eight lanes per hypothesis take the sums
+// that energy_block's eight warps take (every eighth pixel in turn), added in warp order.
+__global__ void __launch_bounds__(256) sum_scores_kernel(const RansacJob* __restrict__ jobs,
+                                                         const int32_t* __restrict__ alive_prefix, int r, int n_split) {
+  static_assert(kRoundWarps == 8, "eight lanes stand for the warps");
+  const int jid = blockIdx.y, n_alive = alive_prefix[jid + 1] - alive_prefix[jid];
+  const int a = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3), w = threadIdx.x & 7, lane = threadIdx.x & 31;
+  const RansacJob& job = jobs[jid];
+  if (n_alive == 0 || !split_scores(job, n_split) || job_skipped(job.skip) || *job.n_valid == 0) return;
+  const float* scores = reinterpret_cast<const float*>(job.refit);
+  float sum = 0.f;
+  if (a < n_alive) {
+#pragma unroll 8
+    for (int i = w; i < job.B; i += kRoundWarps) sum += scores[(size_t)i * n_alive + a];
+  }
+  float e = 0.f;
+#pragma unroll
+  for (int q = 0; q < kRoundWarps; ++q) e += __shfl_sync(0xffffffffu, sum, (lane & 24) + q);
+  if (w == 0 && a < n_alive) {
+    const int h = alive_in(job, r)[a];
+    if (job.hyp_ok[h]) job.energy[h] += (double)e;
+  }
+}
+
 __device__ __forceinline__ unsigned long long order_key(double e) {
   unsigned long long b = (unsigned long long)__double_as_longlong(e);
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
@@ -794,19 +1056,29 @@ __device__ __forceinline__ float dist2_rn(float3 a, float3 b) {
   return __fmaf_rn(dx, dx, __fmaf_rn(dy, dy, __fmul_rn(dz, dz)));
 }
 
+// Shared memory of the re-fit sums: the warps' mode slots, then (the pixels all scored) their sums.
+union RefineShared {
+  ModeSlots slots[kRoundWarps];
+  float red[kRoundWarps][16][32];
+};
+
+// LG: a hypothesis's modes and its sixteen sums are shared among 1 << LG lanes (lane `sub` carries
+// sums sub, sub + (1 << LG), ...), so a CTA takes 32 >> LG survivors.  Every sum sees the same
+// additions in the same order whatever LG is.
+template <int LG>
 __device__ __forceinline__ void refine_block(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ surv_prefix,
-                                             int r, int chunk, int part, int jid, ModeSlot* slots,
-                                             float (*red)[16][32]) {
+                                             int r, int chunk, int part, int jid, RefineShared& sh) {
+  constexpr int kHere = 32 >> LG, kGroup = 1 << LG, kSums = LG < 4 ? 16 >> LG : 1;
   const int n_surv = surv_prefix[jid + 1] - surv_prefix[jid];
-  if (chunk * 32 >= n_surv) return;
+  if (chunk * kHere >= n_surv) return;
   const RansacJob& job = jobs[jid];
   const int n_drawn = (r + 1) * job.B;
   const int p0 = part * kRefinePixels;
   if (p0 >= n_drawn || job_skipped(job.skip) || *job.n_valid == 0) return;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int a = chunk * 32 + lane;
+  const int sub = lane & (kGroup - 1), slot_h = lane >> LG;
+  const int a = chunk * kHere + slot_h;
   const int h = a < n_surv ? alive_out(job, r)[a] : 0;
-  const bool valid = a < n_surv && job.hyp_ok[h];
   const PoseF P = pose_to_float(job.poses + 12 * (size_t)h);
   const float r2 = (float)(job.inlier_dist * job.inlier_dist);
   const float3 cref = record_point(job.pix);
@@ -816,82 +1088,63 @@ __device__ __forceinline__ void refine_block(const RansacJob* __restrict__ jobs,
   // variant of Kahan summation), so the sums hold about twice FP32's precision.  The sums are taken
   // relative to the first drawn pixel; with plain FP32 sums their cancellation against the small
   // spread of a few inliers moved ill-conditioned re-fits by ~1e-4 rad.
-  float acc[16], lo[16];
+  float acc[kSums], lo[kSums];
 #pragma unroll
-  for (int q = 0; q < 16; ++q) acc[q] = lo[q] = 0.f;
-  // adds pixel c (its point x under this lane's hypothesis, best mode mean mu) when it is an inlier
-  auto add_inlier = [&](float3 c, float3 x, float3 mu) {
-    if (dist2_rn(x, mu) < r2) {
-      const float u[3] = {c.x - cref.x, c.y - cref.y, c.z - cref.z};
-      const float w[3] = {mu.x - wref.x, mu.y - wref.y, mu.z - wref.z};
-      acc[0] += 1.f;
+  for (int q = 0; q < kSums; ++q) acc[q] = lo[q] = 0.f;
+  for_staged_pixels(
+      job, job.pix, job.hs, p0 + warp, min(p0 + kRefinePixels, n_drawn), kRoundWarps, sh.slots[warp], lane,
+      [&](int i, float3 c, const ModeSlot& slot, int n_staged) {
+        const float3 x = apply(P, c);
+        float3 mu = make_float3(0.f, 0.f, 0.f);
+        const float best = n_staged >= 0 ? group_best_staged(slot, n_staged, x, sub, LG, &mu)
+                                         : record_best_global(job, job.pix + (size_t)i * job.hs, x, &mu);
+        if (best == -INFINITY || !(dist2_rn(x, mu) < r2)) return;
+        const float u[3] = {c.x - cref.x, c.y - cref.y, c.z - cref.z};
+        const float w[3] = {mu.x - wref.x, mu.y - wref.y, mu.z - wref.z};
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        comp_add(acc[1 + k], lo[1 + k], u[k]);
-        comp_add(acc[4 + k], lo[4 + k], w[k]);
-      }
-#pragma unroll
-      for (int p = 0; p < 3; ++p)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-          const float pr = __fmul_rn(u[p], w[q]);
-          comp_add(acc[7 + 3 * p + q], lo[7 + 3 * p + q], pr);
-          lo[7 + 3 * p + q] = __fadd_rn(lo[7 + 3 * p + q], __fmaf_rn(u[p], w[q], -pr));
+        for (int k = 0; k < kSums; ++k) {
+          const int q = LG == 0 ? k : sub + k * kGroup;  // 0: count, 1..3: u, 4..6: w, 7..15: u w^T
+          if (LG > 4 && q > 15) continue;
+          float first = 1.f, second = 1.f;
+          if (q >= 7) {
+            const int p = (q - 7) / 3, m = (q - 7) - 3 * p;
+            first = p == 0 ? u[0] : p == 1 ? u[1] : u[2];
+            second = m == 0 ? w[0] : m == 1 ? w[1] : w[2];
+          } else if (q > 0) {
+            first = q == 1 ? u[0] : q == 2 ? u[1] : q == 3 ? u[2] : q == 4 ? w[0] : q == 5 ? w[1] : w[2];
+          }
+          // (a product with 1 is exact and its error is 0)
+          const float pr = __fmul_rn(first, second);
+          comp_add(acc[k], lo[k], pr);
+          if (LG > 0 || q >= 7) lo[k] = __fadd_rn(lo[k], __fmaf_rn(first, second, -pr));
         }
-    }
-  };
-  const int n_here = min(32, n_surv - chunk * 32);
-  const int p1 = min(p0 + kRefinePixels, n_drawn);
-  for (int i = p0 + warp; i < p1; i += kRoundWarps) {
-    const int4* rec = job.pix + (size_t)i * job.hs;
-    const float3 c = record_point(rec);
-    const float3 x = apply(P, c);
-    float3 mu;
-    __syncwarp();  // the slot's previous pixel is scored
-    const int n_staged = stage_modes(job, rec, slots[warp], lane);
-    if (n_here <= kFewHyps && n_staged >= 0) {
-      for (int j = 0; j < n_here; ++j) {
-        const float3 xj = make_float3(__shfl_sync(0xffffffffu, x.x, j), __shfl_sync(0xffffffffu, x.y, j),
-                                      __shfl_sync(0xffffffffu, x.z, j));
-        const float best = warp_best_staged(slots[warp], n_staged, xj, lane, &mu);
-        if (lane == j && best != -INFINITY) add_inlier(c, x, mu);
-      }
-    } else {
-      const float best = record_best(job, rec, slots[warp], n_staged, x, &mu);
-      if (best != -INFINITY) add_inlier(c, x, mu);
-    }
-  }
+      });
   // warps w then write sums q = w, w + kRoundWarps: the kRoundWarps partials added in warp order,
   // compensated as above (first their high parts, then their low parts: one shared buffer, two
   // passes), kept as a (high, low) pair that the re-fit adds in FP64
   constexpr int kPer = (16 + kRoundWarps - 1) / kRoundWarps;
-  float sh[kPer], sl[kPer];
+  float s_hi[kPer], s_lo[kPer];
 #pragma unroll
-  for (int i = 0; i < kPer; ++i) sh[i] = sl[i] = 0.f;
+  for (int i = 0; i < kPer; ++i) s_hi[i] = s_lo[i] = 0.f;
 #pragma unroll
   for (int pass = 0; pass < 2; ++pass) {
+    __syncthreads();  // the slots, then the first pass's partials, are read
 #pragma unroll
-    for (int q = 0; q < 16; ++q) red[warp][q][lane] = pass ? lo[q] : acc[q];
+    for (int k = 0; k < kSums; ++k)
+      if (LG <= 4 || sub + k * kGroup < 16) sh.red[warp][sub + k * kGroup][slot_h] = pass ? lo[k] : acc[k];
     __syncthreads();
 #pragma unroll
     for (int i = 0; i < kPer; ++i) {
       const int q = warp + i * kRoundWarps;
-      if (q < 16)
+      if (q < 16 && lane < kHere)
 #pragma unroll
         for (int w = 0; w < kRoundWarps; ++w) {
-          if (pass == 0) comp_add(sh[i], sl[i], red[w][q][lane]);
-          else sl[i] = __fadd_rn(sl[i], red[w][q][lane]);
+          if (pass == 0) comp_add(s_hi[i], s_lo[i], sh.red[w][q][lane]);
+          else s_lo[i] = __fadd_rn(s_lo[i], sh.red[w][q][lane]);
         }
     }
-    __syncthreads();
   }
-  if (!valid) return;
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) {
-    const int q = warp + i * kRoundWarps;
-    if (q < 16) job.refit[((size_t)h * job.refit_parts + part) * 16 + q] = make_float2(sh[i], sl[i]);
-  }
-  if (part == 0 && warp == 0) {
+  if (part == 0 && warp == 0 && sub == 0 && a < n_surv && job.hyp_ok[h]) {
     float* ref = job.refit_ref + (size_t)h * 8;
     ref[0] = cref.x;
     ref[1] = cref.y;
@@ -900,136 +1153,29 @@ __device__ __forceinline__ void refine_block(const RansacJob* __restrict__ jobs,
     ref[4] = wref.y;
     ref[5] = wref.z;
   }
-}
-
-// CTAs per SM the compiler must fit for the re-fit sums (the 16 compensated sums per lane take
-// registers; the fewer a thread holds, the more pixels' loads are in flight per SM)
-#ifndef RELO_REFINE_MIN_BLOCKS
-#define RELO_REFINE_MIN_BLOCKS 2
-#endif
-__global__ void __launch_bounds__(kRoundWarps * 32, RELO_REFINE_MIN_BLOCKS) refine_kernel(const RansacJob* __restrict__ jobs,
-                                                                  const int32_t* __restrict__ surv_prefix, int r) {
-  __shared__ ModeSlot slots[kRoundWarps];
-  __shared__ float red[kRoundWarps][16][32];
-  refine_block(jobs, surv_prefix, r, blockIdx.x, blockIdx.y, blockIdx.z, slots, red);
-}
-
-// Re-fit sums of rounds whose chunks hold at most kFewHyps hypotheses (the last rounds): the same
-// sums as refine_block's, taken with the sixteen sums of hypothesis j spread over lanes 16 j ..
-// 16 j + 15 (lane 16 j + q carries sum q) instead of all sixteen in lane j, so a thread holds one
-// compensated pair instead of sixteen and more CTAs fit an SM.  Every sum sees the same additions
-// in the same order as in refine_block (the pixels of a warp in turn, then the warps in order), so
-// the results are identical.
-__device__ __forceinline__ void refine_few_block(const RansacJob* __restrict__ jobs,
-                                                 const int32_t* __restrict__ surv_prefix, int r, int part, int jid,
-                                                 ModeSlot* slots, float (*red)[16][32]) {
-  const int n_surv = surv_prefix[jid + 1] - surv_prefix[jid];
-  if (n_surv == 0) return;
-  const RansacJob& job = jobs[jid];
-  const int n_drawn = (r + 1) * job.B;
-  const int p0 = part * kRefinePixels;
-  if (p0 >= n_drawn || job_skipped(job.skip) || *job.n_valid == 0) return;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = lane >> 4, q = lane & 15;  // this lane's hypothesis and sum
-  const int n_here = min(kFewHyps, n_surv);
-  const int h = j < n_here ? alive_out(job, r)[j] : 0;
-  const PoseF P = pose_to_float(job.poses + 12 * (size_t)h);
-  const float r2 = (float)(job.inlier_dist * job.inlier_dist);
-  const float3 cref = record_point(job.pix);
-  const float3 wref = apply(P, cref);
-  float acc = 0.f, lo = 0.f;
-  const int p1 = min(p0 + kRefinePixels, n_drawn);
-  for (int i = p0 + warp; i < p1; i += kRoundWarps) {
-    const int4* rec = job.pix + (size_t)i * job.hs;
-    const float3 c = record_point(rec);
-    const float3 x = apply(P, c);  // this lane's hypothesis
-    __syncwarp();  // the slot's previous pixel is scored
-    const int n_staged = stage_modes(job, rec, slots[warp], lane);
-    for (int k = 0; k < n_here; ++k) {
-      float best;
-      float3 mu = make_float3(0.f, 0.f, 0.f);
-      if (n_staged >= 0) {
-        const float3 xk = make_float3(__shfl_sync(0xffffffffu, x.x, 16 * k), __shfl_sync(0xffffffffu, x.y, 16 * k),
-                                      __shfl_sync(0xffffffffu, x.z, 16 * k));
-        best = warp_best_staged(slots[warp], n_staged, xk, lane, &mu);
-      } else {
-        // more modes than a slot holds: the scan of refine_block's per-lane path, by lane 16 k
-        float b = -INFINITY;
-        if (lane == 16 * k) b = record_best(job, rec, slots[warp], -1, x, &mu);
-        best = __shfl_sync(0xffffffffu, b, 16 * k);
-        mu = make_float3(__shfl_sync(0xffffffffu, mu.x, 16 * k), __shfl_sync(0xffffffffu, mu.y, 16 * k),
-                         __shfl_sync(0xffffffffu, mu.z, 16 * k));
-      }
-      if (j == k && best != -INFINITY && dist2_rn(x, mu) < r2) {
-        const float u[3] = {c.x - cref.x, c.y - cref.y, c.z - cref.z};
-        const float w[3] = {mu.x - wref.x, mu.y - wref.y, mu.z - wref.z};
-        if (q == 0) {
-          acc += 1.f;
-        } else if (q < 4) {
-          comp_add(acc, lo, u[q - 1]);
-        } else if (q < 7) {
-          comp_add(acc, lo, w[q - 4]);
-        } else {
-          const float a = u[(q - 7) / 3], b = w[(q - 7) % 3];
-          const float pr = __fmul_rn(a, b);
-          comp_add(acc, lo, pr);
-          lo = __fadd_rn(lo, __fmaf_rn(a, b, -pr));
-        }
-      }
-    }
-  }
-  // the warps' partials combined as in refine_block: sums q = w, w + kRoundWarps of hypothesis
-  // `lane` by warp w, added in warp order
-  constexpr int kPer = (16 + kRoundWarps - 1) / kRoundWarps;
-  float sh[kPer], sl[kPer];
-#pragma unroll
-  for (int i = 0; i < kPer; ++i) sh[i] = sl[i] = 0.f;
-#pragma unroll
-  for (int pass = 0; pass < 2; ++pass) {
-    if (j < n_here) red[warp][q][j] = pass ? lo : acc;
-    __syncthreads();
-    if (lane < n_here) {
-#pragma unroll
-      for (int i = 0; i < kPer; ++i) {
-        const int qq = warp + i * kRoundWarps;
-        if (qq < 16)
-#pragma unroll
-          for (int w = 0; w < kRoundWarps; ++w) {
-            if (pass == 0) comp_add(sh[i], sl[i], red[w][qq][lane]);
-            else sl[i] = __fadd_rn(sl[i], red[w][qq][lane]);
-          }
-      }
-    }
-    __syncthreads();
-  }
-  if (part == 0 && warp == 0 && q == 0 && j < n_here && job.hyp_ok[h]) {
-    float* ref = job.refit_ref + (size_t)h * 8;  // written by the hypothesis's first lane
-    ref[0] = cref.x;
-    ref[1] = cref.y;
-    ref[2] = cref.z;
-    ref[3] = wref.x;
-    ref[4] = wref.y;
-    ref[5] = wref.z;
-  }
-  if (lane >= n_here) return;
-  const int hl = alive_out(job, r)[lane];
+  if (lane >= kHere || chunk * kHere + lane >= n_surv) return;
+  const int hl = alive_out(job, r)[chunk * kHere + lane];
   if (!job.hyp_ok[hl]) return;
 #pragma unroll
   for (int i = 0; i < kPer; ++i) {
-    const int qq = warp + i * kRoundWarps;
-    if (qq < 16) job.refit[((size_t)hl * job.refit_parts + part) * 16 + qq] = make_float2(sh[i], sl[i]);
+    const int q = warp + i * kRoundWarps;
+    if (q < 16) job.refit[((size_t)hl * job.refit_parts + part) * 16 + q] = make_float2(s_hi[i], s_lo[i]);
   }
 }
 
-// CTAs per SM for refine_few_kernel (one compensated pair per thread)
+// CTAs per SM the compiler must fit for the re-fit sums of one lane per survivor (the 16 compensated
+// sums per lane take registers); with more lanes per survivor a lane holds fewer and more CTAs fit
+#ifndef RELO_REFINE_MIN_BLOCKS
+#define RELO_REFINE_MIN_BLOCKS 2
+#endif
 #ifndef RELO_REFINE_FEW_MIN_BLOCKS
 #define RELO_REFINE_FEW_MIN_BLOCKS 4
 #endif
-__global__ void __launch_bounds__(kRoundWarps * 32, RELO_REFINE_FEW_MIN_BLOCKS)
-    refine_few_kernel(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ surv_prefix, int r) {
-  __shared__ ModeSlot slots[kRoundWarps];
-  __shared__ float red[kRoundWarps][16][32];
-  refine_few_block(jobs, surv_prefix, r, blockIdx.y, blockIdx.z, slots, red);
+template <int LG>
+__global__ void __launch_bounds__(kRoundWarps * 32, LG == 0 ? RELO_REFINE_MIN_BLOCKS : LG == 1 ? 3 : RELO_REFINE_FEW_MIN_BLOCKS)
+    refine_kernel(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ surv_prefix, int r) {
+  __shared__ RefineShared sh;
+  refine_block<LG>(jobs, surv_prefix, r, blockIdx.x, blockIdx.y, blockIdx.z, sh);
 }
 
 // Re-fit solve: thread per survivor; the parts' sums are added in order in FP64, then FP64 Horn on
@@ -1060,8 +1206,53 @@ __device__ __forceinline__ void refit_one(const RansacJob& job, int k, int r) {
     wb[k] = (double)ref[3 + k] + mw[k];
   }
   for (int p = 0; p < 3; ++p)
-    for (int q = 0; q < 3; ++q) S[3 * p + q] = f[7 + 3 * p + q] - n * mc[p] * mw[q];
+    for (int q = 0; q < 3; ++q) S[3 * p + q] = __fma_rn(-__dmul_rn(n, mc[p]), mw[q], f[7 + 3 * p + q]);
   horn_pose(S, cb, wb, job.poses + 12 * (size_t)h);
+}
+
+// refit_one of two survivors by a warp (survivor k by the group of 16 lanes; k < 0: none): lane q of
+// the group adds up sum q.
+__device__ __forceinline__ void refit_group(const RansacJob& job, int k, int r) {
+  const int l = threadIdx.x & 15;
+  int h = -1;
+  if (k >= 0 && !job_skipped(job.skip) && *job.n_valid != 0) {
+    h = alive_out(job, r)[k];
+    if (!job.hyp_ok[h]) h = -1;
+  }
+  double f = 0.0, ref = 0.0;
+  if (h >= 0) {
+    const int parts = ((r + 1) * job.B + kRefinePixels - 1) / kRefinePixels;
+    const float2* src = job.refit + (size_t)h * job.refit_parts * 16 + l;
+#pragma unroll 4
+    for (int p = 0; p < parts; ++p) {
+      const float2 v = src[16 * p];
+      f = __dadd_rn(f, __dadd_rn((double)v.x, (double)v.y));
+    }
+    if (l >= 1 && l < 7) ref = (double)job.refit_ref[(size_t)h * 8 + l - 1];
+  }
+  __syncwarp();
+  const double n = group_get(f, 0);
+  if (h >= 0 && l == 0) job.inliers[h] = (int)n;
+  const bool solve = h >= 0 && !(n < 3.0);
+  const double mean = __ddiv_rn(f, n);  // lanes 1..3: of the camera points, 4..6: of the scene points
+  const double centre = __dadd_rn(ref, mean);
+  double cb[3], wb[3];
+#pragma unroll
+  for (int q = 0; q < 3; ++q) {
+    cb[q] = group_get(centre, 1 + q);
+    wb[q] = group_get(centre, 4 + q);
+  }
+  // lane 3 p + q: S(p, q) = f[7 + 3 p + q] - n mc[p] mw[q]
+  const int p = min(l / 3, 2), q = l - 3 * (l / 3);
+  const double sum = group_get(f, min(7 + l, 15)), mc = group_get(mean, 1 + p), mw = group_get(mean, 4 + q);
+  horn_pose_group(__fma_rn(-__dmul_rn(n, mc), mw, sum), cb, wb, solve, h >= 0 ? job.poses + 12 * (size_t)h : nullptr);
+}
+
+__global__ void __launch_bounds__(32) refit_group_kernel(const RansacJob* __restrict__ jobs, int n_jobs,
+                                                         const int32_t* __restrict__ surv_prefix, int total, int r) {
+  const int gid = (int)blockIdx.x * kSolvesPerWarp + ((int)threadIdx.x >> 4);
+  const int jid = find_job_by(surv_prefix, n_jobs, min(gid, total - 1));
+  refit_group(jobs[jid], gid < total ? gid - surv_prefix[jid] : -1, r);
 }
 
 __global__ void __launch_bounds__(32) refit_kernel(const RansacJob* __restrict__ jobs, int n_jobs,
@@ -1073,24 +1264,58 @@ __global__ void __launch_bounds__(32) refit_kernel(const RansacJob* __restrict__
   refit_one(jobs[jid], gid - surv_prefix[jid], r);
 }
 
+template <int LG>
+void launch_refine(const RansacJob* jobs, int n_jobs, const int32_t* surv_prefix, int max_surv, int parts, int round,
+                   cudaStream_t s) {
+  constexpr int kHere = 32 >> LG;
+  refine_kernel<LG><<<dim3((max_surv + kHere - 1) / kHere, parts, n_jobs), kRoundWarps * 32, 0, s>>>(jobs, surv_prefix,
+                                                                                                    round);
+}
+
+int energy_splits(int n_jobs, int max_alive, int B) {
+  int sms = 0;
+  if (device_sms(&sms) != cudaSuccess) sms = 152;
+  const int ctas = (max_alive + 31) / 32 * n_jobs, rows = (B + kRoundWarps - 1) / kRoundWarps;
+  return std::max(1, std::min(rows, 2 * sms / std::max(1, ctas)));
+}
+
+int round_launches(int n_jobs, int max_alive, int B) { return energy_splits(n_jobs, max_alive, B) > 1 ? 5 : 4; }
+
+cudaError_t launch_draw(const RansacJob* jobs, int n_jobs, int round, const int32_t* alive_prefix_dev, cudaStream_t s) {
+  draw_kernel<<<n_jobs, 256, 0, s>>>(jobs, alive_prefix_dev, round);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int32_t* alive_prefix_dev,
                          int total_alive, int max_alive, const int32_t* surv_prefix_dev, int total_surv, int max_surv,
                          int B, cudaStream_t s, const Schedule& sched) {
   if (total_alive <= 0) return cudaSuccess;
   if (sched.refit_per < 0 || sched.refit_per > 32) return cudaErrorInvalidValue;
-  draw_kernel<<<n_jobs, 256, 0, s>>>(jobs, alive_prefix_dev, round);
-  energy_kernel<<<dim3((max_alive + 31) / 32, n_jobs), kRoundWarps * 32, 0, s>>>(jobs, alive_prefix_dev, round);
+  // few jobs: their pixels are split over more CTAs than the hypothesis chunks make
+  const int n_split = energy_splits(n_jobs, max_alive, B);
+  energy_kernel<<<dim3((max_alive + 31) / 32, n_jobs, n_split), kRoundWarps * 32, 0, s>>>(jobs, alive_prefix_dev, round);
+  if (n_split > 1)
+    sum_scores_kernel<<<dim3((max_alive * 8 + 255) / 256, n_jobs), 256, 0, s>>>(jobs, alive_prefix_dev, round, n_split);
   // the largest alive set (4096) bounds the shared memory of the sort
   select_kernel<<<n_jobs, 1024, 4096 * (sizeof(unsigned long long) + sizeof(int)), s>>>(jobs, alive_prefix_dev,
                                                                                         round);
   const int parts = ((round + 1) * B + kRefinePixels - 1) / kRefinePixels;
-  if (max_surv <= kFewHyps)
-    refine_few_kernel<<<dim3(1, parts, n_jobs), kRoundWarps * 32, 0, s>>>(jobs, surv_prefix_dev, round);
-  else
-    refine_kernel<<<dim3((max_surv + 31) / 32, parts, n_jobs), kRoundWarps * 32, 0, s>>>(jobs, surv_prefix_dev, round);
+  switch (group_log2(max_surv)) {
+    case 0: launch_refine<0>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 1: launch_refine<1>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 2: launch_refine<2>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 3: launch_refine<3>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 4: launch_refine<4>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    default: launch_refine<5>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+  }
   int n_sms = 0;
   const cudaError_t e = device_sms(&n_sms);
   if (e != cudaSuccess) return e;
+  if (sched.refit_per == 0 && total_surv <= kGroupSolves) {
+    refit_group_kernel<<<(unsigned)((total_surv + kSolvesPerWarp - 1) / kSolvesPerWarp), 32, 0, s>>>(
+        jobs, n_jobs, surv_prefix_dev, total_surv, round);
+    return cudaGetLastError();
+  }
   const int per = sched.refit_per > 0 ? sched.refit_per
                                      : std::max(1, std::min(32, (total_surv + 2 * n_sms - 1) / (2 * n_sms)));
   refit_kernel<<<(unsigned)((total_surv + per - 1) / per), 32, 0, s>>>(jobs, n_jobs, surv_prefix_dev, total_surv,
@@ -1187,7 +1412,8 @@ __device__ __forceinline__ int ld_acquire_gpu(const int32_t* p) {
 constexpr int kPersistThreads = kRoundWarps * 32;
 static_assert(kPersistThreads == kPersistThreadsHost, "the host's item chunks match the CTA size");
 constexpr size_t kPersistSmem = 4096 * (sizeof(unsigned long long) + sizeof(int));  // the largest sort
-static_assert(kRoundWarps * sizeof(ModeSlot) + sizeof(float) * kRoundWarps * 16 * 32 <= kPersistSmem,
+static_assert(sizeof(ModeSlots) * kRoundWarps + sizeof(float) * kRoundWarps * 32 <= kPersistSmem &&
+                  sizeof(RefineShared) <= kPersistSmem,
               "round stages fit the persistent kernel's shared memory");
 
 __global__ void __launch_bounds__(kPersistThreads, 2) persistent_kernel(PersistArgs a) {
@@ -1208,9 +1434,8 @@ __global__ void __launch_bounds__(kPersistThreads, 2) persistent_kernel(PersistA
   }
   __syncthreads();
   // phase 2: CTA items
-  ModeSlot* slots = reinterpret_cast<ModeSlot*>(psm);
-  float(*part)[32] = reinterpret_cast<float(*)[32]>(psm + kRoundWarps * sizeof(ModeSlot));
-  float(*red)[16][32] = reinterpret_cast<float(*)[16][32]>(psm + kRoundWarps * sizeof(ModeSlot));
+  ModeSlots* slots = reinterpret_cast<ModeSlots*>(psm);
+  float(*part)[32] = reinterpret_cast<float(*)[32]>(psm + kRoundWarps * sizeof(ModeSlots));
   for (;;) {
     if (threadIdx.x == 0) {
       const int it = atomicAdd(a.ctrl + 1, 1);
@@ -1251,14 +1476,15 @@ __global__ void __launch_bounds__(kPersistThreads, 2) persistent_kernel(PersistA
         draw_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.job);
         break;
       case kItemEnergy:
-        energy_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.sub, it.job, slots, part);
+        energy_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.sub, it.job, 0, 1, slots, part);
         break;
       case kItemSelect:
         select_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.job,
                      reinterpret_cast<unsigned long long*>(psm));
         break;
       case kItemRefine:
-        refine_block(a.jobs, a.surv_prefix + (size_t)it.round * np, it.round, it.sub, it.part, it.job, slots, red);
+        refine_block<0>(a.jobs, a.surv_prefix + (size_t)it.round * np, it.round, it.sub, it.part, it.job,
+                        *reinterpret_cast<RefineShared*>(psm));
         break;
       case kItemRefit: {
         const int32_t* sp = a.surv_prefix + (size_t)it.round * np;

@@ -193,6 +193,31 @@ __device__ __forceinline__ float3 apply(const PoseF& P, float3 c) {
                      fmaf(P.r[6], c.x, fmaf(P.r[7], c.y, fmaf(P.r[8], c.z, P.t[2]))));
 }
 
+// Pose [R | t] (12 doubles) of the rotation (w, x, y, z), normalised here, that maps centroid cbar to
+// wbar.  Every operation states its rounding, here and in horn_pose, so that both forms of the solve
+// (horn_pose by a thread, horn_pose_group by 16 lanes) give the same bits.
+__device__ __forceinline__ void quaternion_pose(double w, double x, double y, double z, const double cbar[3],
+                                                const double wbar[3], double* out) {
+  const double n = __dsqrt_rn(__fma_rn(z, z, __fma_rn(y, y, __fma_rn(x, x, __dmul_rn(w, w)))));
+  w = __ddiv_rn(w, n);
+  x = __ddiv_rn(x, n);
+  y = __ddiv_rn(y, n);
+  z = __ddiv_rn(z, n);
+  const double yy = __dmul_rn(y, y), zz = __dmul_rn(z, z);
+  const double R[9] = {__dsub_rn(1.0, 2 * __dadd_rn(yy, zz)),         2 * __fma_rn(x, y, -__dmul_rn(w, z)),
+                       2 * __fma_rn(x, z, __dmul_rn(w, y)),           2 * __fma_rn(x, y, __dmul_rn(w, z)),
+                       __dsub_rn(1.0, 2 * __fma_rn(x, x, zz)),        2 * __fma_rn(y, z, -__dmul_rn(w, x)),
+                       2 * __fma_rn(x, z, -__dmul_rn(w, y)),          2 * __fma_rn(y, z, __dmul_rn(w, x)),
+                       __dsub_rn(1.0, 2 * __fma_rn(x, x, yy))};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    out[4 * i + 0] = R[3 * i + 0];
+    out[4 * i + 1] = R[3 * i + 1];
+    out[4 * i + 2] = R[3 * i + 2];
+    out[4 * i + 3] = __dsub_rn(wbar[i], __fma_rn(R[3 * i + 2], cbar[2], __fma_rn(R[3 * i], cbar[0], __dmul_rn(R[3 * i + 1], cbar[1]))));
+  }
+}
+
 // Rigid transform from centroids and cross-covariance by Horn's closed form (1987): the rotation is
 // the unit quaternion of the largest eigenvalue of the symmetric 4x4 matrix N(S), S = sum of
 // (c - cbar)(w - wbar)^T.  The eigenproblem is solved by cyclic Jacobi rotations in FP64, which
@@ -214,9 +239,9 @@ __device__ inline void horn_pose(const double S[9], const double cbar[3], const 
     double off = 0.0, diag = 0.0;
 #pragma unroll
     for (int p = 0; p < 4; ++p) {
-      diag += A[p][p] * A[p][p];
+      diag = __fma_rn(A[p][p], A[p][p], diag);
 #pragma unroll
-      for (int q = p + 1; q < 4; ++q) off += A[p][q] * A[p][q];
+      for (int q = p + 1; q < 4; ++q) off = __fma_rn(A[p][q], A[p][q], off);
     }
     if (off <= 1e-30 * (diag + 1e-300)) break;
 #pragma unroll
@@ -229,10 +254,11 @@ __device__ inline void horn_pose(const double S[9], const double cbar[3], const 
         cs[r] = 1.0;
         sn[r] = 0.0;
         if (fabs(apq) >= 1e-300) {
-          const double theta = (A[q][q] - A[p][p]) / (2.0 * apq);
-          const double t = (theta >= 0.0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-          cs[r] = rsqrt(t * t + 1.0);
-          sn[r] = t * cs[r];
+          const double theta = __ddiv_rn(__dsub_rn(A[q][q], A[p][p]), 2.0 * apq);
+          const double t = __ddiv_rn(theta >= 0.0 ? 1.0 : -1.0,
+                                     __dadd_rn(fabs(theta), __dsqrt_rn(__fma_rn(theta, theta, 1.0))));
+          cs[r] = rsqrt(__fma_rn(t, t, 1.0));
+          sn[r] = __dmul_rn(t, cs[r]);
         }
       }
 #pragma unroll
@@ -242,20 +268,20 @@ __device__ inline void horn_pose(const double S[9], const double cbar[3], const 
 #pragma unroll
         for (int k = 0; k < 4; ++k) {  // A <- J^T A J
           const double akp = A[k][p], akq = A[k][q];
-          A[k][p] = c * akp - s * akq;
-          A[k][q] = s * akp + c * akq;
+          A[k][p] = __fma_rn(c, akp, -__dmul_rn(s, akq));
+          A[k][q] = __fma_rn(s, akp, __dmul_rn(c, akq));
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const double apk = A[p][k], aqk = A[q][k];
-          A[p][k] = c * apk - s * aqk;
-          A[q][k] = s * apk + c * aqk;
+          A[p][k] = __fma_rn(c, apk, -__dmul_rn(s, aqk));
+          A[q][k] = __fma_rn(s, apk, __dmul_rn(c, aqk));
         }
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
           const double vkp = V[k][p], vkq = V[k][q];
-          V[k][p] = c * vkp - s * vkq;
-          V[k][q] = s * vkp + c * vkq;
+          V[k][p] = __fma_rn(c, vkp, -__dmul_rn(s, vkq));
+          V[k][q] = __fma_rn(s, vkp, __dmul_rn(c, vkq));
         }
       }
     }
@@ -270,17 +296,7 @@ __device__ inline void horn_pose(const double S[9], const double cbar[3], const 
       y = V[2][k];
       z = V[3][k];
     }
-  const double n = sqrt(w * w + x * x + y * y + z * z);
-  w /= n; x /= n; y /= n; z /= n;
-  const double R[9] = {1 - 2 * (y * y + z * z), 2 * (x * y - w * z),     2 * (x * z + w * y),
-                       2 * (x * y + w * z),     1 - 2 * (x * x + z * z), 2 * (y * z - w * x),
-                       2 * (x * z - w * y),     2 * (y * z + w * x),     1 - 2 * (x * x + y * y)};
-  for (int i = 0; i < 3; ++i) {
-    out[4 * i + 0] = R[3 * i + 0];
-    out[4 * i + 1] = R[3 * i + 1];
-    out[4 * i + 2] = R[3 * i + 2];
-    out[4 * i + 3] = wbar[i] - (R[3 * i] * cbar[0] + R[3 * i + 1] * cbar[1] + R[3 * i + 2] * cbar[2]);
-  }
+  quaternion_pose(w, x, y, z, cbar, wbar, out);
 }
 
 // Warp-wide sum (all lanes get the result).
@@ -455,10 +471,15 @@ cudaError_t launch_scene_lookup(SceneView sv, const int32_t* keys, int64_t n, in
 // RANSAC stages over a device array of jobs.
 inline int table_words(int T) { return (3 + T + 7) / 8; }
 cudaError_t launch_compact(const RansacJob* jobs, int n_jobs, int total_chunks, cudaStream_t s);
-// counter_dev: one int of device scratch the search's warps take hypotheses from (zeroed here)
+// counter_dev: one int of device scratch the search's warps take hypotheses from (zeroed here);
+// max_draws > 0: every job's drawn pixels too (all its rounds), max_draws the most of any job
 cudaError_t launch_hypotheses(const RansacJob* jobs, int n_jobs, int total_hyps, int32_t* counter_dev, cudaStream_t s,
-                              const Schedule& sched = Schedule());
-// round r: prefix[n_jobs + 1] = flattened alive-hypothesis offsets of the jobs still running
+                              const Schedule& sched = Schedule(), int max_draws = 0);
+// the drawn pixels of one round
+cudaError_t launch_draw(const RansacJob* jobs, int n_jobs, int round, const int32_t* alive_prefix_dev, cudaStream_t s);
+// round r, its pixels drawn: prefix[n_jobs + 1] = flattened alive-hypothesis offsets of the jobs still
+// running.  It takes round_launches(n_jobs, max_alive, B) launches.
+int round_launches(int n_jobs, int max_alive, int B);
 cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int32_t* alive_prefix_dev,
                          int total_alive, int max_alive, const int32_t* surv_prefix_dev, int total_surv, int max_surv,
                          int B, cudaStream_t s, const Schedule& sched = Schedule());
