@@ -267,8 +267,9 @@ relo_status relo_forest_eval(const relo_forest* forest, const uint16_t* depth_de
  * device and offers each pixel's scene coordinate P * backproject(depth) to its leaf's
  * reservoir (Algorithm R, capacity per leaf, Philox4x32-10 draws keyed by seed at counter
  * (3, tree * 2^depth + leaf, n_lo, n_hi) for the n-th offer, n from 0; the offer replaces
- * slot floor(word0 * (n+1) / 2^32) if that is below capacity).  Reservoir updates run on the
- * host in frame order (synchronous call).  relo_forest_train_finish runs mean shift on every
+ * slot floor(word0 * (n+1) / 2^32) if that is below capacity).  The reservoirs live on the device
+ * (12 bytes per leaf and slot), from the first frame until the forest is destroyed or a training of
+ * another size begins (synchronous call).  relo_forest_train_finish runs mean shift on every
  * leaf (Gaussian kernel of the given bandwidth from every sample, until the shift is below
  * tol or max_iter steps; a converged point joins the first mode whose opening point lies
  * within merge_dist; per mode: mean and covariance of its members + cov_floor I; keep the

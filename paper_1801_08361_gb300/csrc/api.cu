@@ -1064,9 +1064,11 @@ void relo_destroy_forest(relo_forest* f) {
   relo::dev_free(f->d_modes);
   relo::dev_free(f->d_n_modes);
   relo::dev_free(f->d_top);
-  free(f->res_samples);
-  free(f->res_count);
-  free(f->res_seen);
+  relo::dev_free(f->res_samples);
+  relo::dev_free(f->res_count);
+  relo::dev_free(f->res_seen);
+  relo::dev_free(f->res_runs);
+  relo::dev_free(f->d_scratch);
   delete f;
 }
 
@@ -1101,18 +1103,59 @@ relo_status relo_forest_train_begin(relo_forest* f, const relo_train_params* p) 
   if (!f || !p) return fail(RELO_EINVAL, "null forest or params");
   if (p->capacity < 1 || p->capacity > 4096) return fail(RELO_EINVAL, "capacity outside [1, 4096]");
   if (p->stride < 1 || p->max_iter < 1 || !(p->bandwidth > 0)) return fail(RELO_EINVAL, "bad training params");
-  const size_t L = (size_t)f->T << f->D;
-  free(f->res_samples);
-  free(f->res_count);
-  free(f->res_seen);
-  f->res_samples = (float*)calloc(L * p->capacity * 3, sizeof(float));
-  f->res_count = (int32_t*)calloc(L, sizeof(int32_t));
-  f->res_seen = (int64_t*)calloc(L, sizeof(int64_t));
-  if (!f->res_samples || !f->res_count || !f->res_seen) return fail(RELO_ENOMEM, "host reservoirs");
   f->train = *p;
   f->training = true;
+  f->res_ready = false;  // zeroed by the first frame, on its stream
   return RELO_OK;
 }
+
+}  // extern "C"
+
+namespace {
+// The reservoirs of the training begun last, allocated (kept from an earlier training of the same
+// size) and zeroed on s.
+relo_status ready_reservoirs(relo_forest* f, cudaStream_t s) {
+  if (f->res_ready) return RELO_OK;
+  const size_t L = (size_t)f->T << f->D, slots = L * f->train.capacity;
+  if (f->res_slots != slots) {
+    auto release = [f] {
+      relo::dev_free(f->res_samples);
+      relo::dev_free(f->res_count);
+      relo::dev_free(f->res_seen);
+      relo::dev_free(f->res_runs);
+      f->res_samples = nullptr;
+      f->res_count = nullptr;
+      f->res_seen = nullptr;
+      f->res_runs = nullptr;
+      f->res_slots = 0;
+    };
+    release();
+    if (relo::dev_malloc((void**)&f->res_samples, slots * 3 * sizeof(float)) != cudaSuccess ||
+        relo::dev_malloc((void**)&f->res_count, L * sizeof(int32_t)) != cudaSuccess ||
+        relo::dev_malloc((void**)&f->res_seen, L * sizeof(int64_t)) != cudaSuccess ||
+        relo::dev_malloc((void**)&f->res_runs, 2 * L * sizeof(int32_t)) != cudaSuccess) {
+      cudaGetLastError();
+      release();
+      return fail(RELO_ENOMEM, "reservoirs");
+    }
+    f->res_slots = slots;
+  }
+  RELO_CUDA(cudaMemsetAsync(f->res_samples, 0, slots * 3 * sizeof(float), s));
+  RELO_CUDA(cudaMemsetAsync(f->res_count, 0, L * sizeof(int32_t), s));
+  RELO_CUDA(cudaMemsetAsync(f->res_seen, 0, L * sizeof(int64_t), s));
+  RELO_CUDA(cudaMemsetAsync(f->res_runs, 0, 2 * L * sizeof(int32_t), s));
+  f->res_ready = true;
+  return RELO_OK;
+}
+
+// Trees whose items are sorted together: the sort's buffers (16 bytes per grid pixel and tree) stay
+// within half a gigabyte, or one tree's.
+int trees_at_once(int T, int64_t n) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>(T, ((int64_t)512 << 20) / (16 * std::max<int64_t>(n, 1))));
+}
+}  // namespace
+
+extern "C" {
 
 relo_status relo_forest_train_frame(relo_forest* f, const relo_intrinsics* intr, const double pose[16],
                                     const uint16_t* depth, const uint8_t* rgba, relo_stream stream) {
@@ -1122,93 +1165,101 @@ relo_status relo_forest_train_frame(relo_forest* f, const relo_intrinsics* intr,
   if (st) return st;
   const int W = intr->width, H = intr->height, S = f->train.stride, T = f->T;
   const int gw = (W + S - 1) / S, gh = (H + S - 1) / S;
-  const size_t n_pix = (size_t)W * H;
+  const int64_t n = (int64_t)gw * gh;
   cudaStream_t s = (cudaStream_t)stream;
-  uint16_t* d_leaves = nullptr;
-  float* d_coords = nullptr;
-  RELO_CUDA(relo::dev_malloc((void**)&d_leaves, n_pix * T * sizeof(uint16_t)));
-  if (relo::dev_malloc((void**)&d_coords, (size_t)gw * gh * 3 * sizeof(float)) != cudaSuccess) {
-    relo::dev_free(d_leaves);
-    return fail(RELO_ENOMEM, "training scratch");
+  st = ready_reservoirs(f, s);
+  if (st) return st;
+  ReservoirFrame r{};
+  r.depth = depth;
+  r.W = W;
+  r.stride = S;
+  r.gw = gw;
+  r.n = n;
+  r.D = f->D;
+  r.per_block = (int)std::max<int64_t>(kSortItems, ((n + kSortBlocks - 1) / kSortBlocks + 255) / 256 * 256);
+  r.blocks = (int)((n + r.per_block - 1) / r.per_block);
+  r.start = f->res_runs;
+  r.end = f->res_runs + ((size_t)T << f->D);
+  r.samples = f->res_samples;
+  r.count = f->res_count;
+  r.seen = f->res_seen;
+  r.capacity = f->train.capacity;
+  r.key0 = (uint32_t)(f->train.seed & 0xFFFFFFFFu);
+  r.key1 = (uint32_t)(f->train.seed >> 32);
+  const int step = trees_at_once(T, n);
+  uint16_t* leaves = nullptr;
+  float* coords = nullptr;
+  auto layout = [&](char* base) {
+    Carver c{base, 0};
+    leaves = c.take<uint16_t>((size_t)n * T);
+    coords = c.take<float>((size_t)n * 3);
+    r.items[0] = c.take<uint64_t>((size_t)n * step);
+    r.items[1] = c.take<uint64_t>((size_t)n * step);
+    r.hist = c.take<uint32_t>((size_t)256 * r.blocks * step);
+    r.n_valid = c.take<int32_t>(step);
+    return c.off;
+  };
+  const size_t need = layout(nullptr);
+  if (f->scratch_bytes < need) {
+    relo::dev_free(f->d_scratch);
+    f->d_scratch = nullptr;
+    f->scratch_bytes = 0;
+    if (relo::dev_malloc(&f->d_scratch, need) != cudaSuccess) {
+      cudaGetLastError();
+      f->d_scratch = nullptr;
+      return fail(RELO_ENOMEM, "training scratch");
+    }
+    f->scratch_bytes = need;
   }
+  layout((char*)f->d_scratch);
+  r.coords = coords;
   ForestJob j{};
   j.forest = f->view;
   j.depth = depth;
   j.rgba = (const uint32_t*)rgba;
-  j.leaves = d_leaves;
+  j.leaves = leaves;
   j.W = W;
   j.H = H;
-  std::vector<uint16_t> leaves(n_pix * T), dep(n_pix);
-  std::vector<float> coords((size_t)gw * gh * 3);
-  cudaError_t e = launch_forest(nullptr, 1, &j, (int64_t)n_pix, s, T);
-  if (e == cudaSuccess) e = launch_scene_coords(depth, W, H, S, intr->fx, intr->fy, intr->cx, intr->cy, pose, d_coords, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(leaves.data(), d_leaves, leaves.size() * 2, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(dep.data(), depth, n_pix * 2, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(coords.data(), d_coords, coords.size() * 4, cudaMemcpyDeviceToHost, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  relo::dev_free(d_leaves);
-  relo::dev_free(d_coords);
-  if (e != cudaSuccess) return cuda_fail(e, "training frame");
-  // Algorithm R per leaf, offers in raster order, trees in order (host, sequential by definition)
-  const int cap = f->train.capacity;
-  const int64_t L = (int64_t)1 << f->D;
-  const uint32_t k0 = (uint32_t)(f->train.seed & 0xFFFFFFFFu), k1 = (uint32_t)(f->train.seed >> 32);
-  for (int v = 0; v < H; v += S) {
-    for (int u = 0; u < W; u += S) {
-      const size_t pix = (size_t)v * W + u;
-      if (dep[pix] == 0) continue;
-      const float* w = &coords[3 * ((size_t)(v / S) * gw + u / S)];
-      for (int t = 0; t < T; ++t) {
-        const int64_t id = (int64_t)t * L + leaves[(size_t)t * n_pix + pix];
-        const int64_t n = f->res_seen[id]++;
-        int64_t slot = -1;
-        if (n < cap) {
-          slot = n;
-          f->res_count[id] = (int32_t)(n + 1);
-        } else {
-          const uint4 x = philox4x32_10(make_uint4(3u, (uint32_t)id, (uint32_t)(n & 0xFFFFFFFF), (uint32_t)(n >> 32)), k0, k1);
-          const uint64_t jj = ((uint64_t)x.x * (uint64_t)(n + 1)) >> 32;
-          if (jj < (uint64_t)cap) slot = (int64_t)jj;
-        }
-        if (slot >= 0) std::memcpy(&f->res_samples[((size_t)id * cap + slot) * 3], w, 3 * sizeof(float));
-      }
-    }
+  cudaError_t e = launch_forest_grid(j, S, s);
+  if (e == cudaSuccess) e = launch_scene_coords(depth, W, H, S, intr->fx, intr->fy, intr->cx, intr->cy, pose, coords, s);
+  for (int t = 0; e == cudaSuccess && t < T; t += step) {
+    r.leaves = leaves + (size_t)n * t;
+    r.tree0 = t;
+    r.trees = std::min(step, T - t);
+    e = launch_reservoirs(r, s);
   }
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) return cuda_fail(e, "training frame");
   return RELO_OK;
 }
 
 relo_status relo_forest_train_reservoirs(const relo_forest* f, float* samples, int32_t* count) {
   if (!f || !f->training) return fail(RELO_EINVAL, "training not begun");
-  const size_t L = (size_t)f->T << f->D;
-  if (samples) std::memcpy(samples, f->res_samples, L * f->train.capacity * 3 * sizeof(float));
-  if (count) std::memcpy(count, f->res_count, L * sizeof(int32_t));
+  const size_t L = (size_t)f->T << f->D, bytes = L * f->train.capacity * 3 * sizeof(float);
+  if (!f->res_ready) {  // no frame yet
+    if (samples) std::memset(samples, 0, bytes);
+    if (count) std::memset(count, 0, L * sizeof(int32_t));
+    return RELO_OK;
+  }
+  if (samples) RELO_CUDA(cudaMemcpy(samples, f->res_samples, bytes, cudaMemcpyDeviceToHost));
+  if (count) RELO_CUDA(cudaMemcpy(count, f->res_count, L * sizeof(int32_t), cudaMemcpyDeviceToHost));
   return RELO_OK;
 }
 
 relo_status relo_forest_train_finish(relo_forest* f, relo_stream stream) {
   if (!f || !f->training) return fail(RELO_EINVAL, "training not begun");
   const size_t L = (size_t)f->T << f->D;
-  const int cap = f->train.capacity;
   cudaStream_t s = (cudaStream_t)stream;
-  float* d_samples = nullptr;
-  int32_t* d_count = nullptr;
-  RELO_CUDA(relo::dev_malloc((void**)&d_samples, L * cap * 3 * sizeof(float)));
-  if (relo::dev_malloc((void**)&d_count, L * sizeof(int32_t)) != cudaSuccess) {
-    relo::dev_free(d_samples);
-    return fail(RELO_ENOMEM, "training scratch");
-  }
-  cudaError_t e = cudaMemcpyAsync(d_samples, f->res_samples, L * cap * 3 * sizeof(float), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_count, f->res_count, L * sizeof(int32_t), cudaMemcpyHostToDevice, s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(f->d_modes, 0, L * f->M * kModeFloats * sizeof(float), s);
+  const relo_status st = ready_reservoirs(f, s);
+  if (st) return st;
+  cudaError_t e = cudaMemsetAsync(f->d_modes, 0, L * f->M * kModeFloats * sizeof(float), s);
   if (e == cudaSuccess)
-    e = launch_mean_shift(d_samples, d_count, cap, (int)L, (float)f->train.bandwidth, (float)f->train.tol,
-                          f->train.max_iter, (float)f->train.merge_dist, (float)f->train.cov_floor, f->M,
-                          (float*)f->d_modes, (uint8_t*)f->d_n_modes, s);
+    e = launch_mean_shift(f->res_samples, f->res_count, f->train.capacity, (int)L, (float)f->train.bandwidth,
+                          (float)f->train.tol, f->train.max_iter, (float)f->train.merge_dist, (float)f->train.cov_floor,
+                          f->M, (float*)f->d_modes, (uint8_t*)f->d_n_modes, s);
   if (e == cudaSuccess) e = launch_top_modes((const float*)f->d_modes, (const uint8_t*)f->d_n_modes, (int)L, f->M,
                                              (float4*)f->d_top, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  relo::dev_free(d_samples);
-  relo::dev_free(d_count);
   if (e != cudaSuccess) return cuda_fail(e, "mean shift");
   return RELO_OK;
 }

@@ -151,6 +151,29 @@ __device__ __forceinline__ void descend_any(const ForestJob& job, int u, int v, 
   else descend<MT, kDiv, kPacked, true>(job, u, v, dv, node, top_levels);
 }
 
+// The leaf nodes of pixel (u, v) of depth d > 0 in every tree.
+template <int MT>
+__device__ __forceinline__ void descend_pixel(const ForestJob& job, int u, int v, int d, int (&node)[MT],
+                                              int top_levels) {
+  const ForestView& f = job.forest;
+#pragma unroll
+  for (int t = 0; t < MT; ++t) node[t] = 0;
+  if (f.offset_shift == 7 && d >= 16) {
+    const DepthDivisor dv = make_divisor7(d);
+    if (job.packed) descend_any<MT, 2, true>(job, u, v, d, dv, node, top_levels);
+    else descend_any<MT, 2, false>(job, u, v, d, dv, node, top_levels);
+  } else {
+    const DepthDivisor dv = make_divisor(d);
+    if (job.packed) {
+      if (dv.shift >= 32) descend_any<MT, 1, true>(job, u, v, d, dv, node, top_levels);
+      else descend_any<MT, 0, true>(job, u, v, d, dv, node, top_levels);
+    } else {
+      if (dv.shift >= 32) descend_any<MT, 1, false>(job, u, v, d, dv, node, top_levels);
+      else descend_any<MT, 0, false>(job, u, v, d, dv, node, top_levels);
+    }
+  }
+}
+
 // CTAs of 256 threads per SM the compiler must fit: full occupancy (7 and 8 tie, 6 is 10 % slower
 // on the house workload)
 #ifndef RELO_FOREST_MIN_BLOCKS
@@ -222,26 +245,45 @@ __global__ void __launch_bounds__(256, RELO_FOREST_MIN_BLOCKS)
   }
   const int n_int = (1 << f.D) - 1;
   int node[MT];
-#pragma unroll
-  for (int t = 0; t < MT; ++t) node[t] = 0;
-  if (f.offset_shift == 7 && d >= 16) {
-    const DepthDivisor dv = make_divisor7(d);
-    if (job.packed) descend_any<MT, 2, true>(job, u, v, d, dv, node, top_levels);
-    else descend_any<MT, 2, false>(job, u, v, d, dv, node, top_levels);
-  } else {
-    const DepthDivisor dv = make_divisor(d);
-    if (job.packed) {
-      if (dv.shift >= 32) descend_any<MT, 1, true>(job, u, v, d, dv, node, top_levels);
-      else descend_any<MT, 0, true>(job, u, v, d, dv, node, top_levels);
-    } else {
-      if (dv.shift >= 32) descend_any<MT, 1, false>(job, u, v, d, dv, node, top_levels);
-      else descend_any<MT, 0, false>(job, u, v, d, dv, node, top_levels);
-    }
-  }
+  descend_pixel<MT>(job, u, v, d, node, top_levels);
 #pragma unroll
   for (int t = 0; t < MT; ++t)
     if (t < T && RELO_CHECK(node[t] >= n_int && node[t] < 2 * n_int + 1))
       job.leaves[(size_t)t * n_pix + pix] = (uint16_t)(node[t] - n_int);
+}
+
+// Training: the leaves of the pixels on a stride grid, thread per grid pixel.
+template <int MT>
+__global__ void __launch_bounds__(256, RELO_FOREST_MIN_BLOCKS)
+    forest_grid_kernel(const __grid_constant__ ForestJob job, int stride, int gw, int64_t n) {
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  const int u = (int)(i % gw) * stride, v = (int)(i / gw) * stride;
+  const ForestView& f = job.forest;
+  const int T = f.T, n_int = (1 << f.D) - 1;
+  const int d = __ldg(&job.depth[(int64_t)v * job.W + u]);
+  if (d == 0) {
+    for (int t = 0; t < T; ++t) job.leaves[(size_t)t * n + i] = 0xFFFF;
+    return;
+  }
+  int node[MT];
+  descend_pixel<MT>(job, u, v, d, node, 0);
+#pragma unroll
+  for (int t = 0; t < MT; ++t)
+    if (t < T && RELO_CHECK(node[t] >= n_int && node[t] < 2 * n_int + 1))
+      job.leaves[(size_t)t * n + i] = (uint16_t)(node[t] - n_int);
+}
+
+cudaError_t launch_forest_grid(const ForestJob& job, int stride, cudaStream_t s) {
+  const int gw = (job.W + stride - 1) / stride;
+  const int64_t n = (int64_t)gw * ((job.H + stride - 1) / stride);
+  const unsigned grid = (unsigned)((n + 255) / 256);
+  const int T = job.forest.T;
+  if (T <= 4) forest_grid_kernel<4><<<grid, 256, 0, s>>>(job, stride, gw, n);
+  else if (T <= 5) forest_grid_kernel<5><<<grid, 256, 0, s>>>(job, stride, gw, n);
+  else if (T <= 8) forest_grid_kernel<8><<<grid, 256, 0, s>>>(job, stride, gw, n);
+  else forest_grid_kernel<kMaxTrees><<<grid, 256, 0, s>>>(job, stride, gw, n);
+  return cudaGetLastError();
 }
 
 RELO_DEFINE_CHECK_READER(check_failures_forest)

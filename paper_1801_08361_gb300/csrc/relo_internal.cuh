@@ -512,6 +512,32 @@ cudaError_t persistent_grid(int* grid);
 
 
 // Training
+// Leaves of the pixels (u, v) = stride * (grid column, grid row): out [T][ceil(H / stride)][ceil(W / stride)].
+cudaError_t launch_forest_grid(const ForestJob& job, int stride, cudaStream_t s);
+// One frame's offers to the reservoirs of `trees` trees from tree0 (training.cu).
+constexpr int kSortItems = 2048, kSortBlocks = 64;  // the sort's CTAs per tree: at least so many items each, at most so many CTAs
+struct ReservoirFrame {
+  const uint16_t* depth;       // [H][W]
+  const uint16_t* leaves;      // [trees][n] leaf of each grid pixel
+  const float* coords;         // [n][3] scene coordinates of the grid pixels
+  int W, stride, gw;
+  int64_t n;                   // grid pixels
+  int trees, tree0, D;
+  int blocks, per_block;       // CTAs of the sort per tree, items of each (a multiple of 256)
+  // scratch
+  uint64_t* items[2];          // [trees][n] leaf << 32 | grid pixel, after each pass
+  uint32_t* hist;              // [trees][blocks][256]
+  int32_t* n_valid;            // [trees] valid pixels
+  // by global leaf id
+  int32_t* start;              // run of each leaf in its tree's sorted items
+  int32_t* end;
+  float* samples;              // [T][2^D][capacity][3]
+  int32_t* count;
+  int64_t* seen;
+  int capacity;
+  uint32_t key0, key1;
+};
+cudaError_t launch_reservoirs(const ReservoirFrame& f, cudaStream_t s);
 cudaError_t launch_scene_coords(const uint16_t* depth, int W, int H, int stride, double fx, double fy, double cx,
                                 double cy, const double* P /*16 host values passed by value*/, float* out,
                                 cudaStream_t s);
@@ -612,10 +638,16 @@ struct relo_forest {
   void* d_n_modes;
   void* d_top;
   int32_t T, D, M;
-  // training state (host)
+  // training state
   relo_train_params train;
   bool training;
+  // reservoirs on the device, allocated and zeroed by the first frame after train_begin
+  bool res_ready;
   float* res_samples;   // [T][L][cap][3]
   int32_t* res_count;   // [T][L]
   int64_t* res_seen;    // [T][L]
+  int32_t* res_runs;    // [2][T][L] a frame's runs (ReservoirFrame::start, end)
+  size_t res_slots;     // capacity of res_samples (T L cap)
+  void* d_scratch;      // a frame's scratch, kept between frames
+  size_t scratch_bytes;
 };

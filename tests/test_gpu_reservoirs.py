@@ -1,0 +1,51 @@
+"""The reservoirs of forest training against the oracle's (which offers pixel by pixel), at the edges
+of the device's sort: one and two digits of leaf ids, grids below one block and not a multiple of it,
+the largest leaf id, many offers to one leaf (every pixel in the same leaf: offers compete for slots
+within and across steps of 32), frames without depth, and a second training of the same forest."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1801_08361_gb300 import binding as B
+from paper_1801_08361_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda:0")
+
+
+def _frames(W, H, flat, seed):
+    rng = np.random.default_rng(seed)
+    for k in range(3):
+        depth = np.full((H, W), 1500, np.uint16) if flat else rng.integers(300, 6000, (H, W)).astype(np.uint16)
+        if not flat:
+            depth[rng.random((H, W)) < 0.3] = 0
+        if k == 1:
+            depth[:] = 0
+        rgba = np.full((H, W, 4), 90, np.uint8) if flat else rng.integers(0, 256, (H, W, 4)).astype(np.uint8)
+        yield depth, rgba
+
+
+@pytest.mark.parametrize("trees,depth,capacity,stride,W,H,flat", [
+    (1, 3, 5, 1, 17, 11, False), (2, 8, 4, 1, 64, 32, False), (3, 9, 3, 2, 131, 97, False),
+    (2, 16, 2, 1, 90, 50, False), (2, 16, 3, 1, 64, 65, True), (5, 10, 64, 3, 200, 152, False),
+    (1, 1, 40, 1, 96, 72, True)])
+def test_reservoirs_match_the_oracle(trees, depth, capacity, stride, W, H, flat):
+    nodes = synth.random_forest_nodes(trees, depth, seed=depth, offset=130, depth_tau=300, colour_tau=64)
+    if flat:  # equal probes everywhere and thresholds below zero: every pixel goes right, to the last leaf
+        nodes["tau"] = -1
+    intr = synth.Intrinsics.for_size(W, H, 12.0)
+    pose = synth.look_pose(np.array([1.0, 2.0, 1.5]), 0.3, -0.1)
+    f = B.Forest(nodes, max_modes=4)
+    for seed in (5, (7 << 32) + 9):  # the second training starts from empty reservoirs
+        want = oracle.Reservoirs(nodes, oracle.LeafParams(capacity=capacity, max_modes=4, seed=seed, stride=stride))
+        B.forest_train_begin(f, B.train_params(capacity=capacity, stride=stride, seed=seed))
+        for d, c in _frames(W, H, flat, seed % 1000):
+            want.add_frame(intr, pose, d, c)
+            B.forest_train_frame(f, intr, pose, torch.from_numpy(d.view(np.int16)).to(DEV), torch.from_numpy(c).to(DEV))
+        samples, count = B.forest_train_reservoirs(f, capacity)
+        so, co = want.contents()
+        assert np.array_equal(count, co)
+        assert np.array_equal(samples, so)
+        if flat:
+            assert count[:, -1].min() == min(capacity, 2 * len(range(0, W, stride)) * len(range(0, H, stride)))
