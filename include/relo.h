@@ -191,7 +191,8 @@ relo_status relo_render_global(const relo_scene* const* scenes, const double* gl
  * the device allocates them; coordinates and contents do not depend on it.
  * ------------------------------------------------------------------------------------- */
 /* An empty scene with room for capacity_blocks blocks (tsdf f32, colour u8x4 and weight u16 per
- * voxel: 5 KB per block, allocated now) and 2^log2_buckets buckets.
+ * voxel: 5 KB per block, allocated now), 2^log2_buckets buckets and 2 MB of occupancy bits that let
+ * raycasts cross empty space without looking blocks up.
  * Errors: RELO_EINVAL (capacity outside [1, 2^24], log2_buckets outside [4, 30], voxel_size or mu
  * <= 0, max_weight outside [1, 65535]), RELO_ENOMEM, RELO_ECUDA. */
 relo_status relo_create_fusion_scene(int64_t capacity_blocks, double voxel_size, double mu, int32_t log2_buckets,

@@ -600,6 +600,7 @@ void relo_destroy_scene(relo_scene* s) {
   relo::dev_free(s->d_grid);
   relo::dev_free(s->d_tsdf9);
   relo::dev_free(s->d_weight);
+  relo::dev_free(s->d_cells);
   relo::dev_free(s->d_coords);
   relo::dev_free(s->d_counters);
   delete s;
@@ -627,6 +628,8 @@ relo_status relo_create_fusion_scene(int64_t capacity, double voxel, double mu, 
   if (e == cudaSuccess) e = relo::dev_malloc((void**)&s->d_rgba, nv * sizeof(uint32_t));
   if (e == cudaSuccess) e = relo::dev_malloc((void**)&s->d_weight, nv * sizeof(uint16_t));
   if (e == cudaSuccess) e = relo::dev_malloc((void**)&s->d_coords, (size_t)capacity * sizeof(int4));
+  const size_t cell_bytes = sizeof(unsigned long long) << (3 * kCellBits);
+  if (e == cudaSuccess) e = relo::dev_malloc(&s->d_cells, cell_bytes);
   if (e == cudaSuccess) e = relo::dev_malloc((void**)&s->d_counters, 4 * sizeof(int32_t) + sizeof(unsigned long long));
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -640,6 +643,7 @@ relo_status relo_create_fusion_scene(int64_t capacity, double voxel, double mu, 
   if (e == cudaSuccess) e = cudaMemset(s->d_rgba, 0, nv * sizeof(uint32_t));
   if (e == cudaSuccess) e = cudaMemset(s->d_weight, 0, nv * sizeof(uint16_t));
   if (e == cudaSuccess) e = cudaMemset(s->d_counters, 0, 4 * sizeof(int32_t) + sizeof(unsigned long long));
+  if (e == cudaSuccess) e = cudaMemset(s->d_cells, 0, cell_bytes);
   if (e == cudaSuccess) e = launch_fuse_init((float*)s->d_tsdf, (int64_t)nv, nullptr);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
@@ -661,6 +665,7 @@ relo_status relo_create_fusion_scene(int64_t capacity, double voxel, double mu, 
   v.inv_block = (float)(1.0 / (8.0 * voxel));
   v.grid = nullptr;
   v.tsdf9 = nullptr;  // fusion changes the voxels: the raycast reads them directly
+  v.cells = (const unsigned long long*)s->d_cells;
   *out = s;
   return RELO_OK;
 }
@@ -724,6 +729,7 @@ relo_status relo_fuse_frame(relo_scene* scene, const relo_intrinsics* intr, cons
   j.counters = (int32_t*)scene->d_counters;
   j.status = j.counters + 2;
   j.updates = (unsigned long long*)(j.counters + 4);
+  j.cells = (unsigned long long*)scene->d_cells;
   j.bucket_mask = scene->view.mask;
   j.capacity = (int32_t)scene->capacity;
   j.max_weight = scene->max_weight;
@@ -932,7 +938,7 @@ relo_status relo_raycast_views(const relo_scene* scene, const relo_intrinsics* i
   RELO_CUDA(cudaMemcpyAsync(ws, jobs.data(), n * sizeof(RayJob), cudaMemcpyHostToDevice, s));
   // a copy from pageable memory returns once the host buffer has been staged, so jobs may go
   RELO_CUDA(launch_raycast((const RayJob*)ws, n, nullptr, n * tiles, rgba != nullptr, false, s, Schedule(),
-                           scene->view.tsdf9 != nullptr));
+                           scene_mode(scene->view)));
   return RELO_OK;
 }
 
@@ -954,10 +960,10 @@ relo_status relo_render_global(const relo_scene* const* scenes, const double* gl
   if (!ws || ((uintptr_t)ws & 255) != 0 || ws_bytes < relo_render_global_workspace_size(n_scenes))
     return fail(RELO_EINVAL, "workspace missing, misaligned or too small");
   std::vector<RayJob> jobs(n_scenes);
-  bool all_apron = true;
+  int mode = scene_mode(scenes[0] ? scenes[0]->view : SceneView{});
   for (int a = 0; a < n_scenes; ++a) {
     if (!scenes[a]) return fail(RELO_EINVAL, "null scene");
-    all_apron = all_apron && scenes[a]->view.tsdf9 != nullptr;
+    if (scene_mode(scenes[a]->view) != mode) mode = kSceneAny;
     // local camera -> scene-a pose: (gT_a)^-1 P_g, with gT_a rigid (scene a -> global)
     const double* g = global_poses + 16 * (size_t)a;
     double P[16] = {0};
@@ -976,7 +982,7 @@ relo_status relo_render_global(const relo_scene* const* scenes, const double* gl
   cudaStream_t s = (cudaStream_t)stream;
   RELO_CUDA(cudaMemcpyAsync(ws, jobs.data(), n_scenes * sizeof(RayJob), cudaMemcpyHostToDevice, s));
   RELO_CUDA(launch_render_global((const RayJob*)ws, n_scenes, intr->width, intr->height, depth, (uint32_t*)rgba,
-                                 owner, err_dev, s, all_apron));
+                                 owner, err_dev, s, mode));
   return RELO_OK;
 }
 
@@ -2053,7 +2059,7 @@ struct relo_batch {
   int32_t* d_kind = nullptr;
   int32_t* d_errs = nullptr;  // nL + nF words
   int query_tiles = 0, verify_L_tiles = 0, verify_F_tiles = 0, max_trees = 1;
-  bool query_apron = false, verify_apron = false;  // every query / verification scene has its apron copy
+  int query_mode = kSceneAny, verify_mode = kSceneAny;  // the scene_mode that all query / verification scenes share
   int64_t forest_pixels = 0;
   // learned pass
   relo_regressor* reg = nullptr;
@@ -2340,10 +2346,11 @@ void layout_batch(const relo_attempt* at, int n, const relo_ransac_params& p, ch
   b.query_tiles = qt;
   b.verify_L_tiles = vtL;
   b.verify_F_tiles = vtF;
-  b.query_apron = b.verify_apron = true;
+  b.query_mode = scene_mode(at[0].scene_b->view);
+  b.verify_mode = scene_mode(at[0].scene_a->view);
   for (int i = 0; i < n; ++i) {
-    b.query_apron = b.query_apron && h.query[i].scene.tsdf9 != nullptr;
-    b.verify_apron = b.verify_apron && at[i].scene_a->view.tsdf9 != nullptr;
+    if (scene_mode(at[i].scene_b->view) != b.query_mode) b.query_mode = kSceneAny;
+    if (scene_mode(at[i].scene_a->view) != b.verify_mode) b.verify_mode = kSceneAny;
   }
   b.forest_pixels = fpix;
   b.max_trees = maxT;
@@ -2385,7 +2392,7 @@ relo_status issue_batch(relo_batch* b, relo_pose_result* results, cudaStream_t s
   RELO_CUDA(cudaMemsetAsync(b->d_errs, 0, (b->nL + b->nF + 1) * sizeof(int32_t), s));
   RELO_CUDA(launch_init_results(b->d_res_F, b->n, s));
   RELO_CUDA(mark(b, 0, s, capturing));
-  RELO_CUDA(launch_raycast(b->d_query, b->n, nullptr, b->query_tiles, true, false, s, b->sched, b->query_apron));
+  RELO_CUDA(launch_raycast(b->d_query, b->n, nullptr, b->query_tiles, true, false, s, b->sched, b->query_mode));
   L += 2;
   RELO_CUDA(mark(b, 1, s, capturing));
   // pass L: learned attempts
@@ -2401,7 +2408,7 @@ relo_status issue_batch(relo_batch* b, relo_pose_result* results, cudaStream_t s
   if (st) return st;
   if (b->nL > 0) {
     RELO_CUDA(launch_raycast(b->d_verify_L, b->nL, nullptr, b->verify_L_tiles, false, true, s, b->sched,
-                             b->verify_apron));
+                             b->verify_mode));
     RELO_CUDA(launch_verify_decide(b->passL.d_jobs, b->nL, s));
     L += 2;
   }
@@ -2416,7 +2423,7 @@ relo_status issue_batch(relo_batch* b, relo_pose_result* results, cudaStream_t s
   if (st) return st;
   if (b->nF > 0) {
     RELO_CUDA(launch_raycast(b->d_verify_F, b->nF, nullptr, b->verify_F_tiles, false, true, s, b->sched,
-                             b->verify_apron));
+                             b->verify_mode));
     RELO_CUDA(launch_verify_decide(b->passF.d_jobs, b->nF, s));
     L += 2;
   }

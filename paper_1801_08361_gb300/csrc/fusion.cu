@@ -161,6 +161,7 @@ __global__ void __launch_bounds__(256) fuse_insert_kernel(const FuseJob j) {
         link = &j.excess[prev].w;
       }
     }
+    atomicOr(&j.cells[cell_index(x, y, z)], 1ull << cell_bit(x, y, z));
     j.visible[atomicAdd(j.n_visible, 1)] = b;
   }
 }

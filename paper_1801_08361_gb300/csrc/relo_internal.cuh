@@ -83,9 +83,27 @@ struct SceneView {
   // first voxels of the neighbouring block (+1 where that block is unallocated), so the eight
   // corners of every trilinear sample lie in the block holding the sample.
   const float* tsdf9;
-  int32_t pad[2];
+  // Scenes that grow by fusion (null otherwise): one bit per block, 64-bit words of 4 x 4 x 4 blocks
+  // indexed by the low kCellBits bits of the word's coordinates (cell_index), so that words 64 apart
+  // share one.  A clear bit says that the block is not allocated, without a walk of the hash; a set
+  // one, that it may be.
+  const unsigned long long* cells;
 };
 constexpr int kApronStride = 736;  // 729 voxels padded to a multiple of 32 floats (128 bytes)
+constexpr int kCellBits = 6;       // 64^3 words of 64 blocks, 2 MB: 10 m without sharing at 5 mm voxels
+
+__device__ __forceinline__ int cell_index(int bx, int by, int bz) {
+  constexpr int m = (1 << kCellBits) - 1;
+  return ((bx >> 2) & m) | ((by >> 2) & m) << kCellBits | ((bz >> 2) & m) << (2 * kCellBits);
+}
+__device__ __forceinline__ int cell_bit(int bx, int by, int bz) { return (bx & 3) | (by & 3) << 2 | (bz & 3) << 4; }
+
+// How a raycast launch reads its scenes: every scene through its apron copy, every scene a growing
+// one through its cell words and hash, or each by what it has (grid or hash, the blocks' own tsdf).
+enum SceneMode { kSceneAny = 0, kSceneApron = 1, kSceneCells = 2 };
+__host__ __device__ inline int scene_mode(const SceneView& s) {
+  return s.tsdf9 ? kSceneApron : (s.cells && !s.grid) ? kSceneCells : kSceneAny;
+}
 
 // Block index, or -D (see SceneView::grid), through the dense grid (caller checks s.grid).
 // Outside the box D is the Chebyshev distance to the box, a lower bound of the distance to any
@@ -442,12 +460,11 @@ inline int64_t forest_slots(int W, int H) {
   return rows > tiles ? rows : tiles;
 }
 
-// jobs_dev == nullptr: the single job is passed by value.  all_apron: every job of jobs_dev has
-// its scene's apron copy (SceneView::tsdf9), so the launch samples it (a single job's own scene
-// decides for itself).
+// jobs_dev == nullptr: the single job is passed by value.  mode: the scene_mode that all scenes of
+// jobs_dev share, or kSceneAny (a single job's own scene decides for itself).
 cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* single, int total_tiles,
                            bool with_colour, bool compare, cudaStream_t s, const Schedule& sched = Schedule(),
-                           bool all_apron = false);
+                           int mode = kSceneAny);
 // max_trees: the largest tree count among the jobs (selects the kernel's unrolled width).  With
 // sched.forest_tiles, each job must own forest_slots(W, H) slots from its pixel_begin.
 cudaError_t launch_forest(const ForestJob* jobs_dev, int n_jobs, const ForestJob* single, int64_t total_pixels,
@@ -455,7 +472,7 @@ cudaError_t launch_forest(const ForestJob* jobs_dev, int n_jobs, const ForestJob
 int ray_tiles(int W, int H);
 // Global map rendering over n scene jobs sharing one image size (owner, rgba, err_flag nullable).
 cudaError_t launch_render_global(const RayJob* jobs_dev, int n, int W, int H, uint16_t* depth, uint32_t* rgba,
-                                 int8_t* owner, int32_t* err_flag, cudaStream_t s, bool all_apron);
+                                 int8_t* owner, int32_t* err_flag, cudaStream_t s, int mode);
 cudaError_t launch_verify_decide(const RansacJob* jobs, int n_jobs, cudaStream_t s);
 cudaError_t launch_verify_decide_one(relo_pose_result* res, uint64_t omega, cudaStream_t s);
 // Learned batches: mark fallback results not run, then pick each attempt's final result.
@@ -606,6 +623,7 @@ struct FuseJob {
   int32_t* n_new;
   int32_t* n_keys;
   unsigned long long* updates;  // the scene's running count of block updates
+  unsigned long long* cells;    // SceneView::cells
 };
 cudaError_t launch_fuse_frame(const FuseJob& j, cudaStream_t s);
 cudaError_t launch_fuse_init(float* tsdf, int64_t n, cudaStream_t s);
@@ -626,6 +644,7 @@ struct relo_scene {
   int64_t capacity;
   void* d_weight;      // uint16 [capacity][512]
   void* d_coords;      // int4 [capacity]
+  void* d_cells;       // SceneView::cells
   void* d_counters;    // int32 [4]: blocks in use, excess entries in use, status, pad; then uint64 block updates
   int32_t max_weight;
   int64_t n_excess;    // excess entries allocated (the chains' storage)

@@ -17,18 +17,40 @@
 namespace relo {
 
 // ---------------------------------------------------------------------------------------------
-// Trilinear sampling with a per-thread cache of the block holding the previous sample.
+// Trilinear sampling with a per-thread cache of the block holding the previous sample (and, for
+// growing scenes, of the cell word last looked at).
 // ---------------------------------------------------------------------------------------------
+template <int kMode>
 struct BlockCache {
-  int bx, by, bz, ptr;
+  int bx = INT32_MIN, by = INT32_MIN, bz = INT32_MIN, ptr = -1;
+};
+template <>
+struct BlockCache<kSceneCells> {
+  int bx = INT32_MIN, by = INT32_MIN, bz = INT32_MIN, ptr = -1;
+  int cell = -1;
+  unsigned long long word = 0;
 };
 
-__device__ __forceinline__ int cached_block(const SceneView& s, BlockCache& c, int bx, int by, int bz, int* err) {
+// kSceneCells: a ray through free space finds most of its blocks unallocated.  The cell words answer
+// that from a register, with one load of a 2 MB array per four blocks or so, where the hash took a
+// dependent load from its buckets (and chains) for each block, and an empty word is crossed in one step
+// (cell_exit): a 640 x 480 view of a fused room takes about 190 us, 360-500 us through the hash alone.
+template <int kMode>
+__device__ __forceinline__ int cached_block(const SceneView& s, BlockCache<kMode>& c, int bx, int by, int bz, int* err) {
   if (bx != c.bx || by != c.by || bz != c.bz) {
     c.bx = bx;
     c.by = by;
     c.bz = bz;
-    c.ptr = s.grid ? grid_block(s, bx, by, bz) : lookup_block(s, bx, by, bz, err);
+    if constexpr (kMode == kSceneCells) {
+      const int cell = cell_index(bx, by, bz);
+      if (cell != c.cell) {
+        c.cell = cell;
+        c.word = __ldg(&s.cells[cell]);
+      }
+      c.ptr = (c.word >> cell_bit(bx, by, bz)) & 1 ? lookup_block(s, bx, by, bz, err) : -1;
+    } else {
+      c.ptr = s.grid ? grid_block(s, bx, by, bz) : lookup_block(s, bx, by, bz, err);
+    }
   }
   return c.ptr;
 }
@@ -62,11 +84,29 @@ __device__ __forceinline__ float cube_exit(float3 C, const RayExit& e, int bx, i
   return fminf(lx, fminf(ly, lz));
 }
 
+// Exit of the 4 x 4 x 4 blocks (an empty cell word) that hold block (bx, by, bz), or a negative value
+// where a walk of their blocks might not end on it.  The walk leaves a block through a face, steps 1e-5
+// past it and looks again: inside empty blocks whatever it does is free space, and it ends on the
+// cell's face, at the same float, unless it crosses another block face so close to that one that a
+// step's 1e-5 or rounding decides between them.  So the exit counts only where the ray, at it, is at
+// least `margin` blocks (see march_ray) from every block face but the one it leaves through.
+__device__ __forceinline__ float cell_exit(float3 C, float3 d, const RayExit& e, int bx, int by, int bz, float bs,
+                                           float inv_block, float margin) {
+  const float lx = e.zx ? INFINITY : ((float)((bx & ~3) + 4 * e.px) * bs - C.x) * e.inv.x;
+  const float ly = e.zy ? INFINITY : ((float)((by & ~3) + 4 * e.py) * bs - C.y) * e.inv.y;
+  const float lz = e.zz ? INFINITY : ((float)((bz & ~3) + 4 * e.pz) * bs - C.z) * e.inv.z;
+  const float l = fminf(lx, fminf(ly, lz));
+  const float x = fmaf(l, d.x, C.x) * inv_block, y = fmaf(l, d.y, C.y) * inv_block, z = fmaf(l, d.z, C.z) * inv_block;
+  const int near = (fabsf(x - rintf(x)) <= margin) + (fabsf(y - rintf(y)) <= margin) + (fabsf(z - rintf(z)) <= margin);
+  return near <= 1 ? l : -1.0f;  // (one: the face it leaves through)
+}
+
 // Blocks holding the 8 corners of the voxel cell at (i, j, k) (corner n = (i + (n & 1),
 // j + (n >> 1 & 1), k + (n >> 2))), given b0 = the block of (i, j, k): a corner leaves b0 only
 // along the axes where the cell sits on b0's last voxel, so at most 7 further lookups, usually 0
 // or 1 (instead of one per corner through a one-entry cache that neighbouring corners evict).
-__device__ __forceinline__ void corner_blocks(const SceneView& s, BlockCache& c, int b0, int i, int j, int k,
+template <int kMode>
+__device__ __forceinline__ void corner_blocks(const SceneView& s, BlockCache<kMode>& c, int b0, int i, int j, int k,
                                               int (&blk)[8], int* err) {
   const int bx = i >> 3, by = j >> 3, bz = k >> 3;
   const bool ex = (i & 7) == 7, ey = (j & 7) == 7, ez = (k & 7) == 7;
@@ -93,15 +133,15 @@ __device__ __forceinline__ int corner_voxel(int i, int j, int k, int n) {
 }
 
 // Trilinear tsdf at voxel-space point q (= p / voxel), given the block b0 holding floor(q);
-// corners in unallocated blocks read +1.  kApron: from the scene's apron copy (s.tsdf9, which
+// corners in unallocated blocks read +1.  kSceneApron: from the scene's apron copy (s.tsdf9, which
 // every job of the launch has), where all eight corners lie in block b0 and hold the values the
 // neighbour lookups below would read; otherwise from the blocks' own tsdf.
-template <bool kApron>
-__device__ __forceinline__ float trilinear_tsdf(const SceneView& s, BlockCache& c, int b0, int i, int j, int k,
+template <int kMode>
+__device__ __forceinline__ float trilinear_tsdf(const SceneView& s, BlockCache<kMode>& c, int b0, int i, int j, int k,
                                                 float fx, float fy, float fz, int* err) {
   float v[8];
   if (!RELO_CHECK(b0 < s.n_blocks)) return 1.0f;
-  if (kApron) {
+  if (kMode == kSceneApron) {
     const float* base = s.tsdf9 + (size_t)b0 * kApronStride + (i & 7) + 9 * (j & 7) + 81 * (k & 7);
     v[0] = __ldg(base);
     v[1] = __ldg(base + 1);
@@ -141,7 +181,8 @@ __device__ __forceinline__ float trilinear_tsdf(const SceneView& s, BlockCache& 
 }
 
 // Trilinear colour at point p (corners in unallocated blocks read 0), rounded half up.
-__device__ __forceinline__ uint32_t trilinear_rgba(const SceneView& s, BlockCache& c, float3 p, int* err) {
+template <int kMode>
+__device__ __forceinline__ uint32_t trilinear_rgba(const SceneView& s, BlockCache<kMode>& c, float3 p, int* err) {
   const float qx = p.x * s.inv_voxel, qy = p.y * s.inv_voxel, qz = p.z * s.inv_voxel;
   const float flx = floorf(qx), fly = floorf(qy), flz = floorf(qz);
   const int i = (int)flx, j = (int)fly, k = (int)flz;
@@ -167,12 +208,17 @@ __device__ __forceinline__ uint32_t trilinear_rgba(const SceneView& s, BlockCach
 }
 
 // One ray.  Returns the hit depth parameter (camera z, metres) or a negative value if none.
-template <bool kApron>
-__device__ __forceinline__ float march_ray(const SceneView& s, float3 C, float3 d, float dmin, float dmax, BlockCache& c,
-                                           int* err) {
+template <int kMode>
+__device__ __forceinline__ float march_ray(const SceneView& s, float3 C, float3 d, float dmin, float dmax,
+                                           BlockCache<kMode>& c, int* err) {
   const float dn = sqrtf(d.x * d.x + d.y * d.y + d.z * d.z);
   const float inv_dn = 1.0f / dn;
   const RayExit rx = ray_exit(d);
+  // kSceneCells: four of the walk's steps past a face, and the rounding of the ray's points (a few units
+  // in the last place of the largest coordinate it can reach), in blocks
+  const float inv_block = s.inv_voxel * 0.125f;
+  const float reach = fmaxf(fabsf(C.x), fmaxf(fabsf(C.y), fabsf(C.z))) + dmax * dn;
+  const float margin = (4e-5f * dn + 1e-6f * reach) * inv_block;
   float lam = dmin, lam_prev = 0.f, f_prev = 0.f;
   bool have_prev = false;
   for (int it = 0; it < kMaxMarchSamples && lam <= dmax; ++it) {
@@ -187,14 +233,18 @@ __device__ __forceinline__ float march_ray(const SceneView& s, float3 C, float3 
       // around it that holds no allocated block (-b = its Chebyshev distance to one, so the
       // cube's half-size is -b - 1 blocks): stepping block by block through that cube ends on
       // the same exit plane, so the skip changes no sample the march evaluates
-      const float lexit = cube_exit(C, rx, bx, by, bz, -b, s.block_size);
+      float lexit = -1.0f;
+      if constexpr (kMode == kSceneCells) {
+        if (c.word == 0) lexit = cell_exit(C, d, rx, bx, by, bz, s.block_size, inv_block, margin);
+      }
+      if (lexit < 0.0f) lexit = cube_exit(C, rx, bx, by, bz, kMode == kSceneCells ? 1 : -b, s.block_size);
       lam_prev = fmaxf(lexit, lam);
       f_prev = 1.0f;
       have_prev = true;
       lam = lam_prev + 1e-5f;
       continue;
     }
-    const float f = trilinear_tsdf<kApron>(s, c, b, i, j, k, qx - flx, qy - fly, qz - flz, err);
+    const float f = trilinear_tsdf<kMode>(s, c, b, i, j, k, qx - flx, qy - fly, qz - flz, err);
     if (f <= 0.0f) {
       if (!have_prev) return -1.0f;
       return lam_prev + (lam - lam_prev) * f_prev / (f_prev - f);
@@ -210,7 +260,8 @@ __device__ __forceinline__ float march_ray(const SceneView& s, float3 C, float3 
 constexpr int kTile = 16;
 // CTAs per SM the compiler must fit, depth-only and colour renders: the march is latency-bound,
 // so occupancy beats the few registers this spills.  On the house batch: depth-only 12.08 / 11.94
-// / 12.99 ms at 5 / 6 / 7, colour 13.53 / 12.86 / 12.40 / 12.57 ms at 4 / 5 / 6 / 7
+// / 12.99 ms at 5 / 6 / 7, colour 13.53 / 12.86 / 12.40 / 12.57 ms at 4 / 5 / 6 / 7.  Growing scenes
+// (eight frames fused and viewed): 1.97 / 1.93 / 2.06 / 2.24 ms at 4 / 5 / 6 / 8
 #ifndef RELO_RAYCAST_MIN_BLOCKS
 #define RELO_RAYCAST_MIN_BLOCKS 6
 #endif
@@ -218,8 +269,8 @@ constexpr int kTile = 16;
 #define RELO_RAYCAST_COLOUR_MIN_BLOCKS 6
 #endif
 
-template <bool kColour, bool kCompare, bool kApron>
-__global__ void __launch_bounds__(kTile* kTile, kColour ? RELO_RAYCAST_COLOUR_MIN_BLOCKS : RELO_RAYCAST_MIN_BLOCKS)
+template <bool kColour, bool kCompare, int kMode>
+__global__ void __launch_bounds__(kTile* kTile, kMode == kSceneCells ? 5 : kColour ? RELO_RAYCAST_COLOUR_MIN_BLOCKS : RELO_RAYCAST_MIN_BLOCKS)
     raycast_kernel(const RayJob* __restrict__ jobs, int n_jobs, const RayJob single, int warp_log2w) {
   // locate the job owning this tile (jobs are few; binary search on tile_begin)
   int lo = 0, hi = n_jobs - 1;
@@ -279,8 +330,8 @@ __global__ void __launch_bounds__(kTile* kTile, kColour ? RELO_RAYCAST_COLOUR_MI
     const float3 d = make_float3(R[0] * dcx + R[1] * dcy + R[2], R[3] * dcx + R[4] * dcy + R[5],
                                  R[6] * dcx + R[7] * dcy + R[8]);
     const float3 C = make_float3(t[0], t[1], t[2]);
-    BlockCache cache{INT32_MIN, INT32_MIN, INT32_MIN, -1};
-    const float lam = march_ray<kApron>(job.scene, C, d, job.dmin, job.dmax, cache, &err);
+    BlockCache<kMode> cache;
+    const float lam = march_ray<kMode>(job.scene, C, d, job.dmin, job.dmax, cache, &err);
     const size_t pix = (size_t)v * job.W + u;
     uint32_t col = 0u;
     if (lam >= job.dmin && lam <= job.dmax) {
@@ -333,25 +384,27 @@ __global__ void __launch_bounds__(kTile* kTile, kColour ? RELO_RAYCAST_COLOUR_MI
   }
 }
 
-template <bool kApron>
+template <int kMode>
 void launch_raycast_t(const RayJob* jobs_dev, int n_jobs, const RayJob& one, int total_tiles, bool with_colour,
                       bool compare, cudaStream_t s, int w) {
   const dim3 grid(total_tiles), block(kTile * kTile);
-  if (compare) raycast_kernel<false, true, kApron><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
-  else if (with_colour) raycast_kernel<true, false, kApron><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
-  else raycast_kernel<false, false, kApron><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
+  if (compare) raycast_kernel<false, true, kMode><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
+  else if (with_colour) raycast_kernel<true, false, kMode><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
+  else raycast_kernel<false, false, kMode><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
 }
 
 cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* single, int total_tiles,
-                           bool with_colour, bool compare, cudaStream_t s, const Schedule& sched, bool all_apron) {
+                           bool with_colour, bool compare, cudaStream_t s, const Schedule& sched, int mode) {
   if (total_tiles <= 0) return cudaSuccess;
   if (sched.ray_warp_log2w < 1 || sched.ray_warp_log2w > 4) return cudaErrorInvalidValue;
   RayJob one{};
   if (single) one = *single;
-  // a single job's own scene decides; a job array's scenes were checked by the caller
-  const bool apron = single ? one.scene.tsdf9 != nullptr : all_apron;
-  if (apron) launch_raycast_t<true>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, sched.ray_warp_log2w);
-  else launch_raycast_t<false>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, sched.ray_warp_log2w);
+  // a single job's own scene decides; a job array's scenes were looked over by the caller
+  if (single) mode = scene_mode(one.scene);
+  const int w = sched.ray_warp_log2w;
+  if (mode == kSceneApron) launch_raycast_t<kSceneApron>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, w);
+  else if (mode == kSceneCells) launch_raycast_t<kSceneCells>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, w);
+  else launch_raycast_t<kSceneAny>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, w);
   return cudaGetLastError();
 }
 
@@ -361,7 +414,7 @@ cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* sin
 // stops past the depth it would have to beat: any hit nearer than best + 1 mm is detected by a
 // sample at most one march step (<= mu) beyond it, so the cut changes no winner.
 // ---------------------------------------------------------------------------------------------
-template <bool kApron>
+template <int kMode>
 __global__ void __launch_bounds__(kTile* kTile)
     render_global_kernel(const RayJob* __restrict__ jobs, int n, uint16_t* __restrict__ depth,
                          uint32_t* __restrict__ rgba, int8_t* __restrict__ owner, int32_t* __restrict__ err_flag) {
@@ -387,8 +440,8 @@ __global__ void __launch_bounds__(kTile* kTile)
                                  j.R[6] * dcx + j.R[7] * dcy + j.R[8]);
     const float3 C = make_float3(j.t[0], j.t[1], j.t[2]);
     const float lim = best >= 0 ? fminf(j.dmax, (float)(best_mm + 1) * 0.001f + j.scene.mu + j.scene.voxel) : j.dmax;
-    BlockCache cache{INT32_MIN, INT32_MIN, INT32_MIN, -1};
-    const float lam = march_ray<kApron>(j.scene, C, d, j.dmin, lim, cache, &err);
+    BlockCache<kMode> cache;
+    const float lam = march_ray<kMode>(j.scene, C, d, j.dmin, lim, cache, &err);
     if (lam >= j.dmin && lam <= j.dmax) {
       const int mm = round_half_up_clamp(lam * 1000.0f, 1, 65535);
       if (best < 0 || mm < best_mm) {
@@ -404,7 +457,7 @@ __global__ void __launch_bounds__(kTile* kTile)
     const float dcx = ((float)u - j.cx) / j.fx, dcy = ((float)v - j.cy) / j.fy;
     const float3 d = make_float3(j.R[0] * dcx + j.R[1] * dcy + j.R[2], j.R[3] * dcx + j.R[4] * dcy + j.R[5],
                                  j.R[6] * dcx + j.R[7] * dcy + j.R[8]);
-    BlockCache cache{INT32_MIN, INT32_MIN, INT32_MIN, -1};
+    BlockCache<kMode> cache;
     col = trilinear_rgba(j.scene, cache,
                          make_float3(fmaf(best_lam, d.x, j.t[0]), fmaf(best_lam, d.y, j.t[1]), fmaf(best_lam, d.z, j.t[2])),
                          &err);
@@ -417,14 +470,17 @@ __global__ void __launch_bounds__(kTile* kTile)
 }
 
 cudaError_t launch_render_global(const RayJob* jobs_dev, int n, int W, int H, uint16_t* depth, uint32_t* rgba,
-                                 int8_t* owner, int32_t* err_flag, cudaStream_t s, bool all_apron) {
+                                 int8_t* owner, int32_t* err_flag, cudaStream_t s, int mode) {
   if (n < 1 || W < 1 || H < 1) return cudaSuccess;
   const size_t smem = (size_t)n * sizeof(RayJob);
   if (smem > 48 * 1024) return cudaErrorInvalidValue;
-  if (all_apron)
-    render_global_kernel<true><<<ray_tiles(W, H), kTile * kTile, smem, s>>>(jobs_dev, n, depth, rgba, owner, err_flag);
+  const unsigned grid = (unsigned)ray_tiles(W, H);
+  if (mode == kSceneApron)
+    render_global_kernel<kSceneApron><<<grid, kTile * kTile, smem, s>>>(jobs_dev, n, depth, rgba, owner, err_flag);
+  else if (mode == kSceneCells)
+    render_global_kernel<kSceneCells><<<grid, kTile * kTile, smem, s>>>(jobs_dev, n, depth, rgba, owner, err_flag);
   else
-    render_global_kernel<false><<<ray_tiles(W, H), kTile * kTile, smem, s>>>(jobs_dev, n, depth, rgba, owner, err_flag);
+    render_global_kernel<kSceneAny><<<grid, kTile * kTile, smem, s>>>(jobs_dev, n, depth, rgba, owner, err_flag);
   return cudaGetLastError();
 }
 
