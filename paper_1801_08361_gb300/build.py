@@ -22,7 +22,7 @@ NVCC_FLAGS = ARCH + ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-
 # occupancy bounds of the raycast, forest and hypothesis-search kernels (tuning knobs; the defaults come from sweeps)
 NVCC_FLAGS += [f"-D{k}={os.environ[k]}" for k in ("RELO_RAYCAST_MIN_BLOCKS", "RELO_RAYCAST_COLOUR_MIN_BLOCKS",
                                                   "RELO_SEARCH_MIN_BLOCKS", "RELO_FOREST_MIN_BLOCKS",
-                                                  "RELO_REFINE_MIN_BLOCKS", "RELO_GROUP_SOLVES",
+                                                  "RELO_REFINE_MIN_BLOCKS", "RELO_GROUP_SOLVES", "RELO_SEARCH_SHARED", "RELO_SEARCH_WIDE",
                                                   "RELO_REFINE_FEW_MIN_BLOCKS", "RELO_ENERGY_MIN_BLOCKS")
                if k in os.environ]
 

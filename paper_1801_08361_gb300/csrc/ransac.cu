@@ -239,45 +239,66 @@ __global__ void __launch_bounds__(kCompactThreads) compact_scatter_kernel(const 
   const int n_chunks = (n_pix + kCompactChunk - 1) / kCompactChunk;
   const int T = job.forest.T, nv = job.nv;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  constexpr int kWarps = kCompactThreads / 32;
   __shared__ int s_off;
-  __shared__ int s_warp[kCompactThreads / 32];
-  if (threadIdx.x < 32) {
-    int s = 0;
-    for (int c = threadIdx.x; c < chunk; c += 32) s += job.chunk_count[c];
-    s = warp_sum_i(s);
-    if (threadIdx.x == 0) s_off = s;
-  }
-  __syncthreads();
-  int off = s_off;
+  __shared__ int s_count[kIters * kWarps];  // valid pixels per 32, in raster order; then those before them
+  // All of the chunk's depths at once, and two barriers in all: with a barrier pair per 256 pixels a
+  // chunk was 16 dependent rounds (38 us for a lone 640 x 480 view).
+  int d[kIters];
+#pragma unroll
   for (int it = 0; it < kIters; ++it) {
     const int p = chunk * kCompactChunk + it * kCompactThreads + threadIdx.x;
-    const int d = p < n_pix ? job.depth[p] : 0;
-    const unsigned ball = __ballot_sync(0xffffffffu, d > 0);
-    if (lane == 0) s_warp[warp] = __popc(ball);
-    __syncthreads();
-    int before = 0, total = 0;
-    for (int w = 0; w < kCompactThreads / 32; ++w) {
-      const int c = s_warp[w];
-      before += (w < warp) ? c : 0;
-      total += c;
-    }
-    if (d > 0) {
-      const int pos = off + before + __popc(ball & ((1u << lane) - 1u));
-      uint16_t f[24];
-      f[0] = (uint16_t)(p % job.W);
-      f[1] = (uint16_t)(p / job.W);
-      f[2] = (uint16_t)d;
-      for (int t = 0; t < T; ++t) f[3 + t] = job.leaves[(size_t)t * n_pix + p];
-      for (int k = 3 + T; k < 8 * nv; ++k) f[k] = 0;
-      uint4* dst = job.table + (size_t)pos * nv;
-      for (int q = 0; q < nv; ++q)
-        dst[q] = make_uint4(f[8 * q] | ((uint32_t)f[8 * q + 1] << 16), f[8 * q + 2] | ((uint32_t)f[8 * q + 3] << 16),
-                            f[8 * q + 4] | ((uint32_t)f[8 * q + 5] << 16), f[8 * q + 6] | ((uint32_t)f[8 * q + 7] << 16));
-    }
-    off += total;
-    __syncthreads();
+    d[it] = p < n_pix ? job.depth[p] : 0;
   }
-  if (chunk == n_chunks - 1 && threadIdx.x == 0) *job.n_valid = off;
+  if (warp == 0) {
+    int s = 0;
+    for (int c = lane; c < chunk; c += 32) s += job.chunk_count[c];
+    s = warp_sum_i(s);
+    if (lane == 0) s_off = s;
+  }
+  unsigned ball[kIters];
+#pragma unroll
+  for (int it = 0; it < kIters; ++it) {
+    ball[it] = __ballot_sync(0xffffffffu, d[it] > 0);
+    if (lane == 0) s_count[it * kWarps + warp] = __popc(ball[it]);
+  }
+  __syncthreads();
+  if (warp == 0) {
+    constexpr int kPer = kIters * kWarps / 32;
+    int c[kPer], sum = 0;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) sum += c[k] = s_count[lane * kPer + k];
+    int before = sum;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, before, o);
+      if (lane >= o) before += y;
+    }
+    int at = s_off + before - sum;
+#pragma unroll
+    for (int k = 0; k < kPer; ++k) {
+      s_count[lane * kPer + k] = at;
+      at += c[k];
+    }
+    if (chunk == n_chunks - 1 && lane == 31) *job.n_valid = at;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int it = 0; it < kIters; ++it) {
+    if (d[it] == 0) continue;
+    const int p = chunk * kCompactChunk + it * kCompactThreads + threadIdx.x;
+    const int pos = s_count[it * kWarps + warp] + __popc(ball[it] & ((1u << lane) - 1u));
+    // fields u, v, depth, leaf[T], packed two to a word and eight to an entry
+    uint4* dst = job.table + (size_t)pos * nv;
+    const uint16_t* leaves = job.leaves + p;
+    auto field = [&](int k) -> uint32_t {
+      return k == 0 ? (uint32_t)(p % job.W) : k == 1 ? (uint32_t)(p / job.W) : k == 2 ? (uint32_t)d[it]
+             : k < 3 + T ? (uint32_t)leaves[(size_t)(k - 3) * n_pix] : 0u;
+    };
+    for (int q = 0; q < nv; ++q)
+      dst[q] = make_uint4(field(8 * q) | field(8 * q + 1) << 16, field(8 * q + 2) | field(8 * q + 3) << 16,
+                          field(8 * q + 4) | field(8 * q + 5) << 16, field(8 * q + 6) | field(8 * q + 7) << 16);
+  }
 }
 
 cudaError_t launch_compact(const RansacJob* jobs, int n_jobs, int total_chunks, cudaStream_t s) {
@@ -441,9 +462,13 @@ __device__ __forceinline__ int try_status(const RansacJob& job, const TryDraw& d
   return ambiguous ? 2 : 1;
 }
 
-// One warp per hypothesis (four per CTA, no block-wide barriers): each step evaluates 64 tries,
-// two per lane (tries base + lane and base + 32 + lane, whose loads are issued together), and
-// keeps the first one not failing in try order, settling guard-band tries in FP64 in order.
+// Each warp step evaluates 64 tries, two per lane (tries base + lane and base + 32 + lane, whose loads
+// are issued together), and keeps the first one not failing in try order, settling guard-band tries in
+// FP64 in order.  What bounds it is the L1: a gather takes about one cycle per lane, four a try (84 % of
+// the data pipe's peak over a batch).  Tried and slower: queueing the tries that pass their first pair
+// for a dense second stage (house batch 19.2 -> 21.3 ms with the fits and compaction), and testing first
+// pairs from 16-bit position codes in the table, two gathers a try, with such a queue for the one in six
+// that those let through (18.2 ms at best, its second stage a chain of six dependent loads).
 constexpr int kSearchWarps = 4;
 
 // first try of mask (bits = lanes) that passes, settling guard-band statuses in FP64; -1 if none
@@ -470,48 +495,66 @@ __device__ __forceinline__ int first_passing(const RansacJob& job, int h, int n_
 #ifndef RELO_SEARCH_MIN_BLOCKS
 #define RELO_SEARCH_MIN_BLOCKS 5
 #endif
-// The search of hypothesis gw (flattened over the jobs) by one warp.
-__device__ __forceinline__ int search_one(const RansacJob* __restrict__ jobs, int n_jobs, int gw, int lane) {
+__device__ __forceinline__ int hypothesis_job(const RansacJob* __restrict__ jobs, int n_jobs, int gid) {
   int lo = 0, hi = n_jobs - 1;
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].hyp_begin <= gw) lo = mid;
+    if (jobs[mid].hyp_begin <= gid) lo = mid;
     else hi = mid - 1;
   }
-  const RansacJob& job = jobs[lo];
-  const int h = gw - job.hyp_begin;
-  if (h >= job.K || job_skipped(job.skip)) return lo;
+  return lo;
+}
+
+// First passing try of hypothesis h among those of warp `part` of `parts` (steps of 64 tries in turn);
+// INT_MAX if none.  *found (shared by the parts, null for one): the lowest passing try so far, beyond
+// which no part needs to look.
+__device__ __forceinline__ int search_part(const RansacJob& job, int h, int lane, int part, int parts,
+                                           volatile int* found) {
   const int n_valid = *job.n_valid;
+  if (n_valid <= 0) return INT_MAX;
   const float rig = (float)job.rigidity, area = (float)job.min_area;
   // the area test |cross| >= area with its guard band, on squares (both sides non-negative)
   const float area_lo = fmaxf(area - kGuardArea, 0.f), area_hi = area + kGuardArea;
   const float area_lo2 = area_lo * area_lo, area_hi2 = area_hi * area_hi;
   const float ifx = (float)(1.0 / job.fx), ify = (float)(1.0 / job.fy), cx = (float)job.cx, cy = (float)job.cy;
   const int L = 1 << job.forest.D;
-  int found = INT_MAX;
-  if (n_valid > 0) {
-    for (int base = 0; base < job.max_tries && found == INT_MAX; base += 64) {
-      const int ja = base + lane, jb = base + 32 + lane;
-      const TryDraw da = draw_indices(job, h, ja, n_valid), db = draw_indices(job, h, jb, n_valid);
-      const TryPair pa = load_pair(job, da, L), pb = load_pair(job, db, L);
-      const int sa = ja < job.max_tries ? try_status(job, da, pa, L, rig, area_lo2, area_hi2, ifx, ify, cx, cy) : 0;
-      const int sb = jb < job.max_tries ? try_status(job, db, pb, L, rig, area_lo2, area_hi2, ifx, ify, cx, cy) : 0;
-      int w = first_passing(job, h, n_valid, __ballot_sync(0xffffffffu, sa != 0), sa, ja, lane);
-      if (w >= 0) {
-        found = base + w;
-        break;
-      }
-      w = first_passing(job, h, n_valid, __ballot_sync(0xffffffffu, sb != 0), sb, jb, lane);
-      if (w >= 0) found = base + 32 + w;
-    }
+  for (int base = part * 64; base < job.max_tries; base += 64 * parts) {
+    if (found && __shfl_sync(0xffffffffu, *found, 0) < base) break;
+    const int ja = base + lane, jb = base + 32 + lane;
+    const TryDraw da = draw_indices(job, h, ja, n_valid), db = draw_indices(job, h, jb, n_valid);
+    const TryPair pa = load_pair(job, da, L), pb = load_pair(job, db, L);
+    const int sa = ja < job.max_tries ? try_status(job, da, pa, L, rig, area_lo2, area_hi2, ifx, ify, cx, cy) : 0;
+    const int sb = jb < job.max_tries ? try_status(job, db, pb, L, rig, area_lo2, area_hi2, ifx, ify, cx, cy) : 0;
+    int w = first_passing(job, h, n_valid, __ballot_sync(0xffffffffu, sa != 0), sa, ja, lane);
+    if (w >= 0) return base + w;
+    w = first_passing(job, h, n_valid, __ballot_sync(0xffffffffu, sb != 0), sb, jb, lane);
+    if (w >= 0) return base + 32 + w;
   }
-  if (lane == 0) {
-    job.hyp_ok[h] = found != INT_MAX;
-    job.tries[h] = found != INT_MAX ? found : job.max_tries;
-  }
-  return lo;
+  return INT_MAX;
 }
 
+__device__ __forceinline__ void store_search(const RansacJob& job, int h, int found) {
+  job.hyp_ok[h] = found != INT_MAX;
+  job.tries[h] = found != INT_MAX ? found : job.max_tries;
+}
+
+// The search of hypothesis gw (flattened over the jobs) by one warp.
+__device__ __forceinline__ int search_one(const RansacJob* __restrict__ jobs, int n_jobs, int gw, int lane) {
+  const int jid = hypothesis_job(jobs, n_jobs, gw);
+  const RansacJob& job = jobs[jid];
+  const int h = gw - job.hyp_begin;
+  if (h >= job.K || job_skipped(job.skip)) return jid;
+  const int found = search_part(job, h, lane, 0, 1, nullptr);
+  if (lane == 0) store_search(job, h, found);
+  return jid;
+}
+
+#ifndef RELO_SEARCH_WIDE
+#define RELO_SEARCH_WIDE 3
+#endif
+#ifndef RELO_SEARCH_SHARED
+#define RELO_SEARCH_SHARED 3
+#endif
 // Persistent: hypotheses need from one try to max_tries, so each warp takes its next hypothesis
 // from a counter when it finishes one (which warp computes a hypothesis does not change its result).
 __global__ void __launch_bounds__(kSearchWarps * 32, RELO_SEARCH_MIN_BLOCKS)
@@ -523,6 +566,35 @@ __global__ void __launch_bounds__(kSearchWarps * 32, RELO_SEARCH_MIN_BLOCKS)
     gw = __shfl_sync(0xffffffffu, gw, 0);
     if (gw >= total) return;
     search_one(jobs, n_jobs, gw, lane);
+  }
+}
+
+// Few hypotheses: the warps of a CTA share one, each taking every kWarps-th step (a hypothesis that uses
+// up its 10 000 tries is a chain of 157 dependent steps for one warp, which set the time of a lone
+// attempt: 247 us of a house frame's search, 242 of a room's).
+template <int kWarps>
+__global__ void __launch_bounds__(kWarps * 32, RELO_SEARCH_MIN_BLOCKS * kSearchWarps / kWarps)
+    search_shared_kernel(const RansacJob* __restrict__ jobs, int n_jobs, int total, int32_t* __restrict__ counter) {
+  __shared__ int s_found, s_next;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  for (;;) {
+    if (threadIdx.x == 0) {
+      s_next = atomicAdd(counter, 1);
+      s_found = INT_MAX;
+    }
+    __syncthreads();
+    const int gw = s_next;
+    if (gw >= total) return;
+    const RansacJob& job = jobs[hypothesis_job(jobs, n_jobs, gw)];
+    const int h = gw - job.hyp_begin;
+    const bool mine = h < job.K && !job_skipped(job.skip);
+    if (mine) {
+      const int r = search_part(job, h, lane, warp, kWarps, &s_found);
+      if (lane == 0 && r != INT_MAX) atomicMin(&s_found, r);
+    }
+    __syncthreads();
+    if (mine && threadIdx.x == 0) store_search(job, h, s_found);
+    __syncthreads();
   }
 }
 
@@ -630,16 +702,6 @@ __device__ __forceinline__ void fit_group(const RansacJob& job, int h) {
   }
 }
 
-__device__ __forceinline__ int hypothesis_job(const RansacJob* __restrict__ jobs, int n_jobs, int gid) {
-  int lo = 0, hi = n_jobs - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].hyp_begin <= gid) lo = mid;
-    else hi = mid - 1;
-  }
-  return lo;
-}
-
 // The kept tries' poses, and the draws of every round (both need only the table and the search's
 // result, and a round's draws are the same whoever is alive): CTAs below fit_blocks take the fits,
 // draw_blocks CTAs per job after them the job's drawn pixels.  kGroup: two hypotheses per warp
@@ -689,8 +751,16 @@ cudaError_t launch_hypotheses(const RansacJob* jobs, int n_jobs, int total_hyps,
   const int ctas = sched.search_ctas_per_sm == 0 ? per_sm : std::min(per_sm, sched.search_ctas_per_sm);
   e = cudaMemsetAsync(counter, 0, sizeof(int32_t), s);
   if (e != cudaSuccess) return e;
-  const int grid = std::min(sms * ctas, (total_hyps + kSearchWarps - 1) / kSearchWarps);
-  search_kernel<<<grid, kSearchWarps * 32, 0, s>>>(jobs, n_jobs, total_hyps, counter);
+  // warps resident at once against the hypotheses: share each hypothesis among 16 or 4 warps while
+  // that keeps to about one and a half rounds of them
+  const int slots = sms * ctas * kSearchWarps;
+  if (total_hyps * 16 <= RELO_SEARCH_WIDE * slots / 2)
+    search_shared_kernel<16><<<std::min(total_hyps, std::max(1, slots / 16)), 512, 0, s>>>(jobs, n_jobs, total_hyps, counter);
+  else if (total_hyps * 4 <= RELO_SEARCH_SHARED * slots / 2)
+    search_shared_kernel<4><<<std::min(total_hyps, std::max(1, slots / 4)), 128, 0, s>>>(jobs, n_jobs, total_hyps, counter);
+  else
+    search_kernel<<<std::min(sms * ctas, (total_hyps + kSearchWarps - 1) / kSearchWarps), kSearchWarps * 32, 0, s>>>(
+        jobs, n_jobs, total_hyps, counter);
   const bool group = total_hyps <= kGroupSolves;
   const int per_block = group ? kSolvesPerWarp * kFitThreads / 32 : kFitThreads;
   const int fit_blocks = (total_hyps + per_block - 1) / per_block, draw_blocks = (max_draws + kFitThreads - 1) / kFitThreads;
@@ -983,17 +1053,66 @@ __device__ __forceinline__ unsigned long long order_key(double e) {
   return (b >> 63) ? ~b : (b | 0x8000000000000000ull);
 }
 
-// Halving: CTA per job, bitonic sort of (energy key, index) ascending; keep ceil(n/2).
+// Whether (ka, ia) sorts after (kb, ib).
+__device__ __forceinline__ bool sorts_after(unsigned long long ka, int ia, unsigned long long kb, int ib) {
+  return ka > kb || (ka == kb && ia > ib);
+}
+
+// Halving: CTA per job, bitonic sort of (energy key, index) ascending; keep ceil(n/2).  Up to one
+// hypothesis per thread the pairs stay in registers: the network's strides below 32 are shuffles, and
+// only the larger ones (15 of the 55 steps at 1024) go through shared memory with barriers.
 __device__ __forceinline__ void select_block(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ alive_prefix,
                                              int r, int jid, unsigned long long* skey) {
   const int n = alive_prefix[jid + 1] - alive_prefix[jid];
   if (n == 0) return;
   const RansacJob& job = jobs[jid];
   if (job_skipped(job.skip)) return;
-  int npow = 1;
+  int npow = 32;
   while (npow < n) npow <<= 1;
   int* sidx = reinterpret_cast<int*>(skey + npow);
   const int32_t* in = alive_in(job, r);
+  const int keep = (n + 1) / 2;
+  int32_t* out = alive_out(job, r);
+  if (npow <= (int)blockDim.x) {
+    const int i = threadIdx.x;
+    const bool on = i < npow;  // whole warps: npow is a multiple of 32
+    unsigned long long key = ~0ull;
+    int idx = INT_MAX;
+    if (i < n) {
+      idx = in[i];
+      key = order_key(job.energy[idx]);
+    }
+    for (int k = 2; k <= npow; k <<= 1) {
+      for (int jj = k >> 1; jj > 0; jj >>= 1) {
+        unsigned long long ok = 0;
+        int oi = 0;
+        if (jj >= 32) {
+          __syncthreads();  // the step before has read
+          if (on) {
+            skey[i] = key;
+            sidx[i] = idx;
+          }
+          __syncthreads();
+          if (on) {
+            ok = skey[i ^ jj];
+            oi = sidx[i ^ jj];
+          }
+        } else if (on) {
+          ok = __shfl_xor_sync(0xffffffffu, key, jj);
+          oi = __shfl_xor_sync(0xffffffffu, idx, jj);
+        }
+        // the lower of the two places keeps the smaller pair in an ascending run, the larger in a descending one
+        const bool lower = (i & jj) == 0, up = (i & k) == 0;
+        const bool after = sorts_after(key, idx, ok, oi);
+        if (on && after == (lower == up)) {
+          key = ok;
+          idx = oi;
+        }
+      }
+    }
+    if (i < keep) out[i] = idx;
+    return;
+  }
   for (int i = threadIdx.x; i < npow; i += blockDim.x) {
     if (i < n) {
       const int h = in[i];
@@ -1011,7 +1130,7 @@ __device__ __forceinline__ void select_block(const RansacJob* __restrict__ jobs,
         const int l = i ^ jj;
         if (l > i) {
           const bool up = (i & k) == 0;
-          const bool gt = skey[i] > skey[l] || (skey[i] == skey[l] && sidx[i] > sidx[l]);
+          const bool gt = sorts_after(skey[i], sidx[i], skey[l], sidx[l]);
           if (gt == up) {
             const unsigned long long tk = skey[i];
             skey[i] = skey[l];
@@ -1025,8 +1144,6 @@ __device__ __forceinline__ void select_block(const RansacJob* __restrict__ jobs,
       __syncthreads();
     }
   }
-  const int keep = (n + 1) / 2;
-  int32_t* out = alive_out(job, r);
   for (int i = threadIdx.x; i < keep; i += blockDim.x) out[i] = sidx[i];
 }
 
@@ -1296,9 +1413,10 @@ cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int
   energy_kernel<<<dim3((max_alive + 31) / 32, n_jobs, n_split), kRoundWarps * 32, 0, s>>>(jobs, alive_prefix_dev, round);
   if (n_split > 1)
     sum_scores_kernel<<<dim3((max_alive * 8 + 255) / 256, n_jobs), 256, 0, s>>>(jobs, alive_prefix_dev, round, n_split);
-  // the largest alive set (4096) bounds the shared memory of the sort
-  select_kernel<<<n_jobs, 1024, 4096 * (sizeof(unsigned long long) + sizeof(int)), s>>>(jobs, alive_prefix_dev,
-                                                                                        round);
+  int npow = 32;
+  while (npow < max_alive) npow <<= 1;
+  select_kernel<<<n_jobs, std::min(npow, 1024), (size_t)npow * (sizeof(unsigned long long) + sizeof(int)), s>>>(
+      jobs, alive_prefix_dev, round);
   const int parts = ((round + 1) * B + kRefinePixels - 1) / kRefinePixels;
   switch (group_log2(max_surv)) {
     case 0: launch_refine<0>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
