@@ -567,8 +567,8 @@ typedef struct relo_schedule {
   int32_t ray_warp_width;     /* raycasts: each warp covers ray_warp_width x (32 / width) pixels of
                                  its CTA's 16 x 16 tile; 2, 4, 8 or 16 */
   int32_t forest_threads;     /* forest evaluation: threads per CTA, 128 or 256 */
-  int32_t forest_tiles;       /* forest evaluation: 0 = a CTA takes consecutive row-major pixels,
-                                 1 = it takes 32 x 8 pixel tiles */
+  int32_t forest_tiles;       /* forest evaluation: a CTA takes 32 x 8 pixel tiles; 0 = each warp covers
+                                 8 x 4 pixels of one, 1 = a row of 32 */
   int32_t search_ctas_per_sm; /* hypothesis search: persistent CTAs per SM, 0 = as many as fit */
   int32_t refit_per;          /* round re-fits: survivors per one-warp CTA, 1..32; 0 = enough CTAs
                                  for twice the SM count */

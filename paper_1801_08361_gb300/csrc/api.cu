@@ -1008,38 +1008,43 @@ relo_status relo_create_forest(const void* nodes, int32_t T, int32_t D, const fl
   f->D = D;
   f->M = M;
   const size_t n_modes_bytes = (size_t)T * L, modes_bytes = (size_t)T * L * M * kModeFloats * sizeof(float);
-  if (relo::dev_malloc((void**)&f->d_nodes, (size_t)T * n_int * 16) != cudaSuccess ||
+  if (relo::dev_malloc((void**)&f->d_nodes, (size_t)T * L * 16) != cudaSuccess ||
       relo::dev_malloc((void**)&f->d_modes, modes_bytes) != cudaSuccess || relo::dev_malloc((void**)&f->d_n_modes, n_modes_bytes) != cudaSuccess ||
       relo::dev_malloc((void**)&f->d_top, (size_t)T * L * sizeof(float4)) != cudaSuccess) {
     cudaGetLastError();
     relo_destroy_forest(f);
     return fail(RELO_ENOMEM, "device allocation for the forest failed");
   }
-  // device copy of the nodes: the third word becomes {value mask (16 bits), bit offset of probe 1
-  // (8 bits), of probe 2 (8 bits)} in a packed pixel {depth | r << 16 | g << 24 | b << 32}: a depth
-  // node's mask 0xFFFF and offsets 0, a colour node's mask 0xFF and offsets 16 + 8 c1, 16 + 8 c2
-  std::vector<int4> dev_nodes((size_t)T * n_int);
-  std::memcpy(dev_nodes.data(), nodes, dev_nodes.size() * 16);
+  // device copy of the nodes (forest.cu, descend_levels): node number 1 the root, 2 n + 1 the left child
+  // of n and 2 n the right one, at [number][tree]; tau within [-65536, 65536] (the probes' difference
+  // lies within 16 bits and a sign, so no comparison changes); the third word each probe's plane in a tile
+  std::vector<int4> dev_nodes((size_t)T << D, int4{0, 0, 0, 0});
   int max_offset = 0;  // the largest |offset| of any probe: bounds how far a probe can leave its pixel
-  for (int4& nd : dev_nodes) {
-    const int kind = nd.z & 0xFF, c1 = (nd.z >> 8) & 0xFF, c2 = (nd.z >> 16) & 0xFF;
-    nd.z = kind == 0 ? 0xFFFF : (0xFF | (16 + 8 * c1) << 16 | (16 + 8 * c2) << 24);
-    for (const int w : {nd.x, nd.y}) {
+  for (size_t i = 0; i < (size_t)T * n_int; ++i)
+    for (const int w : {in_nodes[i].x, in_nodes[i].y}) {
       max_offset = std::max(max_offset, std::abs((int)(int16_t)(w & 0xFFFF)));
       max_offset = std::max(max_offset, std::abs((int)(int16_t)((uint32_t)w >> 16)));
     }
-  }
   // offsets of at most 255 in magnitude are stored times 128 (still int16), which the evaluation's
   // division by depth takes as they are (forest.cu, probe)
-  if (max_offset <= 255)
-    for (int4& nd : dev_nodes) {
-      int* w[2] = {&nd.x, &nd.y};
-      for (int* p : w) {
-        const int lo = (int)(int16_t)(*p & 0xFFFF) * 128, hi = (int)(int16_t)((uint32_t)*p >> 16) * 128;
-        *p = (int)((uint32_t)(uint16_t)(int16_t)lo | (uint32_t)(uint16_t)(int16_t)hi << 16);
+  const int scale = max_offset <= 255 ? 128 : 1;
+  for (int t = 0; t < T; ++t)
+    for (int level = 0; level < D; ++level)
+      for (size_t p = 0; p < (size_t)1 << level; ++p) {
+        const size_t first = (size_t)1 << level;  // nodes above this level, and in it
+        int4 nd = in_nodes[(size_t)t * n_int + first - 1 + p];
+        const int kind = nd.z & 0xFF, c1 = (nd.z >> 8) & 0xFF, c2 = (nd.z >> 16) & 0xFF;
+        // planes 128 (1 + c); channel 3 reads plane b of a tiled image and is marked by bit 0
+        auto plane = [](int c) { return c == 3 ? 0x181 : 128 * (1 + c); };
+        nd.z = kind == 0 ? 0 : plane(c1) | plane(c2) << 16;
+        nd.w = std::min(std::max(nd.w, -65536), 65536);
+        for (int* w : {&nd.x, &nd.y}) {
+          const int lo = (int)(int16_t)(*w & 0xFFFF) * scale, hi = (int)(int16_t)((uint32_t)*w >> 16) * scale;
+          *w = (int)((uint32_t)(uint16_t)(int16_t)lo | (uint32_t)(uint16_t)(int16_t)hi << 16);
+        }
+        dev_nodes[(first | (first - 1 - p)) * T + t] = nd;
       }
-    }
-  cudaError_t e = cudaMemcpy(f->d_nodes, dev_nodes.data(), (size_t)T * n_int * 16, cudaMemcpyHostToDevice);
+  cudaError_t e = cudaMemcpy(f->d_nodes, dev_nodes.data(), dev_nodes.size() * 16, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = modes ? cudaMemcpy(f->d_modes, modes, modes_bytes, cudaMemcpyHostToDevice)
                                   : cudaMemset(f->d_modes, 0, modes_bytes);
   if (e == cudaSuccess) e = n_modes ? cudaMemcpy(f->d_n_modes, n_modes, n_modes_bytes, cudaMemcpyHostToDevice)
@@ -1090,15 +1095,8 @@ relo_status relo_forest_eval(const relo_forest* f, const uint16_t* depth, const 
                              uint16_t* leaves, relo_stream stream) {
   if (!f || !depth || !rgba || !leaves) return fail(RELO_EINVAL, "null forest or buffer");
   if (bad_size(W, H)) return fail(RELO_EINVAL, "image size outside [1, 16384]");
-  ForestJob j{};
-  j.forest = f->view;
-  j.depth = depth;
-  j.rgba = (const uint32_t*)rgba;
-  j.leaves = leaves;
-  j.W = W;
-  j.H = H;
-  j.pixel_begin = 0;
-  RELO_CUDA(launch_forest(nullptr, 1, &j, (int64_t)W * H, (cudaStream_t)stream, f->T));
+  const ForestJob j = make_forest_job(f->view, depth, (const uint32_t*)rgba, leaves, W, H);
+  RELO_CUDA(launch_forest(&j, 1, (cudaStream_t)stream));
   return RELO_OK;
 }
 
@@ -1219,13 +1217,7 @@ relo_status relo_forest_train_frame(relo_forest* f, const relo_intrinsics* intr,
   }
   layout((char*)f->d_scratch);
   r.coords = coords;
-  ForestJob j{};
-  j.forest = f->view;
-  j.depth = depth;
-  j.rgba = (const uint32_t*)rgba;
-  j.leaves = leaves;
-  j.W = W;
-  j.H = H;
+  const ForestJob j = make_forest_job(f->view, depth, (const uint32_t*)rgba, leaves, W, H);
   cudaError_t e = launch_forest_grid(j, S, s);
   if (e == cudaSuccess) e = launch_scene_coords(depth, W, H, S, intr->fx, intr->fy, intr->cx, intr->cy, pose, coords, s);
   for (int t = 0; e == cudaSuccess && t < T; t += step) {
@@ -2051,16 +2043,15 @@ struct relo_batch {
   RayJob* d_query = nullptr;
   RayJob* d_verify_L = nullptr;
   RayJob* d_verify_F = nullptr;
-  ForestJob* d_forest = nullptr;
+  std::vector<ForestJob> forest;
   RansacPass passL, passF;
   relo_pose_result* d_res_L = nullptr;
   relo_pose_result* d_res_F = nullptr;
   relo_pose_result* d_res = nullptr;
   int32_t* d_kind = nullptr;
   int32_t* d_errs = nullptr;  // nL + nF words
-  int query_tiles = 0, verify_L_tiles = 0, verify_F_tiles = 0, max_trees = 1;
+  int query_tiles = 0, verify_L_tiles = 0, verify_F_tiles = 0;
   int query_mode = kSceneAny, verify_mode = kSceneAny;  // the scene_mode that all query / verification scenes share
-  int64_t forest_pixels = 0;
   // learned pass
   relo_regressor* reg = nullptr;
   int lW = 0, lH = 0;
@@ -2119,7 +2110,6 @@ relo_status check_attempts(const relo_attempt* at, int n, const relo_ransac_para
 
 struct HostJobs {
   std::vector<RayJob> query, verify_L, verify_F;
-  std::vector<ForestJob> forest;
   std::vector<RansacJob> ransac_L, ransac_F;
   std::vector<int32_t> alive_L, surv_L, alive_F, surv_F, kind;
 };
@@ -2148,7 +2138,6 @@ void layout_batch(const relo_attempt* at, int n, const relo_ransac_params& p, ch
   b.d_query = c.take<RayJob>(n);
   b.d_verify_L = c.take<RayJob>(std::max(nL, 1));
   b.d_verify_F = c.take<RayJob>(std::max(nF, 1));
-  b.d_forest = c.take<ForestJob>(std::max(nF, 1));
   b.passL.d_jobs = c.take<RansacJob>(std::max(nL, 1));
   b.passF.d_jobs = c.take<RansacJob>(std::max(nF, 1));
   b.passL.d_counter = c.take<int32_t>(1);
@@ -2233,12 +2222,11 @@ void layout_batch(const relo_attempt* at, int n, const relo_ransac_params& p, ch
   h.query.assign(n, RayJob{});
   h.verify_L.assign(nL, RayJob{});
   h.verify_F.assign(nF, RayJob{});
-  h.forest.assign(nF, ForestJob{});
+  b.forest.assign(nF, ForestJob{});
   h.ransac_L.assign(nL, RansacJob{});
   h.ransac_F.assign(nF, RansacJob{});
   h.kind.assign(kind.begin(), kind.end());
-  int qt = 0, vtL = 0, vtF = 0, chL = 0, chF = 0, hyL = 0, hyF = 0, maxT = 1;
-  int64_t fpix = 0;
+  int qt = 0, vtL = 0, vtF = 0, chL = 0, chF = 0, hyL = 0, hyF = 0, ftiles = 0;
   for (int i = 0; i < n; ++i) {
     const relo_attempt& a = at[i];
     const int W = a.intr.width, H = a.intr.height, K = a.n_hyps > 0 ? a.n_hyps : p.n_hyps;
@@ -2299,27 +2287,23 @@ void layout_batch(const relo_attempt* at, int n, const relo_ransac_params& p, ch
     if (iF[i] >= 0) {
       const int j = iF[i];
       const int T = a.forest_a->T;
-      maxT = std::max(maxT, T);
       uint16_t* leaves = c.take<uint16_t>(n_pix * T);
       b.a_leaves[i] = leaves;
-      // the query raycast also writes the image packed per pixel, which the forest reads
-      uint2* packed = c.take<uint2>(n_pix);
-      h.query[i].packed = packed;
       const int32_t* skip = kind[i] == 2 ? &b.d_res_L[i].verified : nullptr;
-      ForestJob& f = h.forest[j];
-      f.forest = a.forest_a->view;
-      f.depth = depth;
-      f.rgba = rgba;
-      f.packed = packed;
-      f.leaves = leaves;
-      f.W = W;
-      f.H = H;
-      f.pixel_begin = fpix;
+      ForestJob& f = b.forest[j];
+      f = make_forest_job(a.forest_a->view, depth, rgba, leaves, W, H);
+      f.tile_begin = ftiles;
       f.skip = skip;
-      fpix += forest_slots(W, H);  // a forest CTA never spans two jobs, in any schedule
+      ftiles += forest_job_tiles(W, H);
       RansacJob& r = h.ransac_F[j];
       fill_ransac_job(r, a.forest_a->view, depth, leaves, a.intr, p, K, a.seed);
       carve_ransac(c, r, W, H, K, p.batch, r.n_rounds, T);
+      // the query raycast also writes the image in tiles, which the forest reads; the valid-pixel table
+      // is written after the forest has run and may take its place
+      const size_t tiled = tiled_values(W, H);
+      uint16_t* image = tiled * sizeof(uint16_t) <= n_pix * r.nv * sizeof(uint4) ? (uint16_t*)r.table : c.take<uint16_t>(tiled);
+      h.query[i].tiled = image;
+      f.tiled = image;
       // one error word per attempt: a learned attempt's forest fallback shares the learned word
       r.err = iL[i] >= 0 ? b.d_errs + iL[i] : b.d_errs + nL + j;
       r.result = b.d_res_F + i;
@@ -2352,8 +2336,6 @@ void layout_batch(const relo_attempt* at, int n, const relo_ransac_params& p, ch
     if (scene_mode(at[i].scene_b->view) != b.query_mode) b.query_mode = kSceneAny;
     if (scene_mode(at[i].scene_a->view) != b.verify_mode) b.verify_mode = kSceneAny;
   }
-  b.forest_pixels = fpix;
-  b.max_trees = maxT;
   b.passL.n = nL;
   b.passL.R = RL;
   b.passL.chunks = chL;
@@ -2415,8 +2397,8 @@ relo_status issue_batch(relo_batch* b, relo_pose_result* results, cudaStream_t s
   RELO_CUDA(mark(b, 5, s, capturing));
   // pass F: forest attempts and fallbacks (skipped on the device where the learned pose verified)
   if (b->nF > 0) {
-    RELO_CUDA(launch_forest(b->d_forest, b->nF, nullptr, b->forest_pixels, s, b->max_trees, b->sched));
-    L += 1;
+    RELO_CUDA(launch_forest(b->forest.data(), b->nF, s, b->sched));
+    L += forest_launches(b->nF);
   }
   RELO_CUDA(mark(b, 6, s, capturing));
   st = run_pass(b->passF, s, &L, ev ? b->ev[7] : nullptr, ev ? b->ev[8] : nullptr, capturing, b->sched);
@@ -2471,7 +2453,6 @@ relo_status relo_batch_prepare(const relo_attempt* at, int32_t n, const relo_ran
   cudaError_t e = upload(b->d_query, h.query);
   if (e == cudaSuccess) e = upload(b->d_verify_L, h.verify_L);
   if (e == cudaSuccess) e = upload(b->d_verify_F, h.verify_F);
-  if (e == cudaSuccess) e = upload(b->d_forest, h.forest);
   if (e == cudaSuccess) e = upload(b->passL.d_jobs, h.ransac_L);
   if (e == cudaSuccess) e = upload(b->passF.d_jobs, h.ransac_F);
   if (e == cudaSuccess) e = upload(b->passL.d_alive_prefix, h.alive_L);
@@ -2538,7 +2519,7 @@ int32_t relo_batch_launch_count(const relo_batch* b) {
   if (!b) return 0;
   int L = 2 + 1;  // result init + query raycast, merge
   if (b->nL > 0) L += 1 + kRegLayers + 1 + 2 + pass_launches(b->passL, b->sched);
-  if (b->nF > 0) L += 1 + 2 + pass_launches(b->passF, b->sched);
+  if (b->nF > 0) L += forest_launches(b->nF) + 2 + pass_launches(b->passF, b->sched);
   return L;
 }
 

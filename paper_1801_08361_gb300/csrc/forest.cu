@@ -59,8 +59,13 @@ __device__ __forceinline__ DepthDivisor make_divisor7(int d) {
 template <int kDiv, bool kClamp = true>
 __device__ __forceinline__ int probe(int x, int raw, const DepthDivisor& dv, int limit, int oshift) {
   if (kDiv == 2) {
-    const int q = __mulhi(raw, (int)dv.M) - (raw >> 31);
-    return kClamp ? min(max(x + q, 0), limit) : x + q;
+    // one wide multiply-add of {x, raw >> 31}: for raw < 0 the low word's 2^32 - 1 turns the floor of
+    // the high word into the truncation, and x is added on the way
+    int q;
+    asm("{\n .reg .b64 c, r;\n .reg .b32 lo;\n mov.b64 c, {%3, %4};\n mad.wide.s32 r, %1, %2, c;\n mov.b64 {lo, %0}, r;\n}"
+        : "=r"(q)
+        : "r"(raw), "r"((int)dv.M), "r"(raw >> 31), "r"(x));
+    return kClamp ? min(max(q, 0), limit) : q;
   }
   const int n = (raw >> oshift) * 1000;
   int q;
@@ -75,96 +80,115 @@ __device__ __forceinline__ int probe(int x, int raw, const DepthDivisor& dv, int
 }
 
 // Descends pixel (u, v) of depth d through the trees, interleaved level by level so each level
-// issues T independent node loads instead of a chain of T * D dependent ones.  In the device copy
-// of the forest (relo_create_forest) a node's third word holds the mask of a probe's value (0xFFFF
-// for depth, 0xFF for a colour channel) and the bit offsets of its two probes' values in a packed
-// pixel (0 for depth, 16 + 8 c for colour channel c), ready to use.
-// kPacked: probes read the packed image (one 64-bit load, then a shift and a mask: no branch on
-// the node's kind, which differs between neighbouring lanes); otherwise the depth or the colour
-// image, by kind.
-// The CTA's shared-memory copy of the top levels of its forest's trees ([T][2^levels - 1]).
+// issues T independent node loads instead of a chain of T * D dependent ones.  The device copy of the
+// forest (relo_create_forest) is laid out so that a visit takes few instructions:
+//   - nodes are numbered from 1 with the left child at 2 n + 1 and the right one at 2 n, so the next
+//     node is n shifted left with the sign of (a - b - tau) shifted in: one funnel shift (tau is held
+//     within 17 bits, so the difference never wraps), and a leaf is the complement of the node's bits;
+//   - node n of tree t lies at [n][t]: one multiply-add for an address, the tree an immediate offset;
+//   - the third word holds each probe's plane (low and high half) as a byte offset into a tile of the
+//     tiled image.
+// kTiled: probes read the tiled image, 8 x 8 pixels a tile, each tile its depths, then its r, g and b
+// planes as u16 (128 bytes a plane: one cache line).  What bounds the descent is the L1: a warp's load
+// takes about one cycle per distinct line (92.7 % of the data pipe's peak with 8-byte pixels in rows and
+// warps on rows of 32).  A warp of 8 x 4 pixels whose probes land in 8 x 8 planes touches 6.7 lines a
+// probe instead of 11.6, and 3.2 a node instead of 5.5 (counted on a house view).  Otherwise: the depth
+// or the colour image, by the node's kind.
+// 256 house images of five trees: 11.5 ms, 12.8 with pixels in rows and nodes a tree at a time; the L1 is
+// then at 64 % and the instructions bound it.  32 fragment views: 0.50 ms, 0.54 before.
+// Plane of a probe in a node's third word: its byte offset in a tile, 0 the depths, 128 (1 + c) channel c;
+// bit 0 marks channel 3, the alpha of the colour image, which a tiled image does not hold (it reads b).
+constexpr unsigned kPlaneMask = 0x380u;
+__device__ __forceinline__ unsigned plane_shift(unsigned z) { return 8u * (((z & kPlaneMask) >> 7) - 1u + (z & 1u)); }
+
+// The CTA's shared-memory copy of the top levels of its forest's trees ([2^levels][T]).
 extern __shared__ int4 s_forest_top[];
 
 // Levels [level_begin, level_end) with nodes from the forest in global memory, or (kShared) from
-// s_forest_top, which holds n_nodes of each tree.
-template <int MT, int kDiv, bool kPacked, bool kShared, bool kClamp>
+// s_forest_top; n_nodes: the nodes (times trees) that either holds.
+template <int MT, int kDiv, bool kTiled, bool kShared, bool kClamp>
 __device__ __forceinline__ void descend_levels(const ForestJob& job, int u, int v, const DepthDivisor& dv,
                                                int (&node)[MT], int n_nodes, int level_begin, int level_end) {
-  const int T = job.forest.T, W = job.W, H = job.H, os = job.forest.offset_shift;
+  const int T = job.T, W = job.W, H = job.H, os = job.offset_shift;
+  const unsigned row = ((unsigned)(W + 7) >> 3) * 64u - 16u;
   for (int level = level_begin; level < level_end; ++level) {
 #pragma unroll
     for (int t = 0; t < MT; ++t) {
       if (t < T) {
         int4 nd = make_int4(0, 0, 0, 0);
-        if (RELO_CHECK(node[t] >= 0 && node[t] < n_nodes))
-          nd = kShared ? s_forest_top[t * n_nodes + node[t]] : __ldg(&job.forest.nodes[(size_t)t * n_nodes + node[t]]);
+        if (RELO_CHECK(node[t] > 0 && node[t] < n_nodes))
+          nd = kShared ? s_forest_top[node[t] * T + t] : __ldg(job.nodes + (size_t)((unsigned)node[t] * (unsigned)T) + t);
         const int dx1 = (int)(int16_t)(nd.x & 0xFFFF), dy1 = nd.x >> 16;
         const int dx2 = (int)(int16_t)(nd.y & 0xFFFF), dy2 = nd.y >> 16;
-        const int q1 = probe<kDiv, kClamp>(v, dy1, dv, H - 1, os) * W + probe<kDiv, kClamp>(u, dx1, dv, W - 1, os);
-        const int q2 = probe<kDiv, kClamp>(v, dy2, dv, H - 1, os) * W + probe<kDiv, kClamp>(u, dx2, dv, W - 1, os);
+        const int y1 = probe<kDiv, kClamp>(v, dy1, dv, H - 1, os), x1 = probe<kDiv, kClamp>(u, dx1, dv, W - 1, os);
+        const int y2 = probe<kDiv, kClamp>(v, dy2, dv, H - 1, os), x2 = probe<kDiv, kClamp>(u, dx2, dv, W - 1, os);
         int a, b;
-        if (!RELO_CHECK((unsigned)q1 < (unsigned)(W * H) && (unsigned)q2 < (unsigned)(W * H))) {
+        if (!RELO_CHECK((unsigned)y1 < (unsigned)H && (unsigned)x1 < (unsigned)W && (unsigned)y2 < (unsigned)H &&
+                        (unsigned)x2 < (unsigned)W)) {
           node[t] = 2 * node[t] + 1;
           continue;
         }
-        if (kPacked) {
-          const unsigned mask = (unsigned)nd.z & 0xFFFFu, s1 = ((unsigned)nd.z >> 16) & 0xFFu, s2 = (unsigned)nd.z >> 24;
-          const uint2 p1 = __ldg(&job.packed[q1]), p2 = __ldg(&job.packed[q2]);
-          a = (int)(__funnelshift_rc(p1.x, p1.y, s1) & mask);
-          b = (int)(__funnelshift_rc(p2.x, p2.y, s2) & mask);
-        } else if ((nd.z & 0xFFFF) == 0xFFFF) {
-          a = __ldg(&job.depth[q1]);
-          b = __ldg(&job.depth[q2]);
+        const unsigned z = (unsigned)nd.z;
+        if (kTiled) {
+          // byte offset of pixel (x, y): 512 (tile) + plane + 16 (y & 7) + 2 (x & 7)
+          const unsigned o1 = (z & kPlaneMask) + (x1 & ~7) * 62u + (y1 & ~7) * row + 2 * x1 + 16 * y1;
+          const unsigned o2 = ((z >> 16) & kPlaneMask) + (x2 & ~7) * 62u + (y2 & ~7) * row + 2 * x2 + 16 * y2;
+          a = __ldg(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(job.tiled) + o1));
+          b = __ldg(reinterpret_cast<const uint16_t*>(reinterpret_cast<const char*>(job.tiled) + o2));
         } else {
-          a = (__ldg(&job.rgba[q1]) >> ((((unsigned)nd.z >> 16) & 0xFFu) - 16)) & 0xFF;
-          b = (__ldg(&job.rgba[q2]) >> (((unsigned)nd.z >> 24) - 16)) & 0xFF;
+          const int q1 = y1 * W + x1, q2 = y2 * W + x2;
+          if ((z & kPlaneMask) == 0u) {
+            a = __ldg(&job.depth[q1]);
+            b = __ldg(&job.depth[q2]);
+          } else {
+            a = (__ldg(&job.rgba[q1]) >> plane_shift(z)) & 0xFF;
+            b = (__ldg(&job.rgba[q2]) >> plane_shift(z >> 16)) & 0xFF;
+          }
         }
-        node[t] = 2 * node[t] + ((a - b < nd.w) ? 1 : 2);
+        node[t] = (int)__funnelshift_l((unsigned)(a - b - nd.w), (unsigned)node[t], 1);
       }
     }
   }
 }
 
 // The first top_levels levels from s_forest_top, the rest from global memory.
-template <int MT, int kDiv, bool kPacked, bool kClamp>
+template <int MT, int kDiv, bool kTiled, bool kClamp>
 __device__ __forceinline__ void descend(const ForestJob& job, int u, int v, const DepthDivisor& dv, int (&node)[MT],
                                         int top_levels) {
   if (top_levels > 0)
-    descend_levels<MT, kDiv, kPacked, true, kClamp>(job, u, v, dv, node, (1 << top_levels) - 1, 0, top_levels);
-  descend_levels<MT, kDiv, kPacked, false, kClamp>(job, u, v, dv, node, (1 << job.forest.D) - 1, top_levels,
-                                                   job.forest.D);
+    descend_levels<MT, kDiv, kTiled, true, kClamp>(job, u, v, dv, node, 1 << top_levels, 0, top_levels);
+  descend_levels<MT, kDiv, kTiled, false, kClamp>(job, u, v, dv, node, 1 << job.D, top_levels, job.D);
 }
 
 // Descent with or without probe clamping: a warp whose pixels all lie at least the forest's probe
 // reach trunc((max |offset|) * 1000 / d) from every image edge takes the clamp-free instance (its
 // probes cannot leave the image, so both give the same leaves); any other warp clamps.  Instances
 // for more than 6 trees always clamp (a second copy of their descent would spill registers).
-template <int MT, int kDiv, bool kPacked>
+template <int MT, int kDiv, bool kTiled>
 __device__ __forceinline__ void descend_any(const ForestJob& job, int u, int v, int d, const DepthDivisor& dv,
                                             int (&node)[MT], int top_levels) {
   bool inside = false;
-  if (MT <= 6 && job.forest.probe_reach > 0) {
-    const int reach = (int)(((long long)(job.forest.probe_reach - 1) * 1000) / d);
+  if (MT <= 6 && job.probe_reach > 0) {
+    const int reach = (int)(((long long)(job.probe_reach - 1) * 1000) / d);
     inside = u >= reach && u + reach <= job.W - 1 && v >= reach && v + reach <= job.H - 1;
   }
-  if (MT <= 6 && __all_sync(__activemask(), inside)) descend<MT, kDiv, kPacked, false>(job, u, v, dv, node, top_levels);
-  else descend<MT, kDiv, kPacked, true>(job, u, v, dv, node, top_levels);
+  if (MT <= 6 && __all_sync(__activemask(), inside)) descend<MT, kDiv, kTiled, false>(job, u, v, dv, node, top_levels);
+  else descend<MT, kDiv, kTiled, true>(job, u, v, dv, node, top_levels);
 }
 
 // The leaf nodes of pixel (u, v) of depth d > 0 in every tree.
 template <int MT>
 __device__ __forceinline__ void descend_pixel(const ForestJob& job, int u, int v, int d, int (&node)[MT],
                                               int top_levels) {
-  const ForestView& f = job.forest;
 #pragma unroll
-  for (int t = 0; t < MT; ++t) node[t] = 0;
-  if (f.offset_shift == 7 && d >= 16) {
+  for (int t = 0; t < MT; ++t) node[t] = 1;
+  if (job.offset_shift == 7 && d >= 16) {
     const DepthDivisor dv = make_divisor7(d);
-    if (job.packed) descend_any<MT, 2, true>(job, u, v, d, dv, node, top_levels);
+    if (job.tiled) descend_any<MT, 2, true>(job, u, v, d, dv, node, top_levels);
     else descend_any<MT, 2, false>(job, u, v, d, dv, node, top_levels);
   } else {
     const DepthDivisor dv = make_divisor(d);
-    if (job.packed) {
+    if (job.tiled) {
       if (dv.shift >= 32) descend_any<MT, 1, true>(job, u, v, d, dv, node, top_levels);
       else descend_any<MT, 0, true>(job, u, v, d, dv, node, top_levels);
     } else {
@@ -180,87 +204,64 @@ __device__ __forceinline__ void descend_pixel(const ForestJob& job, int u, int v
 #define RELO_FOREST_MIN_BLOCKS 8
 #endif
 
-// One thread per pixel.  tiles == 0: a job's slot k is its pixel k (row-major); tiles == 1: its
-// slots run over 32 x 8 pixel tiles, 256 slots each, tiles row-major (neighbouring threads
-// probe neighbouring pixels in two dimensions).
+// One thread per pixel; a job's pixels in 32 x 8 tiles, tiles row-major, 256 threads each.
+// rows == 0: each warp covers 8 x 4 pixels of its tile; rows == 1: a row of 32.
 // levels > 0: the CTA first copies the top min(levels, D) levels of its job's trees into shared
-// memory (dynamic, top_trees x (2^levels - 1) nodes), so those node visits read shared memory.
-template <int MT>
-__global__ void __launch_bounds__(256, RELO_FOREST_MIN_BLOCKS)
-    forest_kernel(const ForestJob* __restrict__ jobs, int n_jobs, const ForestJob single, int tiles, int levels,
-                  int top_trees) {
-  const int64_t gid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  // jobs start on multiples of the CTA size, so the CTA's first pixel names its job; the job is
-  // staged in shared memory (its fields are read at every node visit)
-  const int64_t first = (int64_t)blockIdx.x * blockDim.x;
+// memory (dynamic, top_trees x 2^levels nodes), so those node visits read shared memory.
+template <int N>
+struct ForestJobs {
+  ForestJob j[N];
+};
+template <int MT, int N>
+__global__ void __launch_bounds__(256, MT <= 6 ? RELO_FOREST_MIN_BLOCKS : MT <= 8 ? 6 : 4)
+    forest_kernel(const __grid_constant__ ForestJobs<N> jobs, int n_jobs, int rows, int levels, int top_trees) {
+  // a CTA's 256 (or 128) threads lie in one tile, so in one job
+  const int tile = (int)(((int64_t)blockIdx.x * blockDim.x) >> 8);
   int lo = 0, hi = n_jobs - 1;
-  while (jobs && lo < hi) {
+  while (N > 1 && lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
-    if (jobs[mid].pixel_begin <= first) lo = mid;
+    if (jobs.j[mid].tile_begin <= tile) lo = mid;
     else hi = mid - 1;
   }
-  __shared__ __align__(16) ForestJob sj;
-  if (jobs) {
-    const unsigned long long* src = reinterpret_cast<const unsigned long long*>(jobs + lo);
-    unsigned long long* dst = reinterpret_cast<unsigned long long*>(&sj);
-    for (int i = threadIdx.x; i < (int)(sizeof(ForestJob) / 8); i += blockDim.x) dst[i] = src[i];
-  } else if (threadIdx.x == 0) {
-    sj = single;
-  }
-  __syncthreads();
-  const ForestJob& job = sj;
+  const ForestJob& job = jobs.j[N > 1 ? lo : 0];
   if (job_skipped(job.skip)) return;
-  // s_forest_top holds top_trees trees of 2^levels - 1 nodes
-  const int top_levels = job.forest.T <= top_trees ? min(levels, job.forest.D) : 0;
+  // s_forest_top holds 2^levels nodes (number 0 unused) of top_trees trees
+  const int top_levels = job.T <= top_trees ? min(levels, job.D) : 0;
   if (top_levels > 0) {
-    const int n_top = (1 << top_levels) - 1, n_int = (1 << job.forest.D) - 1;
-    for (int i = threadIdx.x; i < job.forest.T * n_top; i += blockDim.x) {
-      const int t = i / n_top;
-      s_forest_top[i] = __ldg(&job.forest.nodes[(size_t)t * n_int + (i - t * n_top)]);
-    }
+    for (int i = threadIdx.x; i < job.T << top_levels; i += blockDim.x) s_forest_top[i] = __ldg(&job.nodes[i]);
     __syncthreads();
   }
-  const int64_t slot = gid - job.pixel_begin;
-  const int64_t n_pix = (int64_t)job.W * job.H;
-  const int W = job.W, H = job.H;
-  int u, v;
-  if (tiles) {
-    const int64_t t = slot >> 8;
-    const int i = (int)(slot & 255), tx = (W + 31) >> 5;
-    u = (int)(t % tx) * 32 + (i & 31);
-    v = (int)(t / tx) * 8 + (i >> 5);
-    if (slot < 0 || u >= W || v >= H) return;
-  } else {
-    if (slot < 0 || slot >= n_pix) return;
-    u = (int)(slot % W);
-    v = (int)(slot / W);
-  }
-  const int64_t pix = (int64_t)v * W + u;
-  const ForestView& f = job.forest;
-  const int T = f.T;
+  const int W = job.W, H = job.H, T = job.T;
+  const int t = tile - job.tile_begin, tx = (W + 31) >> 5;
+  const int i = (int)((blockIdx.x * blockDim.x + threadIdx.x) & 255);
+  const int u = t % tx * 32 + (rows ? i & 31 : (i >> 5 & 3) * 8 + (i & 7));
+  const int v = t / tx * 8 + (rows ? i >> 5 : (i >> 7) * 4 + (i >> 3 & 3));
+  if (t < 0 || u >= W || v >= H) return;
+  const int64_t pix = (int64_t)v * W + u, n_pix = (int64_t)W * H;
   const int d = __ldg(&job.depth[pix]);
   if (d == 0) {
-    for (int t = 0; t < T; ++t) job.leaves[(size_t)t * n_pix + pix] = 0xFFFF;
+    for (int k = 0; k < T; ++k) job.leaves[(size_t)k * n_pix + pix] = 0xFFFF;
     return;
   }
-  const int n_int = (1 << f.D) - 1;
+  const int n_leaves = 1 << job.D;
   int node[MT];
   descend_pixel<MT>(job, u, v, d, node, top_levels);
 #pragma unroll
-  for (int t = 0; t < MT; ++t)
-    if (t < T && RELO_CHECK(node[t] >= n_int && node[t] < 2 * n_int + 1))
-      job.leaves[(size_t)t * n_pix + pix] = (uint16_t)(node[t] - n_int);
+  for (int k = 0; k < MT; ++k)
+    if (k < T && RELO_CHECK(node[k] >= n_leaves && node[k] < 2 * n_leaves))
+      job.leaves[(size_t)k * n_pix + pix] = (uint16_t)(~node[k] & (n_leaves - 1));
 }
 
-// Training: the leaves of the pixels on a stride grid, thread per grid pixel.
+// Training: the leaves of the pixels on a stride grid, thread per grid pixel, warps of 8 x 4.
 template <int MT>
-__global__ void __launch_bounds__(256, RELO_FOREST_MIN_BLOCKS)
+__global__ void __launch_bounds__(256, MT <= 6 ? RELO_FOREST_MIN_BLOCKS : MT <= 8 ? 6 : 4)
     forest_grid_kernel(const __grid_constant__ ForestJob job, int stride, int gw, int64_t n) {
-  const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const int u = (int)(i % gw) * stride, v = (int)(i / gw) * stride;
-  const ForestView& f = job.forest;
-  const int T = f.T, n_int = (1 << f.D) - 1;
+  const int tx = (gw + 31) >> 5, k = threadIdx.x;
+  const int gu = (int)(blockIdx.x % tx) * 32 + (k >> 5 & 3) * 8 + (k & 7), gv = (int)(blockIdx.x / tx) * 8 + (k >> 7) * 4 + (k >> 3 & 3);
+  const int64_t i = (int64_t)gv * gw + gu;
+  if (gu >= gw || i >= n) return;
+  const int u = gu * stride, v = gv * stride;
+  const int T = job.T, n_leaves = 1 << job.D;
   const int d = __ldg(&job.depth[(int64_t)v * job.W + u]);
   if (d == 0) {
     for (int t = 0; t < T; ++t) job.leaves[(size_t)t * n + i] = 0xFFFF;
@@ -270,15 +271,16 @@ __global__ void __launch_bounds__(256, RELO_FOREST_MIN_BLOCKS)
   descend_pixel<MT>(job, u, v, d, node, 0);
 #pragma unroll
   for (int t = 0; t < MT; ++t)
-    if (t < T && RELO_CHECK(node[t] >= n_int && node[t] < 2 * n_int + 1))
-      job.leaves[(size_t)t * n + i] = (uint16_t)(node[t] - n_int);
+    if (t < T && RELO_CHECK(node[t] >= n_leaves && node[t] < 2 * n_leaves))
+      job.leaves[(size_t)t * n + i] = (uint16_t)(~node[t] & (n_leaves - 1));
 }
 
 cudaError_t launch_forest_grid(const ForestJob& job, int stride, cudaStream_t s) {
   const int gw = (job.W + stride - 1) / stride;
-  const int64_t n = (int64_t)gw * ((job.H + stride - 1) / stride);
-  const unsigned grid = (unsigned)((n + 255) / 256);
-  const int T = job.forest.T;
+  const int gh = (job.H + stride - 1) / stride;
+  const int64_t n = (int64_t)gw * gh;
+  const unsigned grid = (unsigned)(((gw + 31) / 32) * (int64_t)((gh + 7) / 8));
+  const int T = job.T;
   if (T <= 4) forest_grid_kernel<4><<<grid, 256, 0, s>>>(job, stride, gw, n);
   else if (T <= 5) forest_grid_kernel<5><<<grid, 256, 0, s>>>(job, stride, gw, n);
   else if (T <= 8) forest_grid_kernel<8><<<grid, 256, 0, s>>>(job, stride, gw, n);
@@ -288,32 +290,46 @@ cudaError_t launch_forest_grid(const ForestJob& job, int stride, cudaStream_t s)
 
 RELO_DEFINE_CHECK_READER(check_failures_forest)
 
-cudaError_t launch_forest(const ForestJob* jobs_dev, int n_jobs, const ForestJob* single, int64_t total_pixels,
-                          cudaStream_t s, int max_trees, const Schedule& sched) {
-  if (total_pixels <= 0) return cudaSuccess;
+template <int N>
+void launch_forest_jobs(const ForestJob* jobs, int n, int mt, unsigned grid, int threads, size_t smem, cudaStream_t s,
+                        int rows, int levels, int trees) {
+  ForestJobs<N> a;
+  for (int k = 0; k < n; ++k) {
+    a.j[k] = jobs[k];
+    a.j[k].tile_begin -= jobs[0].tile_begin;
+  }
+  if (mt == 4) forest_kernel<4, N><<<grid, threads, smem, s>>>(a, n, rows, levels, trees);
+  else if (mt == 5) forest_kernel<5, N><<<grid, threads, smem, s>>>(a, n, rows, levels, trees);
+  else if (mt == 6) forest_kernel<6, N><<<grid, threads, smem, s>>>(a, n, rows, levels, trees);
+  else if (mt == 8) forest_kernel<8, N><<<grid, threads, smem, s>>>(a, n, rows, levels, trees);
+  else forest_kernel<kMaxTrees, N><<<grid, threads, smem, s>>>(a, n, rows, levels, trees);
+}
+
+cudaError_t launch_forest(const ForestJob* jobs, int n, cudaStream_t s, const Schedule& sched) {
   const int threads = sched.forest_threads;
   if ((threads != 128 && threads != 256) || (sched.forest_tiles != 0 && sched.forest_tiles != 1) ||
       sched.forest_smem_levels < 0 || sched.forest_smem_levels > kMaxSmemLevels)
     return cudaErrorInvalidValue;
-  ForestJob one{};
-  if (single) one = *single;
-  // total_pixels counts each job's slots, a multiple of 256 (pixel_begin), so no CTA spans two jobs
-  const unsigned grid = (unsigned)((total_pixels + threads - 1) / threads);
-  const int tiles = sched.forest_tiles;
-  // the unrolled width: the smallest instance that holds every job's trees (5, the usual forest
-  // size, has its own: no idle unrolled slots, no spills at 32 registers)
-  const int mt = max_trees <= 4 ? 4 : max_trees <= 5 ? 5 : max_trees <= 6 ? 6 : max_trees <= 8 ? 8 : kMaxTrees;
-  // the staged levels take at most 48 KB of shared memory per CTA (fewer levels for many trees)
-  const size_t trees = (size_t)max(1, min(max_trees, mt));
-  int levels = sched.forest_smem_levels;
-  while (levels > 0 && trees * ((1u << levels) - 1) * sizeof(int4) > 48 * 1024) --levels;
-  const size_t smem = levels > 0 ? trees * ((1u << levels) - 1) * sizeof(int4) : 0;
-  if (mt == 4) forest_kernel<4><<<grid, threads, smem, s>>>(jobs_dev, n_jobs, one, tiles, levels, (int)trees);
-  else if (mt == 5) forest_kernel<5><<<grid, threads, smem, s>>>(jobs_dev, n_jobs, one, tiles, levels, (int)trees);
-  else if (mt == 6) forest_kernel<6><<<grid, threads, smem, s>>>(jobs_dev, n_jobs, one, tiles, levels, (int)trees);
-  else if (mt == 8) forest_kernel<8><<<grid, threads, smem, s>>>(jobs_dev, n_jobs, one, tiles, levels, (int)trees);
-  else forest_kernel<kMaxTrees><<<grid, threads, smem, s>>>(jobs_dev, n_jobs, one, tiles, levels, (int)trees);
-  return cudaGetLastError();
+  for (int first = 0; first < n; first += kMaxForestJobs) {
+    const int here = min(kMaxForestJobs, n - first);
+    const ForestJob& last = jobs[first + here - 1];
+    const int64_t tiles = (int64_t)last.tile_begin + forest_job_tiles(last.W, last.H) - jobs[first].tile_begin;
+    const unsigned grid = (unsigned)(tiles * 256 / threads);
+    // the unrolled width: the smallest instance that holds every job's trees (5, the usual forest
+    // size, has its own: no idle unrolled slots)
+    int trees = 1;
+    for (int k = 0; k < here; ++k) trees = max(trees, jobs[first + k].T);
+    const int mt = trees <= 4 ? 4 : trees <= 5 ? 5 : trees <= 6 ? 6 : trees <= 8 ? 8 : kMaxTrees;
+    // the staged levels take at most 48 KB of shared memory per CTA (fewer levels for many trees)
+    int levels = sched.forest_smem_levels;
+    while (levels > 0 && ((size_t)trees << levels) * sizeof(int4) > 48 * 1024) --levels;
+    const size_t smem = levels > 0 ? ((size_t)trees << levels) * sizeof(int4) : 0;
+    if (here == 1) launch_forest_jobs<1>(jobs + first, here, mt, grid, threads, smem, s, sched.forest_tiles, levels, trees);
+    else launch_forest_jobs<kMaxForestJobs>(jobs + first, here, mt, grid, threads, smem, s, sched.forest_tiles, levels, trees);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 // ---------------------------------------------------------------------------------------------

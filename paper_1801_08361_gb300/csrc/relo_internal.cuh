@@ -152,7 +152,7 @@ __device__ __forceinline__ int lookup_block(const SceneView& s, int x, int y, in
 // Forest
 // ---------------------------------------------------------------------------------------------
 struct ForestView {
-  const int4* nodes;        // [T][2^D - 1] split nodes, 16 bytes each
+  const int4* nodes;        // [2^D][T] split nodes, 16 bytes each (numbered as forest.cu's descent takes them)
   const float* modes;       // [T][2^D][M][12]
   const uint8_t* n_modes;   // [T][2^D]
   const float4* top;        // [T][2^D]: mode 0 mean xyz, w = number of modes
@@ -352,7 +352,7 @@ struct RayJob {
   const uint16_t* depth_ref;   // compare mode: reference depth (D_b)
   unsigned long long* counts;  // compare mode: {omega_a, omega_b, omega_ab, sum |D_a - D_b|}
   int32_t* err;                // device error flag (nullable)
-  uint2* packed;               // nullable, colour renders: {depth | r << 16 | g << 24, b} per pixel
+  uint16_t* tiled;             // nullable, colour renders: the image as the forest reads it (see ForestJob)
   int32_t tile_begin;          // first 16 x 16 tile of this job in the flattened launch
   int32_t pad;                 // size: a multiple of 16 bytes (staged in shared memory)
 };
@@ -361,17 +361,37 @@ static_assert(sizeof(RayJob) % 16 == 0, "RayJob is staged in shared memory as 16
 // ---------------------------------------------------------------------------------------------
 // Forest jobs (one image through one forest)
 // ---------------------------------------------------------------------------------------------
+// Passed to the kernel by value, an array of them for a batch: read at every node visit, a job's fields
+// come from the constant bank as operands, not through registers or shared memory.
 struct ForestJob {
-  ForestView forest;
+  const int4* nodes;           // as ForestView
   const uint16_t* depth;
   const uint32_t* rgba;
-  const uint2* packed;         // nullable: the same image packed per pixel (see RayJob::packed)
+  const uint16_t* tiled;       // nullable: the same image in 8 x 8 tiles, row-major, each [depth, r, g, b][8][8] u16
   uint16_t* leaves;            // [T][H][W]
-  int32_t W, H;
-  int64_t pixel_begin;         // first pixel of this job in the flattened launch (multiple of 256)
   const int32_t* skip;         // when set and non-zero the job does nothing (fallback not needed)
+  int32_t W, H;
+  int32_t T, D;
+  int32_t probe_reach, offset_shift;
+  int32_t tile_begin;          // first 32 x 8 pixel tile of this job in the flattened launch
+  int32_t pad;
 };
-static_assert(sizeof(ForestJob) % 8 == 0, "ForestJob is staged in shared memory as 8-byte words");
+constexpr int kMaxForestJobs = 256;  // per launch (kernel parameters: 80 bytes a job, 20 KB)
+inline ForestJob make_forest_job(const ForestView& f, const uint16_t* depth, const uint32_t* rgba, uint16_t* leaves, int W,
+                                 int H) {
+  ForestJob j{};
+  j.nodes = f.nodes;
+  j.depth = depth;
+  j.rgba = rgba;
+  j.leaves = leaves;
+  j.W = W;
+  j.H = H;
+  j.T = f.T;
+  j.D = f.D;
+  j.probe_reach = f.probe_reach;
+  j.offset_shift = f.offset_shift;
+  return j;
+}
 
 // ---------------------------------------------------------------------------------------------
 // RANSAC jobs (one query view, one forest) and their workspace
@@ -446,29 +466,26 @@ struct Carver {
 struct Schedule {
   int ray_warp_log2w = 3;    // raycast: each warp covers a (1 << w) x (32 >> w) footprint of its 16 x 16 tile
   int forest_threads = 256;  // forest: CTA size (128 or 256)
-  int forest_tiles = 0;      // forest: 0 = each CTA takes consecutive pixels, 1 = 32 x 8 pixel tiles
+  int forest_tiles = 0;      // forest: each warp takes 8 x 4 pixels (0) or a row of 32 (1) of a 32 x 8 tile
   int forest_smem_levels = 0;  // forest: top levels of the trees each CTA copies to shared memory (0: none)
   int search_ctas_per_sm = 0;  // hypothesis search: persistent CTAs per SM (0: occupancy maximum)
   int refit_per = 0;         // re-fit: survivors per one-warp CTA (0: spread over twice the SM count)
   int persistent = 0;        // RANSAC of a batch: 0 = one launch per stage, 1 = one persistent launch
 };
 constexpr int kMaxSmemLevels = 10;
-// Forest slots a job of W x H pixels takes (a multiple of 256 that also holds its 32 x 8 tiles).
-inline int64_t forest_slots(int W, int H) {
-  const int64_t rows = ((int64_t)W * H + 255) / 256 * 256;
-  const int64_t tiles = (int64_t)((W + 31) / 32) * ((H + 7) / 8) * 256;
-  return rows > tiles ? rows : tiles;
-}
+// 32 x 8 pixel tiles of a W x H image.
+inline int forest_job_tiles(int W, int H) { return ((W + 31) / 32) * ((H + 7) / 8); }
+// u16 values of a W x H image in 8 x 8 tiles (ForestJob::tiled).
+inline size_t tiled_values(int W, int H) { return (size_t)((W + 7) / 8) * ((H + 7) / 8) * 256; }
 
 // jobs_dev == nullptr: the single job is passed by value.  mode: the scene_mode that all scenes of
 // jobs_dev share, or kSceneAny (a single job's own scene decides for itself).
 cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* single, int total_tiles,
                            bool with_colour, bool compare, cudaStream_t s, const Schedule& sched = Schedule(),
                            int mode = kSceneAny);
-// max_trees: the largest tree count among the jobs (selects the kernel's unrolled width).  With
-// sched.forest_tiles, each job must own forest_slots(W, H) slots from its pixel_begin.
-cudaError_t launch_forest(const ForestJob* jobs_dev, int n_jobs, const ForestJob* single, int64_t total_pixels,
-                          cudaStream_t s, int max_trees, const Schedule& sched = Schedule());
+// n jobs (host array, tile_begin ascending from 0), forest_launches(n) launches.
+inline int forest_launches(int n) { return (n + kMaxForestJobs - 1) / kMaxForestJobs; }
+cudaError_t launch_forest(const ForestJob* jobs, int n, cudaStream_t s, const Schedule& sched = Schedule());
 int ray_tiles(int W, int H);
 // Global map rendering over n scene jobs sharing one image size (owner, rgba, err_flag nullable).
 cudaError_t launch_render_global(const RayJob* jobs_dev, int n, int W, int H, uint16_t* depth, uint32_t* rgba,

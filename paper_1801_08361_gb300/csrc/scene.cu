@@ -343,7 +343,13 @@ __global__ void __launch_bounds__(kTile* kTile, kMode == kSceneCells ? 5 : kColo
     }
     if (job.depth) job.depth[pix] = (uint16_t)depth_mm;
     if (kColour && job.rgba) job.rgba[pix] = col;
-    if (kColour && job.packed) job.packed[pix] = make_uint2((uint32_t)depth_mm | (col & 0xFFFFu) << 16, (col >> 16) & 0xFFu);
+    if (kColour && job.tiled) {
+      uint16_t* t = job.tiled + ((size_t)(v >> 3) * ((job.W + 7) >> 3) + (u >> 3)) * 256 + (v & 7) * 8 + (u & 7);
+      t[0] = (uint16_t)depth_mm;
+      t[64] = (uint16_t)(col & 0xFFu);
+      t[128] = (uint16_t)((col >> 8) & 0xFFu);
+      t[192] = (uint16_t)((col >> 16) & 0xFFu);
+    }
     if (err && job.err) atomicExch(job.err, RELO_EDEVICE);
   }
   if (kCompare) {
