@@ -1558,9 +1558,10 @@ struct RegBuffers {
   float4* tgt = nullptr;              // [n][Hc][Wc]
   bf16* ghead = nullptr;              // [n][Hc][Wc][16]
   bf16* gpre[kRegLayers] = {};        // gpre[l] = gradient of layer l's pre-activation output (l < 7)
-  float* partial = nullptr;           // backward-weight chunk sums
-  float* bias_scratch = nullptr;
+  float* partial = nullptr;           // backward-weight sums per CTA
   float* loss = nullptr;
+  float* loss_sums = nullptr;
+  int32_t* counters = nullptr;        // scored cells, loss CTAs done
   double* poses = nullptr;            // [n][16]
   size_t bytes = 0;
 };
@@ -1577,33 +1578,41 @@ void reg_layout(char* base, int n, int W, int H, bool training, RegBuffers& b, s
     b.tgt = c.take<float4>(cells);
     b.ghead = c.take<bf16>(cells * 16);
     for (int l = 0; l < kRegLayers - 1; ++l) b.gpre[l] = c.take<bf16>((size_t)n * Hs[l + 1] * Ws[l + 1] * 64);
-    size_t part = 0, bias = 0;
-    for (int l = 0; l < kRegLayers; ++l) {
-      const size_t px = (size_t)n * Hs[l + 1] * Ws[l + 1];
-      const size_t chunks = (px + kWgradChunk - 1) / kWgradChunk;
-      part = std::max(part, chunks * 9 * kRegCoutPad[l] * kRegCinPad[l]);
-      bias = std::max(bias, ((px + 2047) / 2048) * 64);
-    }
+    size_t part = 0;
+    for (int l = 0; l < kRegLayers; ++l)
+      part = std::max(part, wgrad_parts(kRegCinPad[l], n, Hs[l + 1], Ws[l + 1]) * wgrad_partial_floats(kRegCinPad[l], kRegCoutPad[l]));
     b.partial = c.take<float>(part);
-    b.bias_scratch = c.take<float>(bias);
     b.loss = c.take<float>(1);
+    b.loss_sums = c.take<float>(loss_blocks((int)cells));
+    b.counters = c.take<int32_t>(2);
     b.poses = c.take<double>((size_t)n * 16);
   }
   b.bytes = c.off;
 }
 
 relo_status reg_forward(relo_regressor* r, const RegBuffers& b, const uint16_t* depth, const uint8_t* rgba, int n,
-                        int W, int H, cudaStream_t s) {
+                        int W, int H, cudaStream_t s, bool training = false) {
   int Hs[kRegLayers + 1], Ws[kRegLayers + 1];
   reg_sizes(W, H, Hs, Ws);
-  RELO_CUDA(launch_input(depth, (const uint32_t*)rgba, (long)n * H * W, b.x, s));
+  // the tcgen05 first layer reads the images themselves; the backward pass needs the network's input
+  if (training || !g_conv_tcgen05.load()) RELO_CUDA(launch_input(depth, (const uint32_t*)rgba, (long)n * H * W, b.x, s));
   RELO_CUDA(cudaMemsetAsync(r->d_status, 0, sizeof(int32_t), s));
   for (int l = 0; l < kRegLayers; ++l) {
+    if (l == 0 && g_conv_tcgen05.load()) {
+      RELO_CUDA(launch_conv_first(depth, (const uint32_t*)rgba, n, H, W, r->d_wk[0], r->d_bias[0], b.act[1], Hs[1], Ws[1],
+                                  r->d_status, r->n_sms, s, g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
+      continue;
+    }
     if (kRegCoutPad[l] == 64 && g_conv_tcgen05.load()) {
       // every layer but the head on the tcgen05 tensor cores (TMA-fed implicit GEMM)
-      RELO_CUDA(launch_conv_tc(kRegCinPad[l], l == 0 ? b.x : b.act[l], n, Hs[l], Ws[l], r->d_wk[l], r->d_bias[l],
+      RELO_CUDA(launch_conv_tc(kRegCinPad[l], b.act[l], n, Hs[l], Ws[l], r->d_wk[l], r->d_bias[l],
                                nullptr, b.act[l + 1], Hs[l + 1], Ws[l + 1], kRegStride[l], 1, 1, r->d_status, r->n_sms,
                                s, g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
+      continue;
+    }
+    if (l == kRegLayers - 1 && g_conv_tcgen05.load()) {
+      RELO_CUDA(launch_conv_head(b.act[l], n, Hs[l], Ws[l], r->d_wk[l], r->d_bias[l], b.head, r->d_status, r->n_sms, s,
+                                 g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
       continue;
     }
     ConvArgs a{};
@@ -1641,13 +1650,8 @@ relo_status reg_backward(relo_regressor* r, const RegBuffers& b, int n, int W, i
     wa.Wo = Ws[l + 1];
     wa.stride = kRegStride[l];
     wa.GS = gs;
-    wa.chunk_pix = kWgradChunk;
-    RELO_CUDA(launch_wgrad(kRegCinPad[l], kRegCoutPad[l] / 8, wa, s));
-    const long px = (long)n * Hs[l + 1] * Ws[l + 1];
-    const int chunks = (int)((px + kWgradChunk - 1) / kWgradChunk);
-    RELO_CUDA(launch_wgrad_reduce(b.partial, chunks, kRegCoutPad[l], kRegCinPad[l], kRegCin[l], kRegCout[l],
-                                  r->d_g + r->w_off[l], s));
-    RELO_CUDA(launch_bias_grad(g, px, gs, kRegCout[l], b.bias_scratch, r->d_g + r->b_off[l], s));
+    RELO_CUDA(launch_wgrad(kRegCinPad[l], kRegCoutPad[l], wa, kRegCin[l], kRegCout[l], r->d_g + r->w_off[l],
+                           r->d_g + r->b_off[l], s));
     if (l > 0) {
       ConvArgs a{};
       a.in = g;
@@ -1672,6 +1676,9 @@ relo_status reg_backward(relo_regressor* r, const RegBuffers& b, int n, int W, i
         // transposed weights, masked by the ReLU of the layer's input: tcgen05 as well
         RELO_CUDA(launch_conv_tc(gs, g, n, a.Hi, a.Wi, r->d_wt[l], nullptr, b.act[l], b.gpre[l - 1], Hs[l], Ws[l], 1,
                                  1, 0, r->d_status, r->n_sms, s, g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
+      } else if (a.upsample && g_conv_tcgen05.load()) {
+        RELO_CUDA(launch_conv_up(g, n, Hs[l + 1], Ws[l + 1], r->d_wt[l], b.act[l], b.gpre[l - 1], r->d_status, r->n_sms, s,
+                                 g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
       } else {
         RELO_CUDA(launch_conv(gs, 8, a, r->n_sms, s));
       }
@@ -1693,7 +1700,7 @@ relo_status reg_loss_and_grads(relo_regressor* r, const RegBuffers& b, const uin
                                int n, const relo_intrinsics* in, const double* poses, cudaStream_t s) {
   const int W = in->width, H = in->height, Wc = W / 8, Hc = H / 8;
   RELO_CUDA(cudaMemcpyAsync(b.poses, poses, (size_t)n * 16 * sizeof(double), cudaMemcpyHostToDevice, s));
-  relo_status st = reg_forward(r, b, depth, rgba, n, W, H, s);
+  relo_status st = reg_forward(r, b, depth, rgba, n, W, H, s, true);
   if (st) return st;
   CellArgs ca{};
   ca.depth = depth;
@@ -1710,8 +1717,8 @@ relo_status reg_loss_and_grads(relo_regressor* r, const RegBuffers& b, const uin
   ca.ox = r->origin[0];
   ca.oy = r->origin[1];
   ca.oz = r->origin[2];
-  RELO_CUDA(launch_targets(ca, b.tgt, s));
-  RELO_CUDA(launch_loss(b.head, b.tgt, n * Wc * Hc, b.ghead, b.loss, s));
+  RELO_CUDA(launch_targets(ca, b.tgt, b.counters, s));
+  RELO_CUDA(launch_loss(b.head, b.tgt, n * Wc * Hc, b.ghead, b.counters, b.loss_sums, b.loss, s));
   return reg_backward(r, b, n, W, H, s);
 }
 
@@ -1876,8 +1883,20 @@ relo_status relo_regressor_train_step(relo_regressor* r, const uint16_t* depth, 
   if (st) return st;
   cudaStream_t s = (cudaStream_t)stream;
   r->t += 1;
-  RELO_CUDA(launch_adam(r->d_p, r->d_g, r->d_m, r->d_v, r->n_params, lr, r->t, s));
-  return reg_pack(r, s);
+  AdamArgs a{};
+  a.p = r->d_p;
+  a.m = r->d_m;
+  a.v = r->d_v;
+  a.g = r->d_g;
+  a.n = (int)r->n_params;
+  for (int l = 0; l < kRegLayers; ++l) {
+    a.w_off[l] = (int)r->w_off[l];
+    a.wk[l] = r->d_wk[l];
+    a.wt[l] = r->d_wt[l];
+    a.bias[l] = r->d_bias[l];
+  }
+  RELO_CUDA(launch_adam(a, lr, r->t, s));
+  return RELO_OK;
 }
 
 

@@ -17,7 +17,9 @@
 // channels, contracted over 9 taps x input channels; each CTA (4 warps) keeps all 9 taps of the
 // weights in shared memory and loops over 64-pixel tiles, gathering one tap's input rows per
 // step.  The backward-data pass of a stride-2 layer is the same kernel reading its input
-// through a virtual zero-inserted upsampling, with the weights flipped and transposed.
+// through a virtual zero-inserted upsampling, with the weights flipped and transposed.  That
+// kernel (conv_kernel) is what the tcgen05 convolutions (conv_tc.cu), which run by default, are
+// compared with bit for bit; the other kernels here serve both.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -38,9 +40,6 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 }
 
 __device__ __forceinline__ uint32_t ld32(const bf16* p) { return *reinterpret_cast<const uint32_t*>(p); }
-
-
-constexpr int kConvPix = 64;  // output pixels per backward-weight tile (wgrad_kernel)
 
 // ldmatrix: four (or two) 8 x 8 b16 matrices from shared memory, rows addressed by lanes 8q..8q+7
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const bf16* p) {
@@ -216,12 +215,19 @@ cudaError_t launch_conv(int cin, int nt, const ConvArgs& a, int n_sms, cudaStrea
 }
 
 // ---------------------------------------------------------------------------------------------
-// Backward-weight: partial[chunk][tap][n][k] = sum over the chunk's output pixels p of
-// g[p, n] * in[src(p, tap), k]; a second kernel sums the chunks in a fixed order.
-// A CTA (8 warps) owns one tap and one chunk of pixels; per 64-pixel tile it stages the gradient
-// rows and the tap's gathered input rows as stored (pixel-major, 16-byte vectors, the next tile
-// prefetched into registers) and contracts over the pixels with ldmatrix.trans fragments:
-// M = input channels, N = output channels, K = pixels.
+// Backward-weight: gw[tap][k][n] = sum over output pixels p of in[src(p, tap), k] g[p, n], and the bias
+// gradient, the sum of g.  A persistent CTA (8 warps) walks tiles of 8 x 8 output pixels; a tile's
+// input window and its gradients come into shared memory once, by asynchronous copies while the
+// previous tile is multiplied, and serve all nine taps (a CTA per tap read both nine times over and
+// left 75 to 1200 partial sums per weight: 1.2 ms of a 2.9 ms step with its sums and a bias pass of
+// its own).  Contraction over the pixels with ldmatrix.trans fragments: M = input channels, N = output
+// channels, K = the 16 pixels of two tile rows.  The tensor core sums the 64 pixels of a tile; tiles are
+// added to the sums of all taps, in registers (144 a thread at 64 x 64 channels), by rounded FP32
+// additions -- the tensor core's own additions drop bits, which a chain over hundreds of tiles shows --
+// and one partial per CTA is left to sum.
+// The bias is one more product, with a row of ones.  16 views of 640 x 480: 0.38 ms with the sums for
+// all layers; the 64-channel kernels are bound by mma.sync (288 products a scheduler and tile), the
+// first layer's by its three passes over 157 MB and by latency, hence two CTAs an SM there.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const bf16* p) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(p);
@@ -235,182 +241,234 @@ __device__ __forceinline__ void ldsm_x2_t(uint32_t& r0, uint32_t& r1, const bf16
   asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(a));
 }
 
-constexpr int kWgradThreads = 256;
+// 16 bytes to shared memory, zeros where !ok (src is then not read)
+__device__ __forceinline__ void copy_or_zero16(bf16* dst, const bf16* src, bool ok) {
+  const unsigned a = (unsigned)__cvta_generic_to_shared(dst);
+  const int n = ok ? 16 : 0;
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"(a), "l"(src), "r"(n) : "memory");
+}
 
-template <int CIN, int NT>
-__global__ void __launch_bounds__(kWgradThreads) wgrad_kernel(WgradArgs a) {
-  constexpr int N = NT * 8;
-  constexpr int MT = CIN / 16;                          // m16 tiles over the input channels
-  constexpr int WM = (MT >= 2 && MT * NT >= 32) ? 2 : 1;  // m16 tiles per warp
-  constexpr int WN = (NT >= 2 && MT * NT >= 32) ? 2 : 1;  // n8 tiles per warp
-  constexpr int MG = MT / WM, NG = NT / WN;
-  static_assert(MG * NG <= kWgradThreads / 32, "warp split");
-  constexpr int RI = CIN + 8;                           // row strides (bf16): conflict-free ldmatrix
-  constexpr int RG = (N < 16 ? 16 : N) + 8;
-  constexpr int CI = CIN / 8, CG = N / 8;               // 16-B chunks per pixel row
-  constexpr int PI = (kConvPix * CI + kWgradThreads - 1) / kWgradThreads;
-  constexpr int PG = (kConvPix * CG + kWgradThreads - 1) / kWgradThreads;
-  __shared__ __align__(16) bf16 sI[kConvPix][RI];
-  __shared__ __align__(16) bf16 sG[kConvPix][RG];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, t = lane & 3;
-  const int tap = blockIdx.y, ky = tap / 3, kx = tap % 3;
-  const long total = (long)a.B * a.Ho * a.Wo;
-  const long p_begin = (long)blockIdx.x * a.chunk_pix;
-  const long p_end = min(p_begin + (long)a.chunk_pix, total);
-  const int mg = warp % MG, ng = warp / MG;
-  const bool mma_warp = warp < MG * NG;
-  float acc[WM][WN][4];
-#pragma unroll
-  for (int i = 0; i < WM; ++i)
-#pragma unroll
-    for (int j = 0; j < WN; ++j) acc[i][j][0] = acc[i][j][1] = acc[i][j][2] = acc[i][j][3] = 0.f;
+constexpr int kWgradThreads = 256, kWgradW = 8, kWgradH = 8;  // a tile's output pixels
+constexpr int kWgradK = kWgradW * kWgradH / 16;               // products' depth: pairs of tile rows
 
-  uint4 vi[PI], vg[PG];
-  auto fetch = [&](long p0) {
+// CIN input channels (16 or 64), NW n8 tiles of output channels per warp: N = 16 NW channels of g rows
+// of GS; STRIDE 1 or 2.
+template <int CIN, int NW, int STRIDE>
+struct WgradShape {
+  static constexpr int kHaloW = (kWgradW - 1) * STRIDE + 3, kHaloH = (kWgradH - 1) * STRIDE + 3;
+  static constexpr int kN = 16 * NW;
+  static constexpr int kRowI = CIN + 8, kRowG = kN + 8;  // padded rows (bf16): conflict-free ldmatrix
+  static constexpr int kInElems = kHaloW * kHaloH * kRowI, kGElems = kWgradW * kWgradH * kRowG;
+  static constexpr int kStage = kInElems + kGElems;
+  static constexpr int kStages = 4;
+  static constexpr size_t kSmem = kStages * (size_t)kStage * sizeof(bf16);
+  // warps: MG groups of 16 input channels x 2 halves of the output channels x TG groups of taps
+  static constexpr int kMG = CIN / 16, kTG = 8 / (2 * kMG), kTaps = (9 + kTG - 1) / kTG;
+};
+
+template <int CIN, int NW, int STRIDE>
+__global__ void __launch_bounds__(kWgradThreads, CIN == 16 ? 2 : 1) wgrad_kernel(WgradArgs a) {
+  using S = WgradShape<CIN, NW, STRIDE>;
+  extern __shared__ __align__(16) unsigned char wgrad_smem[];
+  bf16* smem = reinterpret_cast<bf16*>(wgrad_smem);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int mg = warp % S::kMG, nh = (warp / S::kMG) & 1, tg = warp / (2 * S::kMG);
+  const int tap0 = tg * S::kTaps;
+  const bool bias_warp = mg == 0 && tg == 0;
+  float acc[S::kTaps][NW][4], accb[NW][2];
 #pragma unroll
-    for (int i = 0; i < PI; ++i) {
-      const int v = tid + i * kWgradThreads;
-      vi[i] = make_uint4(0u, 0u, 0u, 0u);
-      const long p = p0 + v / CI;
-      if (v < kConvPix * CI && p < p_end) {
-        const int ox = (int)(p % a.Wo), oy = (int)((p / a.Wo) % a.Ho), b = (int)(p / ((long)a.Wo * a.Ho));
-        const int iy = oy * a.stride + ky - 1, ix = ox * a.stride + kx - 1;
-        if (iy >= 0 && ix >= 0 && iy < a.Hi && ix < a.Wi)
-          vi[i] = __ldg(reinterpret_cast<const uint4*>(a.in + (((size_t)b * a.Hi + iy) * a.Wi + ix) * CIN) + v % CI);
-      }
+  for (int t = 0; t < S::kTaps; ++t)
+#pragma unroll
+    for (int j = 0; j < NW; ++j) acc[t][j][0] = acc[t][j][1] = acc[t][j][2] = acc[t][j][3] = 0.f;
+#pragma unroll
+  for (int j = 0; j < NW; ++j) accb[j][0] = accb[j][1] = 0.f;
+  const uint32_t ones[4] = {0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u};
+  const int tiles_x = (a.Wo + kWgradW - 1) / kWgradW, tiles_y = (a.Ho + kWgradH - 1) / kWgradH;
+  const int n_tiles = a.B * tiles_x * tiles_y;
+
+  auto load = [&](int tile, int stage) {
+    bf16* sI = smem + stage * S::kStage;
+    bf16* sG = sI + S::kInElems;
+    const int b = tile / (tiles_x * tiles_y), q = tile % (tiles_x * tiles_y);
+    const int oy0 = q / tiles_x * kWgradH, ox0 = q % tiles_x * kWgradW;
+    constexpr int CI = CIN / 8, CG = S::kN / 8;
+    for (int v = tid; v < S::kHaloW * S::kHaloH * CI; v += kWgradThreads) {
+      const int px = v / CI, c = v % CI, hy = px / S::kHaloW, hx = px % S::kHaloW;
+      const int iy = oy0 * STRIDE - 1 + hy, ix = ox0 * STRIDE - 1 + hx;
+      const bool ok = iy >= 0 && ix >= 0 && iy < a.Hi && ix < a.Wi;
+      copy_or_zero16(sI + px * S::kRowI + c * 8, ok ? a.in + (((size_t)b * a.Hi + iy) * a.Wi + ix) * CIN + c * 8 : a.in, ok);
     }
-#pragma unroll
-    for (int i = 0; i < PG; ++i) {
-      const int v = tid + i * kWgradThreads;
-      vg[i] = make_uint4(0u, 0u, 0u, 0u);
-      const long p = p0 + v / CG;
-      if (v < kConvPix * CG && p < p_end)
-        vg[i] = __ldg(reinterpret_cast<const uint4*>(a.g + (size_t)p * a.GS) + v % CG);
+    for (int v = tid; v < kWgradW * kWgradH * CG; v += kWgradThreads) {
+      const int px = v / CG, c = v % CG, oy = oy0 + px / kWgradW, ox = ox0 + px % kWgradW;
+      const bool ok = oy < a.Ho && ox < a.Wo;
+      copy_or_zero16(sG + px * S::kRowG + c * 8, ok ? a.g + (((size_t)b * a.Ho + oy) * a.Wo + ox) * a.GS + c * 8 : a.g, ok);
     }
   };
-  fetch(p_begin);
-  for (long p0 = p_begin; p0 < p_end; p0 += kConvPix) {
-    __syncthreads();  // the previous tile's fragments are read
+
+  // the next kStages - 1 tiles are on their way while one is multiplied (a group per tile, empty past the end)
 #pragma unroll
-    for (int i = 0; i < PI; ++i) {
-      const int v = tid + i * kWgradThreads;
-      if (v < kConvPix * CI) *reinterpret_cast<uint4*>(&sI[v / CI][(v % CI) * 8]) = vi[i];
-    }
+  for (int k = 0; k < S::kStages - 1; ++k) {
+    if ((int)(blockIdx.x + k * gridDim.x) < n_tiles) load(blockIdx.x + k * gridDim.x, k);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  int stage = 0;
+  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, stage = stage + 1 < S::kStages ? stage + 1 : 0) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(S::kStages - 2) : "memory");
+    __syncthreads();  // the tile is here for all, and the one before is read
+    const int next = tile + (S::kStages - 1) * gridDim.x;
+    if (next < n_tiles) load(next, stage > 0 ? stage - 1 : S::kStages - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const bf16* sI = smem + stage * S::kStage;
+    const bf16* sG = sI + S::kInElems;
+    const int q = lane >> 3, r = lane & 7;
+    uint32_t bf[kWgradK][NW][2];
 #pragma unroll
-    for (int i = 0; i < PG; ++i) {
-      const int v = tid + i * kWgradThreads;
-      if (v < kConvPix * CG) *reinterpret_cast<uint4*>(&sG[v / CG][(v % CG) * 8]) = vg[i];
-    }
-    __syncthreads();
-    if (p0 + kConvPix < p_end) fetch(p0 + kConvPix);  // in flight during this tile's MMAs
-    if (mma_warp) {
+    for (int ks = 0; ks < kWgradK; ++ks) {
+      if (NW == 1) {
+        ldsm_x2_t(bf[ks][0][0], bf[ks][0][1], sG + (ks * 16 + r + 8 * (q & 1)) * S::kRowG + nh * 8);
+      } else {
 #pragma unroll
-      for (int ks = 0; ks < kConvPix / 16; ++ks) {
-        const int q = lane >> 3, r = lane & 7;
-        uint32_t af[WM][4];
-#pragma unroll
-        for (int wm = 0; wm < WM; ++wm)
-          ldsm_x4_t(af[wm], &sI[ks * 16 + r + 8 * (q >> 1)][(mg * WM + wm) * 16 + 8 * (q & 1)]);
-        uint32_t bf[WN][2];
-        if (WN == 2) {
+        for (int j = 0; j + 1 < NW; j += 2) {
           uint32_t b4[4];
-          ldsm_x4_t(b4, &sG[ks * 16 + r + 8 * (q & 1)][ng * 16 + 8 * (q >> 1)]);
-          bf[0][0] = b4[0];
-          bf[0][1] = b4[1];
-          bf[WN - 1][0] = b4[2];
-          bf[WN - 1][1] = b4[3];
-        } else {
-          ldsm_x2_t(bf[0][0], bf[0][1], &sG[ks * 16 + r + 8 * (q & 1)][ng * 8]);
+          ldsm_x4_t(b4, sG + (ks * 16 + r + 8 * (q & 1)) * S::kRowG + (nh * NW + j) * 8 + 8 * (q >> 1));
+          bf[ks][j][0] = b4[0];
+          bf[ks][j][1] = b4[1];
+          bf[ks][j + 1 < NW ? j + 1 : j][0] = b4[2];
+          bf[ks][j + 1 < NW ? j + 1 : j][1] = b4[3];
         }
+      }
+    }
 #pragma unroll
-        for (int wm = 0; wm < WM; ++wm)
+    for (int t = 0; t < S::kTaps; ++t) {
+      const int tap = tap0 + t;
+      if (S::kTG * S::kTaps > 9 && tap > 8) continue;
+      const int ky = tap / 3, kx = tap - 3 * ky;
+      float sum[NW][4];  // of this tile alone
 #pragma unroll
-          for (int wn = 0; wn < WN; ++wn) mma_bf16(acc[wm][wn], af[wm], bf[wn][0], bf[wn][1]);
+      for (int j = 0; j < NW; ++j) sum[j][0] = sum[j][1] = sum[j][2] = sum[j][3] = 0.f;
+#pragma unroll
+      for (int ks = 0; ks < kWgradK; ++ks) {
+        uint32_t af[4];
+        ldsm_x4_t(af, sI + (((2 * ks + (q >> 1)) * STRIDE + ky) * S::kHaloW + r * STRIDE + kx) * S::kRowI + mg * 16 + 8 * (q & 1));
+#pragma unroll
+        for (int j = 0; j < NW; ++j) mma_bf16(sum[j], af, bf[ks][j][0], bf[ks][j][1]);
+      }
+#pragma unroll
+      for (int j = 0; j < NW; ++j)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) acc[t][j][e] += sum[j][e];
+    }
+    if (bias_warp) {
+      float sum[NW][4];
+#pragma unroll
+      for (int j = 0; j < NW; ++j) {
+        sum[j][0] = sum[j][1] = sum[j][2] = sum[j][3] = 0.f;
+#pragma unroll
+        for (int ks = 0; ks < kWgradK; ++ks) mma_bf16(sum[j], ones, bf[ks][j][0], bf[ks][j][1]);
+        accb[j][0] += sum[j][0];
+        accb[j][1] += sum[j][1];
       }
     }
   }
-  if (mma_warp) {
-    float* out = a.partial + ((size_t)blockIdx.x * 9 + tap) * N * CIN;
+  float* out = a.partial + (size_t)blockIdx.x * (9 * S::kN * CIN + S::kN);
+  const int g = lane >> 2, t2 = 2 * (lane & 3);
 #pragma unroll
-    for (int wm = 0; wm < WM; ++wm)
+  for (int t = 0; t < S::kTaps; ++t) {
+    const int tap = tap0 + t;
+    if (tap > 8) continue;
 #pragma unroll
-      for (int wn = 0; wn < WN; ++wn) {
-        const int k = (mg * WM + wm) * 16 + g, n = (ng * WN + wn) * 8 + 2 * t;
-        out[(size_t)n * CIN + k] = acc[wm][wn][0];
-        out[(size_t)(n + 1) * CIN + k] = acc[wm][wn][1];
-        out[(size_t)n * CIN + k + 8] = acc[wm][wn][2];
-        out[(size_t)(n + 1) * CIN + k + 8] = acc[wm][wn][3];
-      }
+    for (int j = 0; j < NW; ++j) {
+      const int k = mg * 16 + g, n = (nh * NW + j) * 8 + t2;
+      float* o = out + ((size_t)tap * S::kN + n) * CIN + k;
+      o[0] = acc[t][j][0];
+      o[CIN] = acc[t][j][1];
+      o[8] = acc[t][j][2];
+      o[CIN + 8] = acc[t][j][3];
+    }
   }
+  if (bias_warp && g == 0)
+#pragma unroll
+    for (int j = 0; j < NW; ++j) {
+      float* o = out + 9 * S::kN * CIN + (nh * NW + j) * 8 + t2;
+      o[0] = accb[j][0];
+      o[1] = accb[j][1];
+    }
 }
 
-cudaError_t launch_wgrad(int cin, int nt, const WgradArgs& a, cudaStream_t s) {
-  const long total = (long)a.B * a.Ho * a.Wo;
-  const unsigned chunks = (unsigned)((total + a.chunk_pix - 1) / a.chunk_pix);
-  const dim3 grid(chunks, 9);
-  if (cin == 16 && nt == 8) wgrad_kernel<16, 8><<<grid, kWgradThreads, 0, s>>>(a);
-  else if (cin == 64 && nt == 8) wgrad_kernel<64, 8><<<grid, kWgradThreads, 0, s>>>(a);
-  else if (cin == 64 && nt == 1) wgrad_kernel<64, 1><<<grid, kWgradThreads, 0, s>>>(a);
-  else return cudaErrorInvalidValue;
+template <int CIN, int NW, int STRIDE>
+cudaError_t launch_wgrad_t(const WgradArgs& a, int grid, cudaStream_t s) {
+  using S = WgradShape<CIN, NW, STRIDE>;
+  static PerDevice configured;
+  int dummy = 0;
+  const cudaError_t e = per_device(configured, &dummy, [](int, int* v) {
+    *v = 1;
+    return cudaFuncSetAttribute(wgrad_kernel<CIN, NW, STRIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::kSmem);
+  });
+  if (e != cudaSuccess) return e;
+  wgrad_kernel<CIN, NW, STRIDE><<<grid, kWgradThreads, S::kSmem, s>>>(a);
   return cudaGetLastError();
 }
 
-// Sum of the chunk partials in chunk order into the master-layout gradient [3][3][cin][cout]
-// (only the real channels: cin_real, cout_real), one thread per weight; neighbouring threads take
-// neighbouring input channels, which are contiguous in the partials.
-__global__ void wgrad_reduce_kernel(const float* __restrict__ partial, int n_chunks, int N, int CIN, int cin_real,
-                                    int cout_real, float* __restrict__ gw) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  const int per_tap = cin_real * cout_real;
-  if (i >= 9 * per_tap) return;
-  const int tap = i / per_tap, r = i % per_tap, co = r / cin_real, ci = r % cin_real;
+// Sum of the CTAs' partials into the master-layout gradients gw [3][3][cin][cout] and gb [cout] (only
+// the real channels): 32 neighbouring weights per CTA, eight warps taking every eighth partial each,
+// added in a fixed order.
+__global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restrict__ partial, int n_parts, int N, int CIN,
+                                                           int cin_real, int cout_real, float* __restrict__ gw,
+                                                           float* __restrict__ gb) {
+  __shared__ float part[8][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int per_tap = cin_real * cout_real, n_w = 9 * per_tap;
+  const int i = blockIdx.x * 32 + lane;
+  const size_t pitch = (size_t)9 * N * CIN + N;
+  size_t src = 0;
+  float* dst = nullptr;
+  if (i < n_w) {
+    const int tap = i / per_tap, r = i % per_tap, co = r / cin_real, ci = r % cin_real;
+    src = ((size_t)tap * N + co) * CIN + ci;
+    dst = gw + (size_t)tap * per_tap + (size_t)ci * cout_real + co;
+  } else if (i < n_w + cout_real) {
+    src = (size_t)9 * N * CIN + (i - n_w);
+    dst = gb + (i - n_w);
+  }
   float s = 0.f;
-  for (int c = 0; c < n_chunks; ++c) s += partial[(((size_t)c * 9 + tap) * N + co) * CIN + ci];
-  gw[(size_t)tap * per_tap + (size_t)ci * cout_real + co] = s;
-}
-
-// Bias gradient: sum over pixels of g[p, n] in a fixed order: per chunk, 4 pixel groups x the
-// channels (neighbouring threads read neighbouring channels), groups added in order; then the
-// chunks in order.
-constexpr int kBiasGroups = 4;
-
-__global__ void bias_partial_kernel(const bf16* __restrict__ g, long total, int GS, int n_real, int chunk,
-                                    float* __restrict__ partial) {
-  __shared__ float part[kBiasGroups][64];
-  const int n = threadIdx.x & 63, grp = threadIdx.x >> 6;
-  float s = 0.f;
-  const long p0 = (long)blockIdx.x * chunk;
-  if (n < n_real)
-    for (long p = p0 + grp; p < p0 + chunk && p < total; p += kBiasGroups) s += __bfloat162float(g[(size_t)p * GS + n]);
-  part[grp][n] = s;
+  if (dst) {
+#pragma unroll 8
+    for (int c = warp; c < n_parts; c += 8) s += partial[(size_t)c * pitch + src];
+  }
+  part[warp][lane] = s;
   __syncthreads();
-  if (grp == 0 && n < n_real) {
-    float v = part[0][n];
-    for (int q = 1; q < kBiasGroups; ++q) v += part[q][n];
-    partial[(size_t)blockIdx.x * n_real + n] = v;
+  if (warp == 0 && dst) {
+    float v = part[0][lane];
+#pragma unroll
+    for (int w = 1; w < 8; ++w) v += part[w][lane];
+    *dst = v;
   }
 }
 
-__global__ void bias_reduce_kernel(const float* __restrict__ partial, int n_chunks, int n_real, float* __restrict__ gb) {
-  const int n = threadIdx.x;
-  if (n >= n_real) return;
-  float s = 0.f;
-  for (int c = 0; c < n_chunks; ++c) s += partial[(size_t)c * n_real + n];
-  gb[n] = s;
+int wgrad_parts(int cin, int B, int Ho, int Wo) {
+  const long tiles = (long)B * ((Wo + kWgradW - 1) / kWgradW) * ((Ho + kWgradH - 1) / kWgradH);
+  const int most = kWgradCtas * (cin == 16 ? 2 : 1);
+  return (int)(tiles < most ? tiles : most);
 }
 
-cudaError_t launch_bias_grad(const bf16* g, long total, int GS, int n_real, float* scratch, float* gb, cudaStream_t s) {
-  const int chunk = 2048;
-  const int chunks = (int)((total + chunk - 1) / chunk);
-  bias_partial_kernel<<<chunks, 64 * kBiasGroups, 0, s>>>(g, total, GS, n_real, chunk, scratch);
-  bias_reduce_kernel<<<1, 64, 0, s>>>(scratch, chunks, n_real, gb);
-  return cudaGetLastError();
+size_t wgrad_partial_floats(int cin, int cout_pad) {
+  const int n = cout_pad < 16 ? 16 : cout_pad;
+  return (size_t)9 * n * cin + n;
 }
 
-cudaError_t launch_wgrad_reduce(const float* partial, int n_chunks, int N, int CIN, int cin_real, int cout_real,
-                                float* gw, cudaStream_t s) {
-  const int n = 9 * cin_real * cout_real;
-  wgrad_reduce_kernel<<<(n + 255) / 256, 256, 0, s>>>(partial, n_chunks, N, CIN, cin_real, cout_real, gw);
+cudaError_t launch_wgrad(int cin, int cout_pad, const WgradArgs& a, int cin_real, int cout_real, float* gw, float* gb,
+                         cudaStream_t s) {
+  const int parts = wgrad_parts(cin, a.B, a.Ho, a.Wo);
+  if (parts <= 0) return cudaSuccess;
+  cudaError_t e = cudaErrorInvalidValue;
+  if (cin == 16 && cout_pad == 64 && a.stride == 2) e = launch_wgrad_t<16, 4, 2>(a, parts, s);
+  else if (cin == 64 && cout_pad == 64 && a.stride == 2) e = launch_wgrad_t<64, 4, 2>(a, parts, s);
+  else if (cin == 64 && cout_pad == 64 && a.stride == 1) e = launch_wgrad_t<64, 4, 1>(a, parts, s);
+  else if (cin == 64 && cout_pad == 8 && a.stride == 1) e = launch_wgrad_t<64, 1, 1>(a, parts, s);
+  if (e != cudaSuccess) return e;
+  const int n = 9 * cin_real * cout_real + cout_real;
+  wgrad_reduce_kernel<<<(n + 31) / 32, 256, 0, s>>>(a.partial, parts, cout_pad < 16 ? 16 : cout_pad, cin, cin_real, cout_real,
+                                                    gw, gb);
   return cudaGetLastError();
 }
 
@@ -457,14 +515,10 @@ __global__ void input_kernel(const uint16_t* __restrict__ depth, const uint32_t*
                              bf16* __restrict__ x) {
   const long p = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= n_pix) return;
-  // centred and scaled: (depth m - 3) / 2, (colour / 255 - 1/2) x 4
-  const float d = ((float)depth[p] * 0.001f - 3.0f) * 0.5f;
   const uint32_t c = rgba[p];
   __align__(16) bf16 v[16];
-  v[0] = __float2bfloat16(d);
-  v[1] = __float2bfloat16(((float)(c & 0xFF) / 255.f - 0.5f) * 4.0f);
-  v[2] = __float2bfloat16(((float)((c >> 8) & 0xFF) / 255.f - 0.5f) * 4.0f);
-  v[3] = __float2bfloat16(((float)((c >> 16) & 0xFF) / 255.f - 0.5f) * 4.0f);
+  v[0] = input_depth(depth[p]);
+  for (int k = 0; k < 3; ++k) v[1 + k] = input_colour((c >> (8 * k)) & 0xFF);
   for (int k = 4; k < 16; ++k) v[k] = __float2bfloat16(0.f);
   uint4* dst = reinterpret_cast<uint4*>(x + (size_t)p * 16);
   dst[0] = *reinterpret_cast<uint4*>(&v[0]);
@@ -478,10 +532,18 @@ cudaError_t launch_input(const uint16_t* depth, const uint32_t* rgba, long n_pix
 
 
 
-// Targets: scene coordinate of each cell's centre pixel minus the origin; w = 1 if scored.
-__global__ void targets_kernel(CellArgs a, float4* __restrict__ tgt) {
+// Targets: scene coordinate of each cell's centre pixel minus the origin; w = 1 if scored.  The scored
+// cells are counted into *scored (zeroed before).
+__global__ void __launch_bounds__(256) targets_kernel(CellArgs a, float4* __restrict__ tgt, int32_t* __restrict__ scored) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   const int per = a.Wc * a.Hc;
+  bool on = false;
+  if (i < a.n * per) {
+    const int img = i / per, c = i % per;
+    on = a.depth[((size_t)img * a.H + c / a.Wc * 8 + 4) * a.W + c % a.Wc * 8 + 4] != 0;
+  }
+  const int count = __syncthreads_count(on);
+  if (threadIdx.x == 0 && count) atomicAdd(scored, count);
   if (i >= a.n * per) return;
   const int img = i / per, c = i % per, cx = c % a.Wc, cy = c / a.Wc;
   const int u = cx * 8 + 4, v = cy * 8 + 4;
@@ -499,42 +561,38 @@ __global__ void targets_kernel(CellArgs a, float4* __restrict__ tgt) {
   tgt[i] = make_float4((float)y0, (float)y1, (float)y2, 1.f);
 }
 
-cudaError_t launch_targets(const CellArgs& a, float4* tgt, cudaStream_t s) {
+cudaError_t launch_targets(const CellArgs& a, float4* tgt, int32_t* counters, cudaStream_t s) {
   const int n = a.n * a.Wc * a.Hc;
-  targets_kernel<<<(n + 255) / 256, 256, 0, s>>>(a, tgt);
+  const cudaError_t e = cudaMemsetAsync(counters, 0, 2 * sizeof(int32_t), s);
+  if (e != cudaSuccess) return e;
+  targets_kernel<<<(n + 255) / 256, 256, 0, s>>>(a, tgt, counters);
   return cudaGetLastError();
 }
 
 // Loss and its gradient with respect to the head output (stored [cell][8] FP32), written as the
-// BF16 gradient [cell][16] (channels 4..15 zero).  One CTA: scored cells are counted first so
-// the mean and the summation order are fixed.
-__global__ void __launch_bounds__(1024) loss_kernel(const float* __restrict__ out, const float4* __restrict__ tgt,
-                                                     int n_cells, bf16* __restrict__ grad, float* __restrict__ loss) {
-  __shared__ float red[32];
-  __shared__ int redi[32];
-  __shared__ float s_inv;
-  int cnt = 0;
-  for (int i = threadIdx.x; i < n_cells; i += blockDim.x) cnt += tgt[i].w > 0.5f;
-  cnt = warp_sum_i(cnt);
-  if ((threadIdx.x & 31) == 0) redi[threadIdx.x >> 5] = cnt;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int c = 0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) c += redi[w];
-    s_inv = 1.0f / (float)(c > 0 ? c : 1);
-  }
-  __syncthreads();
-  const float inv = s_inv;
+// BF16 gradient [cell][16] (channels 4..15 zero).  counters: [0] scored cells (targets_kernel), [1]
+// CTAs done.  Each CTA leaves its sum; the last one to finish adds them in order, so the loss does not
+// depend on scheduling (one CTA over all cells took 118 us for 16 views).
+constexpr int kLossThreads = 256;
+__global__ void __launch_bounds__(kLossThreads) loss_kernel(const float* __restrict__ out, const float4* __restrict__ tgt,
+                                                            int n_cells, bf16* __restrict__ grad,
+                                                            int32_t* __restrict__ counters, float* __restrict__ sums,
+                                                            float* __restrict__ loss) {
+  __shared__ float red[kLossThreads / 32];
+  __shared__ int s_last;
+  const int scored = counters[0];
+  const float inv = 1.0f / (float)(scored > 0 ? scored : 1);
   float acc = 0.f;
-  for (int i = threadIdx.x; i < n_cells; i += blockDim.x) {
+  const int i = blockIdx.x * kLossThreads + threadIdx.x;
+  if (i < n_cells) {
     const float4 y = tgt[i];
-    const float* o = out + (size_t)i * 8;
+    const float4 o = *reinterpret_cast<const float4*>(out + (size_t)i * 8);
     __align__(16) bf16 gv[16];
     for (int k = 0; k < 16; ++k) gv[k] = __float2bfloat16(0.f);
     if (y.w > 0.5f) {
       // rho(e) + 1/2 e^2 exp(-s) + 3/2 s, rho(e) = sqrt(e^2 + 1e-6): the coordinates follow d rho,
       // s the NLL's derivative with the error held fixed
-      const float e0 = o[0] - y.x, e1 = o[1] - y.y, e2 = o[2] - y.z, s = o[3];
+      const float e0 = o.x - y.x, e1 = o.y - y.y, e2 = o.z - y.z, s = o.w;
       const float sq = e0 * e0 + e1 * e1 + e2 * e2, es = expf(-s), rho = sqrtf(sq + 1e-6f);
       acc += rho + 0.5f * sq * es + 1.5f * s;
       const float gc = inv / rho;
@@ -552,32 +610,65 @@ __global__ void __launch_bounds__(1024) loss_kernel(const float* __restrict__ ou
   __syncthreads();
   if (threadIdx.x == 0) {
     float s = 0.f;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += red[w];
-    *loss = s * inv;
+    for (int w = 0; w < kLossThreads / 32; ++w) s += red[w];
+    sums[blockIdx.x] = s;
+    __threadfence();
+    s_last = atomicAdd(&counters[1], 1) == (int)gridDim.x - 1;
   }
+  __syncthreads();
+  if (!s_last || threadIdx.x >= 32) return;
+  __threadfence();
+  float s = 0.f;
+  for (int c = threadIdx.x; c < (int)gridDim.x; c += 32) s += __ldcg(&sums[c]);
+  s = warp_sum(s);
+  if (threadIdx.x == 0) *loss = s * inv;
 }
 
-cudaError_t launch_loss(const float* out, const float4* tgt, int n_cells, bf16* grad, float* loss, cudaStream_t s) {
-  loss_kernel<<<1, 1024, 0, s>>>(out, tgt, n_cells, grad, loss);
+int loss_blocks(int n_cells) { return (n_cells + kLossThreads - 1) / kLossThreads; }
+
+cudaError_t launch_loss(const float* out, const float4* tgt, int n_cells, bf16* grad, int32_t* counters, float* sums,
+                        float* loss, cudaStream_t s) {
+  loss_kernel<<<loss_blocks(n_cells), kLossThreads, 0, s>>>(out, tgt, n_cells, grad, counters, sums, loss);
   return cudaGetLastError();
 }
 
-__global__ void adam_kernel(float* __restrict__ p, const float* __restrict__ g, float* __restrict__ m,
-                            float* __restrict__ v, long n, float lr, float b1, float b2, float eps, float c1, float c2) {
-  const long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float gi = g[i];
-  const float mi = b1 * m[i] + (1.f - b1) * gi;
-  const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-  m[i] = mi;
-  v[i] = vi;
-  p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+// One Adam step of every parameter, and the BF16 weights and padded biases that the convolutions
+// read (their padding stays as launch_pack left it): one launch instead of an update and 23 small
+// packing launches (65 us a step).
+constexpr int kCinFirst = kRegCin[0], kCinFirstPad = kRegCinPad[0];
+constexpr int kCoutHead = kRegCout[kRegLayers - 1], kCoutHeadPad = kRegCoutPad[kRegLayers - 1];
+__global__ void __launch_bounds__(256) adam_kernel(AdamArgs a, float lr, float b1, float b2, float eps, float c1, float c2) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= a.n) return;
+  const float gi = a.g[i];
+  const float mi = b1 * a.m[i] + (1.f - b1) * gi;
+  const float vi = b2 * a.v[i] + (1.f - b2) * gi * gi;
+  a.m[i] = mi;
+  a.v[i] = vi;
+  float p = a.p[i];
+  p -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  a.p[i] = p;
+  int l = 0;
+#pragma unroll
+  for (int k = 1; k < kRegLayers; ++k) l += i >= a.w_off[k];
+  const int cin = l == 0 ? kCinFirst : 64, cout = l == kRegLayers - 1 ? kCoutHead : 64;
+  const int cin_pad = l == 0 ? kCinFirstPad : 64, cout_pad = l == kRegLayers - 1 ? kCoutHeadPad : 64;
+  const int r = i - a.w_off[l];
+  if (r >= 9 * cin * cout) {
+    a.bias[l][r - 9 * cin * cout] = p;
+    return;
+  }
+  const int tap = r / (cin * cout), k = r / cout % cin, n = r % cout;
+  const bf16 w = __float2bfloat16(p);
+  a.wk[l][((size_t)tap * cout_pad + n) * cin_pad + k] = w;
+  const int pad_t = l == kRegLayers - 1 ? 16 : 64;
+  if (l > 0) a.wt[l][((size_t)(8 - tap) * cin + k) * pad_t + n] = w;
 }
 
-cudaError_t launch_adam(float* p, const float* g, float* m, float* v, long n, float lr, int t, cudaStream_t s) {
+cudaError_t launch_adam(const AdamArgs& a, float lr, int t, cudaStream_t s) {
   const float b1 = 0.9f, b2 = 0.999f;
   const float c1 = 1.f - powf(b1, (float)t), c2 = 1.f - powf(b2, (float)t);
-  adam_kernel<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(p, g, m, v, n, lr, b1, b2, 1e-8f, c1, c2);
+  adam_kernel<<<(unsigned)((a.n + 255) / 256), 256, 0, s>>>(a, lr, b1, b2, 1e-8f, c1, c2);
   return cudaGetLastError();
 }
 

@@ -26,13 +26,12 @@ struct ConvArgs {
   int relu, upsample;
 };
 
-// Backward-weight partial sums (see wgrad_kernel)
+// Backward-weight sums (see wgrad_kernel)
 struct WgradArgs {
   const bf16* in;     // layer input [B][Hi][Wi][CIN]
   const bf16* g;      // gradient of the pre-activation output [B][Ho][Wo][GS] (first N channels used)
-  float* partial;     // [n_chunks][9][N][CIN]
+  float* partial;     // [wgrad_parts][wgrad_partial_floats]
   int B, Hi, Wi, Ho, Wo, stride, GS;
-  int chunk_pix;      // multiple of 64
 };
 
 // Targets (see targets_kernel)
@@ -58,25 +57,45 @@ struct CellForestArgs {
   uint16_t* depth_lr;      // [n][Hc][Wc]
 };
 
+// The network's input per pixel: centred and scaled depth, (depth m - 3) / 2, and colour channels,
+// (c / 255 - 1/2) x 4.
+__device__ __forceinline__ bf16 input_depth(uint32_t mm) { return __float2bfloat16(((float)mm * 0.001f - 3.0f) * 0.5f); }
+__device__ __forceinline__ bf16 input_colour(uint32_t c) { return __float2bfloat16(((float)c / 255.f - 0.5f) * 4.0f); }
+
 constexpr int kRegLayers = 8;
 constexpr int kRegStride[kRegLayers] = {2, 2, 2, 1, 1, 1, 1, 1};
 constexpr int kRegCin[kRegLayers] = {4, 64, 64, 64, 64, 64, 64, 64};
 constexpr int kRegCout[kRegLayers] = {64, 64, 64, 64, 64, 64, 64, 4};
 constexpr int kRegCinPad[kRegLayers] = {16, 64, 64, 64, 64, 64, 64, 64};
 constexpr int kRegCoutPad[kRegLayers] = {64, 64, 64, 64, 64, 64, 64, 8};
-constexpr int kWgradChunk = 1024;  // output pixels per backward-weight CTA (multiple of 64)
+constexpr int kWgradCtas = 152;  // most CTAs (partial sums per weight) of a backward-weight launch; 16 channels: twice that
+
+// Adam step of all parameters and the operands derived from them (see adam_kernel)
+struct AdamArgs {
+  float *p, *m, *v;
+  const float* g;
+  int n;
+  int w_off[kRegLayers];   // first weight of each layer; its biases follow its weights
+  bf16* wk[kRegLayers];
+  bf16* wt[kRegLayers];
+  float* bias[kRegLayers];
+};
 
 cudaError_t launch_conv(int cin, int nt, const ConvArgs& a, int n_sms, cudaStream_t s);
-cudaError_t launch_wgrad(int cin, int nt, const WgradArgs& a, cudaStream_t s);
-cudaError_t launch_wgrad_reduce(const float* partial, int n_chunks, int N, int CIN, int cin_real, int cout_real,
-                                float* gw, cudaStream_t s);
-cudaError_t launch_bias_grad(const bf16* g, long total, int GS, int n_real, float* scratch, float* gb, cudaStream_t s);
+// Gradients gw [3][3][cin_real][cout_real] and gb [cout_real] of a layer.
+int wgrad_parts(int cin, int B, int Ho, int Wo);
+size_t wgrad_partial_floats(int cin, int cout_pad);
+cudaError_t launch_wgrad(int cin, int cout_pad, const WgradArgs& a, int cin_real, int cout_real, float* gw, float* gb,
+                         cudaStream_t s);
 cudaError_t launch_pack(const float* w, int cin, int cout, int cin_pad, int cout_pad, bf16* wk, bf16* wt,
                         int cout_pad_t, cudaStream_t s);
 cudaError_t launch_input(const uint16_t* depth, const uint32_t* rgba, long n_pix, bf16* x, cudaStream_t s);
-cudaError_t launch_targets(const CellArgs& a, float4* tgt, cudaStream_t s);
-cudaError_t launch_loss(const float* out, const float4* tgt, int n_cells, bf16* grad, float* loss, cudaStream_t s);
-cudaError_t launch_adam(float* p, const float* g, float* m, float* v, long n, float lr, int t, cudaStream_t s);
+// counters (2 words): [0] receives the scored cells, [1] is zeroed for launch_loss
+cudaError_t launch_targets(const CellArgs& a, float4* tgt, int32_t* counters, cudaStream_t s);
+int loss_blocks(int n_cells);  // floats of launch_loss's sums
+cudaError_t launch_loss(const float* out, const float4* tgt, int n_cells, bf16* grad, int32_t* counters, float* sums,
+                        float* loss, cudaStream_t s);
+cudaError_t launch_adam(const AdamArgs& a, float lr, int t, cudaStream_t s);
 cudaError_t launch_cell_forest(const CellForestArgs& a, cudaStream_t s);
 
 // Forward 3x3 convolution of a cin -> 64-channel layer (cin 16 or 64) on the tcgen05 tensor cores
@@ -87,6 +106,17 @@ cudaError_t launch_cell_forest(const CellForestArgs& a, cudaStream_t s);
 cudaError_t launch_conv_tc(int cin, const bf16* in, int B, int Hi, int Wi, const bf16* w, const float* bias,
                            const bf16* mask, bf16* out, int Ho, int Wo, int stride, int dil, int relu, int32_t* status,
                            int n_sms, cudaStream_t s, unsigned long long timeout_ns, int stall_tile);
+// The first layer from the images (depth [B][H][W] mm, rgba): w [9][64][16], out [B][Ho][Wo][64], ReLU.
+cudaError_t launch_conv_first(const uint16_t* depth, const uint32_t* rgba, int B, int H, int W, const bf16* w,
+                              const float* bias, bf16* out, int Ho, int Wo, int32_t* status, int n_sms, cudaStream_t s,
+                              unsigned long long timeout_ns, int stall_tile);
+// Backward-data of a stride-2 layer: g [B][Hg][Wg][64], w [9][64][64] flipped and transposed, mask and out
+// [B][2 Hg][2 Wg][64].
+cudaError_t launch_conv_up(const bf16* g, int B, int Hg, int Wg, const bf16* w, const bf16* mask, bf16* out, int32_t* status,
+                           int n_sms, cudaStream_t s, unsigned long long timeout_ns, int stall_tile);
+// The head: 64 -> 8 channels (w [9][8][64], bias [8]), stride 1, FP32 out [B][H][W][8].
+cudaError_t launch_conv_head(const bf16* in, int B, int H, int W, const bf16* w, const float* bias, float* out,
+                             int32_t* status, int n_sms, cudaStream_t s, unsigned long long timeout_ns, int stall_tile);
 cudaError_t launch_head_copy(const float* head, long n_cells, float* out4, cudaStream_t s);
 
 }  // namespace relo
