@@ -2393,7 +2393,8 @@ relo_status issue_batch(relo_batch* b, relo_pose_result* results, cudaStream_t s
   RELO_CUDA(cudaMemsetAsync(b->d_errs, 0, (b->nL + b->nF + 1) * sizeof(int32_t), s));
   RELO_CUDA(launch_init_results(b->d_res_F, b->n, s));
   RELO_CUDA(mark(b, 0, s, capturing));
-  RELO_CUDA(launch_raycast(b->d_query, b->n, nullptr, b->query_tiles, true, false, s, b->sched, b->query_mode));
+  RELO_CUDA(launch_raycast(b->d_query, b->n, nullptr, b->query_tiles, true, false, s, b->sched, b->query_mode,
+                           true));
   L += 2;
   RELO_CUDA(mark(b, 1, s, capturing));
   // pass L: learned attempts

@@ -479,10 +479,11 @@ inline int forest_job_tiles(int W, int H) { return ((W + 31) / 32) * ((H + 7) / 
 inline size_t tiled_values(int W, int H) { return (size_t)((W + 7) / 8) * ((H + 7) / 8) * 256; }
 
 // jobs_dev == nullptr: the single job is passed by value.  mode: the scene_mode that all scenes of
-// jobs_dev share, or kSceneAny (a single job's own scene decides for itself).
+// jobs_dev share, or kSceneAny (a single job's own scene decides for itself).  tiled: jobs have tiled
+// images to write (RayJob::tiled), which the launch ignores otherwise.
 cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* single, int total_tiles,
                            bool with_colour, bool compare, cudaStream_t s, const Schedule& sched = Schedule(),
-                           int mode = kSceneAny);
+                           int mode = kSceneAny, bool tiled = false);
 // n jobs (host array, tile_begin ascending from 0), forest_launches(n) launches.
 inline int forest_launches(int n) { return (n + kMaxForestJobs - 1) / kMaxForestJobs; }
 cudaError_t launch_forest(const ForestJob* jobs, int n, cudaStream_t s, const Schedule& sched = Schedule());

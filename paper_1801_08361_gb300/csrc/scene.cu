@@ -9,6 +9,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include <cmath>
 #include <vector>
 
@@ -269,8 +271,13 @@ constexpr int kTile = 16;
 #define RELO_RAYCAST_COLOUR_MIN_BLOCKS 6
 #endif
 
-template <bool kColour, bool kCompare, int kMode>
-__global__ void __launch_bounds__(kTile* kTile, kMode == kSceneCells ? 5 : kColour ? RELO_RAYCAST_COLOUR_MIN_BLOCKS : RELO_RAYCAST_MIN_BLOCKS)
+// kFew: launches of at most kFewTiles CTAs an SM, which are resident together however many registers a
+// thread takes: 64 of them, so nothing spills in the march, whose latency such a launch waits for.
+// A house view of 300 x 220 (266 CTAs): 73 us for the call, 75 with the spills.
+constexpr int kFewTiles = 4;
+
+template <bool kColour, bool kCompare, bool kTiled, int kMode, bool kFew>
+__global__ void __launch_bounds__(kTile* kTile, kFew ? kFewTiles : kMode == kSceneCells ? 5 : kColour ? RELO_RAYCAST_COLOUR_MIN_BLOCKS : RELO_RAYCAST_MIN_BLOCKS)
     raycast_kernel(const RayJob* __restrict__ jobs, int n_jobs, const RayJob single, int warp_log2w) {
   // locate the job owning this tile (jobs are few; binary search on tile_begin)
   int lo = 0, hi = n_jobs - 1;
@@ -343,7 +350,7 @@ __global__ void __launch_bounds__(kTile* kTile, kMode == kSceneCells ? 5 : kColo
     }
     if (job.depth) job.depth[pix] = (uint16_t)depth_mm;
     if (kColour && job.rgba) job.rgba[pix] = col;
-    if (kColour && job.tiled) {
+    if (kTiled && job.tiled) {
       uint16_t* t = job.tiled + ((size_t)(v >> 3) * ((job.W + 7) >> 3) + (u >> 3)) * 256 + (v & 7) * 8 + (u & 7);
       t[0] = (uint16_t)depth_mm;
       t[64] = (uint16_t)(col & 0xFFu);
@@ -390,17 +397,18 @@ __global__ void __launch_bounds__(kTile* kTile, kMode == kSceneCells ? 5 : kColo
   }
 }
 
-template <int kMode>
+template <int kMode, bool kFew>
 void launch_raycast_t(const RayJob* jobs_dev, int n_jobs, const RayJob& one, int total_tiles, bool with_colour,
-                      bool compare, cudaStream_t s, int w) {
+                      bool tiled, bool compare, cudaStream_t s, int w) {
   const dim3 grid(total_tiles), block(kTile * kTile);
-  if (compare) raycast_kernel<false, true, kMode><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
-  else if (with_colour) raycast_kernel<true, false, kMode><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
-  else raycast_kernel<false, false, kMode><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
+  if (compare) raycast_kernel<false, true, false, kMode, kFew><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
+  else if (with_colour && tiled) raycast_kernel<true, false, true, kMode, kFew><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
+  else if (with_colour) raycast_kernel<true, false, false, kMode, kFew><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
+  else raycast_kernel<false, false, false, kMode, kFew><<<grid, block, 0, s>>>(jobs_dev, n_jobs, one, w);
 }
 
 cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* single, int total_tiles,
-                           bool with_colour, bool compare, cudaStream_t s, const Schedule& sched, int mode) {
+                           bool with_colour, bool compare, cudaStream_t s, const Schedule& sched, int mode, bool tiled) {
   if (total_tiles <= 0) return cudaSuccess;
   if (sched.ray_warp_log2w < 1 || sched.ray_warp_log2w > 4) return cudaErrorInvalidValue;
   RayJob one{};
@@ -408,9 +416,17 @@ cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* sin
   // a single job's own scene decides; a job array's scenes were looked over by the caller
   if (single) mode = scene_mode(one.scene);
   const int w = sched.ray_warp_log2w;
-  if (mode == kSceneApron) launch_raycast_t<kSceneApron>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, w);
-  else if (mode == kSceneCells) launch_raycast_t<kSceneCells>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, w);
-  else launch_raycast_t<kSceneAny>(jobs_dev, n_jobs, one, total_tiles, with_colour, compare, s, w);
+  int sms = 0;
+  const cudaError_t e = device_sms(&sms);
+  if (e != cudaSuccess) return e;
+  auto launch = [&](auto few) {
+    constexpr bool kFew = decltype(few)::value;
+    if (mode == kSceneApron) launch_raycast_t<kSceneApron, kFew>(jobs_dev, n_jobs, one, total_tiles, with_colour, tiled, compare, s, w);
+    else if (mode == kSceneCells) launch_raycast_t<kSceneCells, kFew>(jobs_dev, n_jobs, one, total_tiles, with_colour, tiled, compare, s, w);
+    else launch_raycast_t<kSceneAny, kFew>(jobs_dev, n_jobs, one, total_tiles, with_colour, tiled, compare, s, w);
+  };
+  if (total_tiles <= kFewTiles * sms) launch(std::true_type{});
+  else launch(std::false_type{});
   return cudaGetLastError();
 }
 
