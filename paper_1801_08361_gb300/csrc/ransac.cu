@@ -80,14 +80,17 @@ __device__ __forceinline__ void cam_point_d(int u, int v, int d, double fx, doub
 }
 
 // ---------------------------------------------------------------------------------------------
-// horn_pose (relo_internal.cuh) by 16 lanes, two solves per warp: lane 4 i + j of a half-warp holds
-// entries (i, j) of A and V.  The FP64 pipe takes many cycles per warp instruction however few lanes
-// are active, so one thread's solve (about 700 FP64 instructions a sweep) is bound by that pipe's
-// latency: 84-105 us whether one hypothesis or two thousand are re-fitted.  Sharing the entries among
-// lanes leaves about 200 a sweep, most of them the two rotations' angles, which both halves of the
-// columns take at once.  Every entry goes through horn_pose's operations in its order and rounding,
-// so both forms give the same bits.  Used where a launch has at most kGroupSolves solves; beyond,
-// the 32 solves a warp of the other form advances per instruction win.
+// horn_pose (relo_internal.cuh) by 16 lanes, two solves per warp.  Every lane of a group runs
+// horn_refined on the same matrix (a warp's instruction costs the same for 2 lanes and 32); where a group
+// has to take the FP64 rotations, lane 4 i + j of it holds entries (i, j) of A and V.  The FP64 pipe
+// takes many cycles per warp instruction however few lanes are active, so one thread's rotations (about
+// 700 FP64 instructions a sweep) are bound by that pipe's latency: 84-105 us whether one hypothesis or two
+// thousand are re-fitted.  Sharing the entries among lanes leaves about 200 a sweep, most of them the two
+// rotations' angles, which both halves of the columns take at once.  Every entry goes through
+// horn_jacobi's operations in its order and rounding, so both forms give the same bits.  Used where a
+// launch has at most kGroupSolves solves; beyond, the 32 solves a warp of the other form advances per
+// instruction win.  A house frame's re-fit: 95 us a round by single threads, 35 with the rotations
+// shared, 18 now.
 // ---------------------------------------------------------------------------------------------
 #ifndef RELO_GROUP_SOLVES
 #define RELO_GROUP_SOLVES 2048
@@ -106,6 +109,12 @@ __device__ __forceinline__ void horn_pose_group(double S_lane, const double cbar
   double S[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) S[k] = group_get(S_lane, k);
+  double q[4];
+  if (active && horn_refined(S, q)) {
+    if (l == 0) quaternion_pose(q[0], q[1], q[2], q[3], cbar, wbar, out);
+    active = false;
+  }
+  if (!__any_sync(0xffffffffu, active)) return;
   const double Sxx = S[0], Sxy = S[1], Sxz = S[2], Syx = S[3], Syy = S[4], Syz = S[5], Szx = S[6], Szy = S[7],
                Szz = S[8];
   double A, V = i == j ? 1.0 : 0.0;
@@ -162,7 +171,7 @@ __device__ __forceinline__ void horn_pose_group(double S_lane, const double cbar
         const double x = first ? mine : other, y = first ? other : mine;
         return __fma_rn(first ? cc : ss, x, __dmul_rn(first ? -ss : cc, y));
       };
-      // horn_pose rotates pair 0's columns, its rows, then pair 1's columns and rows: entries in
+      // horn_jacobi rotates pair 0's columns, its rows, then pair 1's columns and rows: entries in
       // pair 0's rows and pair 1's columns see the row rotation first, all others the column's
       const bool row_first = i0 && !j0;
       double other = group_get(A, row_first ? 4 * ip + j : 4 * i + jp);
@@ -1418,7 +1427,15 @@ cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int
   select_kernel<<<n_jobs, std::min(npow, 1024), (size_t)npow * (sizeof(unsigned long long) + sizeof(int)), s>>>(
       jobs, alive_prefix_dev, round);
   const int parts = ((round + 1) * B + kRefinePixels - 1) / kRefinePixels;
-  switch (group_log2(max_surv)) {
+  int n_sms = 0;
+  const cudaError_t e = device_sms(&n_sms);
+  if (e != cudaSuccess) return e;
+  // Few survivors in all: a hypothesis is shared by more lanes, up to sixteen, while the CTAs leave SMs
+  // idle (a house frame's first round: 16 chunks of 32 survivors, one part of 64 pixels).  Re-fit sums of a
+  // frame's ten rounds: 320 -> 275 us; batches of 32 attempts and more keep one survivor a lane.
+  int lg = group_log2(max_surv);
+  while (lg < 4 && (long)((max_surv + (32 >> lg) - 1) / (32 >> lg)) * parts * n_jobs < 2 * n_sms) ++lg;
+  switch (lg) {
     case 0: launch_refine<0>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
     case 1: launch_refine<1>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
     case 2: launch_refine<2>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
@@ -1426,9 +1443,6 @@ cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int
     case 4: launch_refine<4>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
     default: launch_refine<5>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
   }
-  int n_sms = 0;
-  const cudaError_t e = device_sms(&n_sms);
-  if (e != cudaSuccess) return e;
   if (sched.refit_per == 0 && total_surv <= kGroupSolves) {
     refit_group_kernel<<<(unsigned)((total_surv + kSolvesPerWarp - 1) / kSolvesPerWarp), 32, 0, s>>>(
         jobs, n_jobs, surv_prefix_dev, total_surv, round);
@@ -1445,6 +1459,7 @@ cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int
 // summed by the 32 lanes of a warp; every lane returns the total.
 __device__ __forceinline__ unsigned long long job_tries(const RansacJob& job, int lane) {
   unsigned long long tries = 0;
+#pragma unroll 8
   for (int q = lane; q < job.K; q += 32)
     tries += job.hyp_ok[q] ? (unsigned long long)job.tries[q] + 1 : job.max_tries;
 #pragma unroll

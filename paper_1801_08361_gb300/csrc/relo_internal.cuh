@@ -212,7 +212,7 @@ __device__ __forceinline__ float3 apply(const PoseF& P, float3 c) {
 }
 
 // Pose [R | t] (12 doubles) of the rotation (w, x, y, z), normalised here, that maps centroid cbar to
-// wbar.  Every operation states its rounding, here and in horn_pose, so that both forms of the solve
+// wbar.  Every operation states its rounding, here and in the solves, so that both forms of a solve
 // (horn_pose by a thread, horn_pose_group by 16 lanes) give the same bits.
 __device__ __forceinline__ void quaternion_pose(double w, double x, double y, double z, const double cbar[3],
                                                 const double wbar[3], double* out) {
@@ -238,9 +238,145 @@ __device__ __forceinline__ void quaternion_pose(double w, double x, double y, do
 
 // Rigid transform from centroids and cross-covariance by Horn's closed form (1987): the rotation is
 // the unit quaternion of the largest eigenvalue of the symmetric 4x4 matrix N(S), S = sum of
-// (c - cbar)(w - wbar)^T.  The eigenproblem is solved by cyclic Jacobi rotations in FP64, which
-// keeps the decomposition stable for near-degenerate point sets.  Writes 12 doubles [R | t].
-__device__ inline void horn_pose(const double S[9], const double cbar[3], const double wbar[3], double* out) {
+// (c - cbar)(w - wbar)^T.  horn_refined solves the eigenproblem where the largest eigenvalue stands
+// clear of the others, horn_jacobi, by cyclic Jacobi rotations in FP64 (stable for near-degenerate point
+// sets), where it does not.
+
+// The largest eigenvalue's eigenvector (near unit length) by FP32 Jacobi rotations and refinement in
+// FP64: with approximate eigenvectors v_k and eigenvalues l_k, the residual r = N q - rho q in FP64
+// gives the correction sum of v_k (v_k . r) / (l_max - l_k), which FP32 suffices for (iterative
+// refinement; the first-order perturbation of an eigenvector).  Each turn leaves about kappa = 4e-7 / gap
+// of the error, so two are usual, and what remains is the residual's own rounding: that of FP64
+// rotations.  About 100 FP64 operations where the rotations take 700 a sweep and five sweeps, on a pipe
+// that takes 16 cycles or more a warp.  False (the caller takes horn_jacobi): a relative gap under 5e-4
+// (beyond, the residual's rounding would pass for a step; about one in a thousand random triples),
+// no convergence, or entries FP32 cannot hold (zeros, infinities, NaN).
+__device__ __forceinline__ bool horn_refined(const double S_in[9], double (&q)[4]) {
+  int top = 0;
+#pragma unroll
+  for (int k = 0; k < 9; ++k) top = max(top, __double2hiint(S_in[k]) & 0x7FFFFFFF);
+  const int e = top >> 20;  // biased exponent of the largest entry
+  if (e < 64 || e > 1980) return false;
+  const double scale = __hiloint2double((2046 - e) << 20, 0);  // 2^(1023 - e): exact
+  double S[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) S[k] = __dmul_rn(S_in[k], scale);
+  double N[4][4];
+  N[0][0] = __dadd_rn(__dadd_rn(S[0], S[4]), S[8]);
+  N[1][1] = __dsub_rn(__dsub_rn(S[0], S[4]), S[8]);
+  N[2][2] = __dsub_rn(__dsub_rn(S[4], S[0]), S[8]);
+  N[3][3] = __dsub_rn(__dsub_rn(S[8], S[0]), S[4]);
+  N[0][1] = N[1][0] = __dsub_rn(S[5], S[7]);
+  N[0][2] = N[2][0] = __dsub_rn(S[6], S[2]);
+  N[0][3] = N[3][0] = __dsub_rn(S[1], S[3]);
+  N[1][2] = N[2][1] = __dadd_rn(S[1], S[3]);
+  N[1][3] = N[3][1] = __dadd_rn(S[6], S[2]);
+  N[2][3] = N[3][2] = __dadd_rn(S[5], S[7]);
+  float d[4], o[6], V[4][4];  // diagonal; (0,1) (0,2) (0,3) (1,2) (1,3) (2,3); columns: eigenvectors
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    d[i] = (float)N[i][i];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) V[i][j] = i == j ? 1.f : 0.f;
+  }
+  o[0] = (float)N[0][1], o[1] = (float)N[0][2], o[2] = (float)N[0][3];
+  o[3] = (float)N[1][2], o[4] = (float)N[1][3], o[5] = (float)N[2][3];
+  // (x, y) <- (c x - s y, s x + c y)
+  auto rotate = [](float& x, float& y, float c, float s) {
+    const float a = __fmaf_rn(c, x, -__fmul_rn(s, y));
+    y = __fmaf_rn(s, x, __fmul_rn(c, y));
+    x = a;
+  };
+  auto angle = [](float& dp, float& dq, float& apq, float& c, float& s) {
+    c = 1.f, s = 0.f;
+    if (fabsf(apq) < 1e-30f) return;
+    const float theta = __fdividef(__fsub_rn(dq, dp), __fmul_rn(2.f, apq));
+    const float t = __fdividef(theta >= 0.f ? 1.f : -1.f, __fadd_rn(fabsf(theta), __fsqrt_rn(__fmaf_rn(theta, theta, 1.f))));
+    c = rsqrtf(__fmaf_rn(t, t, 1.f));
+    s = __fmul_rn(t, c);
+    dp = __fmaf_rn(-t, apq, dp);
+    dq = __fmaf_rn(t, apq, dq);
+    apq = 0.f;
+  };
+  // disjoint pairs (p, q), (r, s) and the entries between them
+  auto stage = [&](int p, int q_, int r, int s_, float& apq, float& ars, float& bpr, float& bps, float& bqr, float& bqs) {
+    float c1, s1, c2, s2;
+    angle(d[p], d[q_], apq, c1, s1);
+    angle(d[r], d[s_], ars, c2, s2);
+    rotate(bpr, bqr, c1, s1);
+    rotate(bps, bqs, c1, s1);
+    rotate(bpr, bps, c2, s2);
+    rotate(bqr, bqs, c2, s2);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      rotate(V[k][p], V[k][q_], c1, s1);
+      rotate(V[k][r], V[k][s_], c2, s2);
+    }
+  };
+  for (int sweep = 0; sweep < 10; ++sweep) {
+    float off = 0.f, diag = 0.f;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) off = __fmaf_rn(o[k], o[k], off);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) diag = __fmaf_rn(d[k], d[k], diag);
+    if (off <= __fmul_rn(1e-13f, diag)) break;
+    stage(0, 1, 2, 3, o[0], o[5], o[1], o[2], o[3], o[4]);
+    stage(0, 2, 1, 3, o[1], o[4], o[0], o[2], o[3], o[5]);
+    stage(0, 3, 1, 2, o[2], o[3], o[0], o[1], o[4], o[5]);
+  }
+  float best = d[0], size = fabsf(d[0]);
+  float b[4] = {V[0][0], V[1][0], V[2][0], V[3][0]};
+  int at = 0;
+#pragma unroll
+  for (int k = 1; k < 4; ++k) {
+    size = fmaxf(size, fabsf(d[k]));
+    if (d[k] > best) {
+      best = d[k];
+      at = k;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) b[i] = V[i][k];
+    }
+  }
+  float gap = INFINITY, inv[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float g = __fsub_rn(best, d[k]);
+    if (k != at) gap = fminf(gap, g);
+    inv[k] = k != at ? __fdividef(1.f, g) : 0.f;
+  }
+  if (!(gap > __fmul_rn(5e-4f, size))) return false;
+  const float kappa = __fdividef(__fmul_rn(4e-7f, size), gap);
+#pragma unroll
+  for (int i = 0; i < 4; ++i) q[i] = (double)b[i];
+  for (int it = 0; it < 6; ++it) {
+    double y[4], nn = 0.0, rho = 0.0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      y[i] = __fma_rn(N[i][3], q[3], __fma_rn(N[i][2], q[2], __fma_rn(N[i][1], q[1], __dmul_rn(N[i][0], q[0]))));
+      nn = __fma_rn(q[i], q[i], nn);
+      rho = __fma_rn(q[i], y[i], rho);
+    }
+    const double t = __dsub_rn(2.0, nn);  // rho / nn by two Newton steps: nn is 1 + (an error of q)^2
+    rho = __dmul_rn(rho, __dmul_rn(t, __fma_rn(-nn, t, 2.0)));
+    float r[4], c[4], s2 = 0.f;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) r[i] = (float)__fma_rn(-rho, q[i], y[i]);
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      const float dot = __fmaf_rn(V[3][k], r[3], __fmaf_rn(V[2][k], r[2], __fmaf_rn(V[1][k], r[1], __fmul_rn(V[0][k], r[0]))));
+      c[k] = __fmul_rn(dot, inv[k]);
+      s2 = __fmaf_rn(c[k], c[k], s2);
+    }
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      q[i] = __dadd_rn(q[i], (double)__fmaf_rn(V[i][3], c[3], __fmaf_rn(V[i][2], c[2], __fmaf_rn(V[i][1], c[1], __fmul_rn(V[i][0], c[0])))));
+    const float step = __fsqrt_rn(s2);
+    if (__fmul_rn(__fadd_rn(kappa, step), step) <= 1e-16f) return true;
+  }
+  return false;
+}
+
+__device__ inline void horn_jacobi(const double S[9], const double cbar[3], const double wbar[3], double* out) {
   const double Sxx = S[0], Sxy = S[1], Sxz = S[2], Syx = S[3], Syy = S[4], Syz = S[5], Szx = S[6], Szy = S[7],
                Szz = S[8];
   double A[4][4] = {{Sxx + Syy + Szz, Syz - Szy, Szx - Sxz, Sxy - Syx},
@@ -315,6 +451,13 @@ __device__ inline void horn_pose(const double S[9], const double cbar[3], const 
       z = V[3][k];
     }
   quaternion_pose(w, x, y, z, cbar, wbar, out);
+}
+
+// Writes 12 doubles [R | t].
+__device__ __forceinline__ void horn_pose(const double S[9], const double cbar[3], const double wbar[3], double* out) {
+  double q[4];
+  if (horn_refined(S, q)) quaternion_pose(q[0], q[1], q[2], q[3], cbar, wbar, out);
+  else horn_jacobi(S, cbar, wbar, out);
 }
 
 // Warp-wide sum (all lanes get the result).
