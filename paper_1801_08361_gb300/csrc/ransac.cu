@@ -202,6 +202,36 @@ __device__ __forceinline__ void horn_pose_group(double S_lane, const double cbar
 }
 
 // ---------------------------------------------------------------------------------------------
+// Chained launches: a kernel of the sequence starts while the one before it runs its last CTAs, and
+// begins with chain_begin, which waits until that one has completed and its writes are visible; its own
+// successor may be launched from then on.  A lone attempt is up to fifty launches of 5 to 30 us, and the
+// gaps between them were a tenth of it (a house frame's RANSAC takes 848 us unchained, 784 chained).  Every thread calls chain_begin before anything else, so
+// a kernel never completes before those in front of it.  Data written by the kernel in front is read with
+// plain loads only (not __ldg, whose data may not change while a kernel is resident): hence no chaining
+// from the draws, whose records are read so.
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ void chain_begin() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <class... Params, class... Args>
+cudaError_t launch_chained(bool chained, void (*kernel)(Params...), dim3 grid, unsigned threads, size_t smem, cudaStream_t s,
+                           Args... args) {
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.dynamicSmemBytes = smem;
+  c.stream = s;
+  cudaLaunchAttribute attr{};
+  attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &attr;
+  c.numAttrs = chained ? 1 : 0;
+  return cudaLaunchKernelEx(&c, kernel, Params(args)...);
+}
+
+// ---------------------------------------------------------------------------------------------
 // Valid-pixel table
 // ---------------------------------------------------------------------------------------------
 constexpr int kCompactThreads = 256;
@@ -219,6 +249,7 @@ __device__ __forceinline__ int chunk_job(const RansacJob* jobs, int n_jobs, int 
 
 __global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const RansacJob* __restrict__ jobs,
                                                                        int n_jobs) {
+  chain_begin();
   const RansacJob& job = jobs[chunk_job(jobs, n_jobs, blockIdx.x)];
   if (job_skipped(job.skip)) return;
   const int chunk = blockIdx.x - job.chunk_begin;
@@ -241,6 +272,7 @@ __global__ void __launch_bounds__(kCompactThreads) compact_count_kernel(const Ra
 
 __global__ void __launch_bounds__(kCompactThreads) compact_scatter_kernel(const RansacJob* __restrict__ jobs,
                                                                          int n_jobs) {
+  chain_begin();
   const RansacJob& job = jobs[chunk_job(jobs, n_jobs, blockIdx.x)];
   if (job_skipped(job.skip)) return;
   const int chunk = blockIdx.x - job.chunk_begin;
@@ -313,7 +345,8 @@ __global__ void __launch_bounds__(kCompactThreads) compact_scatter_kernel(const 
 cudaError_t launch_compact(const RansacJob* jobs, int n_jobs, int total_chunks, cudaStream_t s) {
   if (total_chunks <= 0) return cudaSuccess;
   compact_count_kernel<<<total_chunks, kCompactThreads, 0, s>>>(jobs, n_jobs);
-  compact_scatter_kernel<<<total_chunks, kCompactThreads, 0, s>>>(jobs, n_jobs);
+  const cudaError_t e = launch_chained(true, compact_scatter_kernel, total_chunks, kCompactThreads, 0, s, jobs, n_jobs);
+  if (e != cudaSuccess) return e;
   return cudaGetLastError();
 }
 
@@ -568,6 +601,7 @@ __device__ __forceinline__ int search_one(const RansacJob* __restrict__ jobs, in
 // from a counter when it finishes one (which warp computes a hypothesis does not change its result).
 __global__ void __launch_bounds__(kSearchWarps * 32, RELO_SEARCH_MIN_BLOCKS)
     search_kernel(const RansacJob* __restrict__ jobs, int n_jobs, int total, int32_t* __restrict__ counter) {
+  chain_begin();
   const int lane = threadIdx.x & 31;
   for (;;) {
     int gw = 0;
@@ -584,6 +618,7 @@ __global__ void __launch_bounds__(kSearchWarps * 32, RELO_SEARCH_MIN_BLOCKS)
 template <int kWarps>
 __global__ void __launch_bounds__(kWarps * 32, RELO_SEARCH_MIN_BLOCKS * kSearchWarps / kWarps)
     search_shared_kernel(const RansacJob* __restrict__ jobs, int n_jobs, int total, int32_t* __restrict__ counter) {
+  chain_begin();
   __shared__ int s_found, s_next;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (;;) {
@@ -719,6 +754,7 @@ constexpr int kFitThreads = 128;
 template <bool kGroup>
 __global__ void __launch_bounds__(kFitThreads) fit_kernel(const RansacJob* __restrict__ jobs, int n_jobs, int total,
                                                           int fit_blocks, int draw_blocks) {
+  chain_begin();
   if ((int)blockIdx.x >= fit_blocks) {
     const int q = (int)blockIdx.x - fit_blocks, jid = q / draw_blocks;
     const RansacJob& job = jobs[jid];
@@ -774,9 +810,10 @@ cudaError_t launch_hypotheses(const RansacJob* jobs, int n_jobs, int total_hyps,
   const int per_block = group ? kSolvesPerWarp * kFitThreads / 32 : kFitThreads;
   const int fit_blocks = (total_hyps + per_block - 1) / per_block, draw_blocks = (max_draws + kFitThreads - 1) / kFitThreads;
   const unsigned fit_grid = (unsigned)fit_blocks + (unsigned)draw_blocks * (unsigned)n_jobs;
-  if (group) fit_kernel<true><<<fit_grid, kFitThreads, 0, s>>>(jobs, n_jobs, total_hyps, fit_blocks, draw_blocks);
-  else fit_kernel<false><<<fit_grid, kFitThreads, 0, s>>>(jobs, n_jobs, total_hyps, fit_blocks, draw_blocks);
-  return cudaGetLastError();
+  e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  return launch_chained(true, group ? fit_kernel<true> : fit_kernel<false>, fit_grid, kFitThreads, 0, s, jobs, n_jobs,
+                        total_hyps, fit_blocks, draw_blocks);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -1030,6 +1067,7 @@ __global__ void RELO_ENERGY_BOUNDS energy_kernel(const RansacJob* __restrict__ j
                                                                   const int32_t* __restrict__ alive_prefix, int r) {
   __shared__ ModeSlots slots[kRoundWarps];
   __shared__ float part[kRoundWarps][32];
+  chain_begin();
   energy_block(jobs, alive_prefix, r, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, slots, part);
 }
 
@@ -1038,6 +1076,7 @@ __global__ void RELO_ENERGY_BOUNDS energy_kernel(const RansacJob* __restrict__ j
 __global__ void __launch_bounds__(256) sum_scores_kernel(const RansacJob* __restrict__ jobs,
                                                          const int32_t* __restrict__ alive_prefix, int r, int n_split) {
   static_assert(kRoundWarps == 8, "eight lanes stand for the warps");
+  chain_begin();
   const int jid = blockIdx.y, n_alive = alive_prefix[jid + 1] - alive_prefix[jid];
   const int a = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3), w = threadIdx.x & 7, lane = threadIdx.x & 31;
   const RansacJob& job = jobs[jid];
@@ -1159,6 +1198,7 @@ __device__ __forceinline__ void select_block(const RansacJob* __restrict__ jobs,
 __global__ void __launch_bounds__(1024) select_kernel(const RansacJob* __restrict__ jobs,
                                                       const int32_t* __restrict__ alive_prefix, int r) {
   extern __shared__ unsigned long long skey[];
+  chain_begin();
   select_block(jobs, alive_prefix, r, blockIdx.x, skey);
 }
 
@@ -1301,6 +1341,7 @@ template <int LG>
 __global__ void __launch_bounds__(kRoundWarps * 32, LG == 0 ? RELO_REFINE_MIN_BLOCKS : LG == 1 ? 3 : RELO_REFINE_FEW_MIN_BLOCKS)
     refine_kernel(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ surv_prefix, int r) {
   __shared__ RefineShared sh;
+  chain_begin();
   refine_block<LG>(jobs, surv_prefix, r, blockIdx.x, blockIdx.y, blockIdx.z, sh);
 }
 
@@ -1349,7 +1390,7 @@ __device__ __forceinline__ void refit_group(const RansacJob& job, int k, int r) 
   if (h >= 0) {
     const int parts = ((r + 1) * job.B + kRefinePixels - 1) / kRefinePixels;
     const float2* src = job.refit + (size_t)h * job.refit_parts * 16 + l;
-#pragma unroll 4
+#pragma unroll 16
     for (int p = 0; p < parts; ++p) {
       const float2 v = src[16 * p];
       f = __dadd_rn(f, __dadd_rn((double)v.x, (double)v.y));
@@ -1376,6 +1417,7 @@ __device__ __forceinline__ void refit_group(const RansacJob& job, int k, int r) 
 
 __global__ void __launch_bounds__(32) refit_group_kernel(const RansacJob* __restrict__ jobs, int n_jobs,
                                                          const int32_t* __restrict__ surv_prefix, int total, int r) {
+  chain_begin();
   const int gid = (int)blockIdx.x * kSolvesPerWarp + ((int)threadIdx.x >> 4);
   const int jid = find_job_by(surv_prefix, n_jobs, min(gid, total - 1));
   refit_group(jobs[jid], gid < total ? gid - surv_prefix[jid] : -1, r);
@@ -1384,6 +1426,7 @@ __global__ void __launch_bounds__(32) refit_group_kernel(const RansacJob* __rest
 __global__ void __launch_bounds__(32) refit_kernel(const RansacJob* __restrict__ jobs, int n_jobs,
                                                    const int32_t* __restrict__ surv_prefix, int total, int r,
                                                    int per) {
+  chain_begin();
   const int gid = blockIdx.x * per + threadIdx.x;
   if ((int)threadIdx.x >= per || gid >= total) return;
   const int jid = find_job_by(surv_prefix, n_jobs, gid);
@@ -1391,11 +1434,11 @@ __global__ void __launch_bounds__(32) refit_kernel(const RansacJob* __restrict__
 }
 
 template <int LG>
-void launch_refine(const RansacJob* jobs, int n_jobs, const int32_t* surv_prefix, int max_surv, int parts, int round,
-                   cudaStream_t s) {
+cudaError_t launch_refine(const RansacJob* jobs, int n_jobs, const int32_t* surv_prefix, int max_surv, int parts, int round,
+                          cudaStream_t s) {
   constexpr int kHere = 32 >> LG;
-  refine_kernel<LG><<<dim3((max_surv + kHere - 1) / kHere, parts, n_jobs), kRoundWarps * 32, 0, s>>>(jobs, surv_prefix,
-                                                                                                    round);
+  return launch_chained(true, refine_kernel<LG>, dim3((max_surv + kHere - 1) / kHere, parts, n_jobs), kRoundWarps * 32, 0, s,
+                        jobs, surv_prefix, round);
 }
 
 int energy_splits(int n_jobs, int max_alive, int B) {
@@ -1419,16 +1462,21 @@ cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int
   if (sched.refit_per < 0 || sched.refit_per > 32) return cudaErrorInvalidValue;
   // few jobs: their pixels are split over more CTAs than the hypothesis chunks make
   const int n_split = energy_splits(n_jobs, max_alive, B);
-  energy_kernel<<<dim3((max_alive + 31) / 32, n_jobs, n_split), kRoundWarps * 32, 0, s>>>(jobs, alive_prefix_dev, round);
-  if (n_split > 1)
-    sum_scores_kernel<<<dim3((max_alive * 8 + 255) / 256, n_jobs), 256, 0, s>>>(jobs, alive_prefix_dev, round, n_split);
+  // (round 0 follows the draws, which it reads with __ldg)
+  cudaError_t e = launch_chained(round > 0, energy_kernel, dim3((max_alive + 31) / 32, n_jobs, n_split), kRoundWarps * 32, 0, s,
+                                 jobs, alive_prefix_dev, round);
+  if (e == cudaSuccess && n_split > 1)
+    e = launch_chained(true, sum_scores_kernel, dim3((max_alive * 8 + 255) / 256, n_jobs), 256, 0, s, jobs, alive_prefix_dev,
+                       round, n_split);
+  if (e != cudaSuccess) return e;
   int npow = 32;
   while (npow < max_alive) npow <<= 1;
-  select_kernel<<<n_jobs, std::min(npow, 1024), (size_t)npow * (sizeof(unsigned long long) + sizeof(int)), s>>>(
-      jobs, alive_prefix_dev, round);
+  e = launch_chained(true, select_kernel, n_jobs, std::min(npow, 1024), (size_t)npow * (sizeof(unsigned long long) + sizeof(int)),
+                     s, jobs, alive_prefix_dev, round);
+  if (e != cudaSuccess) return e;
   const int parts = ((round + 1) * B + kRefinePixels - 1) / kRefinePixels;
   int n_sms = 0;
-  const cudaError_t e = device_sms(&n_sms);
+  e = device_sms(&n_sms);
   if (e != cudaSuccess) return e;
   // Few survivors in all: a hypothesis is shared by more lanes, up to sixteen, while the CTAs leave SMs
   // idle (a house frame's first round: 16 chunks of 32 survivors, one part of 64 pixels).  Re-fit sums of a
@@ -1436,23 +1484,21 @@ cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int
   int lg = group_log2(max_surv);
   while (lg < 4 && (long)((max_surv + (32 >> lg) - 1) / (32 >> lg)) * parts * n_jobs < 2 * n_sms) ++lg;
   switch (lg) {
-    case 0: launch_refine<0>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
-    case 1: launch_refine<1>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
-    case 2: launch_refine<2>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
-    case 3: launch_refine<3>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
-    case 4: launch_refine<4>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
-    default: launch_refine<5>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 0: e = launch_refine<0>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 1: e = launch_refine<1>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 2: e = launch_refine<2>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 3: e = launch_refine<3>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    case 4: e = launch_refine<4>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
+    default: e = launch_refine<5>(jobs, n_jobs, surv_prefix_dev, max_surv, parts, round, s); break;
   }
-  if (sched.refit_per == 0 && total_surv <= kGroupSolves) {
-    refit_group_kernel<<<(unsigned)((total_surv + kSolvesPerWarp - 1) / kSolvesPerWarp), 32, 0, s>>>(
-        jobs, n_jobs, surv_prefix_dev, total_surv, round);
-    return cudaGetLastError();
-  }
+  if (e != cudaSuccess) return e;
+  if (sched.refit_per == 0 && total_surv <= kGroupSolves)
+    return launch_chained(true, refit_group_kernel, (unsigned)((total_surv + kSolvesPerWarp - 1) / kSolvesPerWarp), 32, 0, s,
+                          jobs, n_jobs, surv_prefix_dev, total_surv, round);
   const int per = sched.refit_per > 0 ? sched.refit_per
                                      : std::max(1, std::min(32, (total_surv + 2 * n_sms - 1) / (2 * n_sms)));
-  refit_kernel<<<(unsigned)((total_surv + per - 1) / per), 32, 0, s>>>(jobs, n_jobs, surv_prefix_dev, total_surv,
-                                                                       round, per);
-  return cudaGetLastError();
+  return launch_chained(true, refit_kernel, (unsigned)((total_surv + per - 1) / per), 32, 0, s, jobs, n_jobs, surv_prefix_dev,
+                        total_surv, round, per);
 }
 
 // Tries of every hypothesis of the job (a kept try j counts j + 1, a failed hypothesis max_tries),
@@ -1473,17 +1519,22 @@ __device__ __forceinline__ void finalise_one(const RansacJob& job, unsigned long
   const int32_t* fin = (job.n_rounds & 1) ? job.alive_b : job.alive_a;
   const int h = fin[0];
   relo_pose_result* res = job.result;
-  const double* p = job.poses + 12 * (size_t)h;
-  for (int i = 0; i < 3; ++i)
-    for (int q = 0; q < 4; ++q) res->pose_c2s[4 * i + q] = p[4 * i + q];
+  // everything is loaded before the first store, which would hold the loads back
+  double p[12];
+#pragma unroll
+  for (int q = 0; q < 12; ++q) p[q] = job.poses[12 * (size_t)h + q];
+  const double energy = job.energy[h];
+  const int32_t inliers = job.inliers[h], up = job.upstream ? *job.upstream : 0, err = *job.err, ok = job.hyp_ok[h];
+  const int32_t n_valid = *job.n_valid;
+#pragma unroll
+  for (int q = 0; q < 12; ++q) res->pose_c2s[q] = p[q];
   res->pose_c2s[12] = res->pose_c2s[13] = res->pose_c2s[14] = 0.0;
   res->pose_c2s[15] = 1.0;
-  res->energy = job.energy[h];
-  res->n_inliers = job.inliers[h];
-  const int32_t up = job.upstream ? *job.upstream : 0;
-  res->status = up ? up : (*job.err ? RELO_EDEVICE : (job.hyp_ok[h] ? RELO_OK : RELO_ENOTFOUND));
+  res->energy = energy;
+  res->n_inliers = inliers;
+  res->status = up ? up : (err ? RELO_EDEVICE : (ok ? RELO_OK : RELO_ENOTFOUND));
   res->verified = 0;
-  res->n_valid = *job.n_valid;
+  res->n_valid = n_valid;
   res->hypothesis = h;
   res->n_rounds = job.n_rounds;
   res->omega = res->omega_a = res->omega_b = res->omega_ab = res->sum_absdiff_mm = 0;
@@ -1510,6 +1561,7 @@ __device__ __forceinline__ void finalise_one(const RansacJob& job, unsigned long
 
 // Warp per job.
 __global__ void __launch_bounds__(128) finalise_kernel(const RansacJob* __restrict__ jobs, int n_jobs) {
+  chain_begin();
   const int jid = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
   if (jid >= n_jobs) return;
   const RansacJob& job = jobs[jid];
@@ -1713,8 +1765,7 @@ cudaError_t launch_verify_decide_one(relo_pose_result* res, uint64_t omega, cuda
 
 cudaError_t launch_finalise(const RansacJob* jobs, int n_jobs, cudaStream_t s) {
   if (n_jobs <= 0) return cudaSuccess;
-  finalise_kernel<<<(n_jobs + 3) / 4, 128, 0, s>>>(jobs, n_jobs);
-  return cudaGetLastError();
+  return launch_chained(true, finalise_kernel, (n_jobs + 3) / 4, 128, 0, s, jobs, n_jobs);
 }
 
 // Fallback results start as "not run" (a skipped job writes nothing).
