@@ -1580,7 +1580,7 @@ void reg_layout(char* base, int n, int W, int H, bool training, RegBuffers& b, s
     for (int l = 0; l < kRegLayers - 1; ++l) b.gpre[l] = c.take<bf16>((size_t)n * Hs[l + 1] * Ws[l + 1] * 64);
     size_t part = 0;
     for (int l = 0; l < kRegLayers; ++l)
-      part = std::max(part, wgrad_parts(kRegCinPad[l], n, Hs[l + 1], Ws[l + 1]) * wgrad_partial_floats(kRegCinPad[l], kRegCoutPad[l]));
+      part = std::max(part, wgrad_parts(kRegCin[l], n, Hs[l + 1], Ws[l + 1]) * wgrad_partial_floats(kRegCin[l], kRegCoutPad[l]));
     b.partial = c.take<float>(part);
     b.loss = c.take<float>(1);
     b.loss_sums = c.take<float>(loss_blocks((int)cells));
@@ -1591,11 +1591,11 @@ void reg_layout(char* base, int n, int W, int H, bool training, RegBuffers& b, s
 }
 
 relo_status reg_forward(relo_regressor* r, const RegBuffers& b, const uint16_t* depth, const uint8_t* rgba, int n,
-                        int W, int H, cudaStream_t s, bool training = false) {
+                        int W, int H, cudaStream_t s) {
   int Hs[kRegLayers + 1], Ws[kRegLayers + 1];
   reg_sizes(W, H, Hs, Ws);
-  // the tcgen05 first layer reads the images themselves; the backward pass needs the network's input
-  if (training || !g_conv_tcgen05.load()) RELO_CUDA(launch_input(depth, (const uint32_t*)rgba, (long)n * H * W, b.x, s));
+  // the tcgen05 first layer reads the images themselves
+  if (!g_conv_tcgen05.load()) RELO_CUDA(launch_input(depth, (const uint32_t*)rgba, (long)n * H * W, b.x, s));
   RELO_CUDA(cudaMemsetAsync(r->d_status, 0, sizeof(int32_t), s));
   for (int l = 0; l < kRegLayers; ++l) {
     if (l == 0 && g_conv_tcgen05.load()) {
@@ -1633,14 +1633,17 @@ relo_status reg_forward(relo_regressor* r, const RegBuffers& b, const uint16_t* 
   return RELO_OK;
 }
 
-relo_status reg_backward(relo_regressor* r, const RegBuffers& b, int n, int W, int H, cudaStream_t s) {
+relo_status reg_backward(relo_regressor* r, const RegBuffers& b, const uint16_t* depth, const uint8_t* rgba, int n, int W,
+                         int H, cudaStream_t s) {
   int Hs[kRegLayers + 1], Ws[kRegLayers + 1];
   reg_sizes(W, H, Hs, Ws);
   const bf16* g = b.ghead;
   int gs = 16;
   for (int l = kRegLayers - 1; l >= 0; --l) {
     WgradArgs wa{};
-    wa.in = l == 0 ? b.x : b.act[l];
+    wa.in = l > 0 ? b.act[l] : nullptr;
+    wa.depth = depth;
+    wa.rgba = (const uint32_t*)rgba;
     wa.g = g;
     wa.partial = b.partial;
     wa.B = n;
@@ -1650,7 +1653,7 @@ relo_status reg_backward(relo_regressor* r, const RegBuffers& b, int n, int W, i
     wa.Wo = Ws[l + 1];
     wa.stride = kRegStride[l];
     wa.GS = gs;
-    RELO_CUDA(launch_wgrad(kRegCinPad[l], kRegCoutPad[l], wa, kRegCin[l], kRegCout[l], r->d_g + r->w_off[l],
+    RELO_CUDA(launch_wgrad(kRegCin[l], kRegCoutPad[l], wa, kRegCin[l], kRegCout[l], r->d_g + r->w_off[l],
                            r->d_g + r->b_off[l], s));
     if (l > 0) {
       ConvArgs a{};
@@ -1700,7 +1703,7 @@ relo_status reg_loss_and_grads(relo_regressor* r, const RegBuffers& b, const uin
                                int n, const relo_intrinsics* in, const double* poses, cudaStream_t s) {
   const int W = in->width, H = in->height, Wc = W / 8, Hc = H / 8;
   RELO_CUDA(cudaMemcpyAsync(b.poses, poses, (size_t)n * 16 * sizeof(double), cudaMemcpyHostToDevice, s));
-  relo_status st = reg_forward(r, b, depth, rgba, n, W, H, s, true);
+  relo_status st = reg_forward(r, b, depth, rgba, n, W, H, s);
   if (st) return st;
   CellArgs ca{};
   ca.depth = depth;
@@ -1719,7 +1722,7 @@ relo_status reg_loss_and_grads(relo_regressor* r, const RegBuffers& b, const uin
   ca.oz = r->origin[2];
   RELO_CUDA(launch_targets(ca, b.tgt, b.counters, s));
   RELO_CUDA(launch_loss(b.head, b.tgt, n * Wc * Hc, b.ghead, b.counters, b.loss_sums, b.loss, s));
-  return reg_backward(r, b, n, W, H, s);
+  return reg_backward(r, b, depth, rgba, n, W, H, s);
 }
 
 }  // namespace

@@ -226,8 +226,7 @@ cudaError_t launch_conv(int cin, int nt, const ConvArgs& a, int n_sms, cudaStrea
 // additions -- the tensor core's own additions drop bits, which a chain over hundreds of tiles shows --
 // and one partial per CTA is left to sum.
 // The bias is one more product, with a row of ones.  16 views of 640 x 480: 0.38 ms with the sums for
-// all layers; the 64-channel kernels are bound by mma.sync (288 products a scheduler and tile), the
-// first layer's by its three passes over 157 MB and by latency, hence two CTAs an SM there.
+// all layers; bound by mma.sync (288 products a scheduler and tile of 64 channels, 17 cycles each).
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const bf16* p) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(p);
@@ -251,7 +250,7 @@ __device__ __forceinline__ void copy_or_zero16(bf16* dst, const bf16* src, bool 
 constexpr int kWgradThreads = 256, kWgradW = 8, kWgradH = 8;  // a tile's output pixels
 constexpr int kWgradK = kWgradW * kWgradH / 16;               // products' depth: pairs of tile rows
 
-// CIN input channels (16 or 64), NW n8 tiles of output channels per warp: N = 16 NW channels of g rows
+// CIN input channels (64), NW n8 tiles of output channels per warp: N = 16 NW channels of g rows
 // of GS; STRIDE 1 or 2.
 template <int CIN, int NW, int STRIDE>
 struct WgradShape {
@@ -267,7 +266,7 @@ struct WgradShape {
 };
 
 template <int CIN, int NW, int STRIDE>
-__global__ void __launch_bounds__(kWgradThreads, CIN == 16 ? 2 : 1) wgrad_kernel(WgradArgs a) {
+__global__ void __launch_bounds__(kWgradThreads, 1) wgrad_kernel(WgradArgs a) {
   using S = WgradShape<CIN, NW, STRIDE>;
   extern __shared__ __align__(16) unsigned char wgrad_smem[];
   bf16* smem = reinterpret_cast<bf16*>(wgrad_smem);
@@ -409,6 +408,125 @@ cudaError_t launch_wgrad_t(const WgradArgs& a, int grid, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// The first layer's, straight from the depth and colour images: a CTA converts the 17 x 17 pixels under
+// its tile of 8 x 8 outputs as it loads them (the next tile's are on their way meanwhile), 4 channels = 8
+// bytes a pixel, so that 16 bytes hold two neighbouring taps and an operand row of a kernel row ky is
+// its four columns' channels (the fourth column's products are dropped): three products a 16-pixel step
+// where nine taps of 16 padded channels took nine.  A warp per 8 output channels, four CTAs an SM.
+// 16 views of 640 x 480: 73 us; the padded operand's kernel took 127 us and making that
+// operand another 31.  The gradient's 157 MB would take 23.
+constexpr int kWgrad0Cols = 2 * kWgradW + 2, kWgrad0Rows = 2 * kWgradH + 1, kWgrad0Px = kWgrad0Cols * kWgrad0Rows;
+constexpr int kWgrad0Stages = 3, kWgrad0RowG = 64 + 8;
+__global__ void __launch_bounds__(kWgradThreads, 4) wgrad_first_kernel(WgradArgs a) {
+  static_assert(kWgradThreads == 256 && kWgrad0Px <= 2 * kWgradThreads, "eight warps of 8 channels, two pixels a thread");
+  __shared__ __align__(16) bf16 s_in[2][kWgrad0Px * 4];
+  __shared__ __align__(16) bf16 s_g[kWgrad0Stages][kWgradW * kWgradH * kWgrad0RowG];
+  __shared__ bf16 s_colour[256];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  s_colour[tid] = input_colour((uint32_t)tid);
+  const uint32_t ones[4] = {0x3F803F80u, 0x3F803F80u, 0x3F803F80u, 0x3F803F80u};
+  const int tiles_x = (a.Wo + kWgradW - 1) / kWgradW, tiles_y = (a.Ho + kWgradH - 1) / kWgradH;
+  const int n_tiles = a.B * tiles_x * tiles_y;
+
+  uint32_t dep[2], col[2];
+  auto fetch = [&](int tile) {
+    const int b = tile / (tiles_x * tiles_y), q = tile % (tiles_x * tiles_y);
+    const int iy0 = q / tiles_x * kWgradH * 2 - 1, ix0 = q % tiles_x * kWgradW * 2 - 1;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int p = tid + k * kWgradThreads, row = p / kWgrad0Cols, c = p - row * kWgrad0Cols;
+      const int iy = iy0 + row, ix = ix0 + c;
+      dep[k] = 0x10000u;  // outside the image (and the fourth column's last pixel): zeros
+      col[k] = 0;
+      if (p < kWgrad0Px && c < kWgrad0Cols - 1 && iy >= 0 && ix >= 0 && iy < a.Hi && ix < a.Wi) {
+        const size_t px = ((size_t)b * a.Hi + iy) * a.Wi + ix;
+        dep[k] = __ldg(&a.depth[px]);
+        col[k] = __ldg(&a.rgba[px]);
+      }
+    }
+  };
+  auto load_g = [&](int tile, int stage) {
+    const int b = tile / (tiles_x * tiles_y), q = tile % (tiles_x * tiles_y);
+    const int oy0 = q / tiles_x * kWgradH, ox0 = q % tiles_x * kWgradW;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int v = tid + k * kWgradThreads, px = v >> 3, c = v & 7, oy = oy0 + px / kWgradW, ox = ox0 + px % kWgradW;
+      const bool ok = oy < a.Ho && ox < a.Wo;
+      copy_or_zero16(&s_g[stage][px * kWgrad0RowG + c * 8], ok ? a.g + (((size_t)b * a.Ho + oy) * a.Wo + ox) * a.GS + c * 8 : a.g, ok);
+    }
+  };
+
+  float acc[3][4] = {}, accb[2] = {};
+  if ((int)blockIdx.x < n_tiles) fetch(blockIdx.x);
+#pragma unroll
+  for (int k = 0; k < kWgrad0Stages - 1; ++k) {
+    if ((int)(blockIdx.x + k * gridDim.x) < n_tiles) load_g(blockIdx.x + k * gridDim.x, k);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  __syncthreads();  // the colour table
+  const int q = lane >> 3, r = lane & 7;
+  int stage = 0, buf = 0;
+  for (int tile = blockIdx.x; tile < n_tiles; tile += gridDim.x, buf ^= 1, stage = stage + 1 < kWgrad0Stages ? stage + 1 : 0) {
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const int p = tid + k * kWgradThreads;
+      if (p >= kWgrad0Px) continue;
+      const bf16 d = input_depth(dep[k]);
+      const uint16_t* lut = reinterpret_cast<const uint16_t*>(s_colour);
+      uint2 v = make_uint2(*reinterpret_cast<const uint16_t*>(&d) | (uint32_t)lut[col[k] & 0xFF] << 16,
+                           (uint32_t)lut[(col[k] >> 8) & 0xFF] | (uint32_t)lut[(col[k] >> 16) & 0xFF] << 16);
+      if (dep[k] & 0x10000u) v = make_uint2(0u, 0u);
+      *reinterpret_cast<uint2*>(&s_in[buf][p * 4]) = v;
+    }
+    asm volatile("cp.async.wait_group %0;" ::"n"(kWgrad0Stages - 2) : "memory");
+    __syncthreads();  // the tile is here for all, and the one before is read
+    if (tile + (int)gridDim.x < n_tiles) fetch(tile + gridDim.x);
+    const int next = tile + (kWgrad0Stages - 1) * gridDim.x;
+    if (next < n_tiles) load_g(next, stage > 0 ? stage - 1 : kWgrad0Stages - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    const bf16 *sI = s_in[buf], *sG = s_g[stage];
+    uint32_t bf[kWgradK][2];
+#pragma unroll
+    for (int ks = 0; ks < kWgradK; ++ks)
+      ldsm_x2_t(bf[ks][0], bf[ks][1], sG + (ks * 16 + r + 8 * (q & 1)) * kWgrad0RowG + warp * 8);
+#pragma unroll
+    for (int ky = 0; ky < 3; ++ky) {
+      float sum[4] = {};
+#pragma unroll
+      for (int ks = 0; ks < kWgradK; ++ks) {
+        uint32_t af[4];
+        ldsm_x4_t(af, sI + ((2 * (2 * ks + (q >> 1)) + ky) * kWgrad0Cols + 2 * r + 2 * (q & 1)) * 4);
+        mma_bf16(sum, af, bf[ks][0], bf[ks][1]);
+      }
+#pragma unroll
+      for (int e = 0; e < 4; ++e) acc[ky][e] += sum[e];
+    }
+    float sum[4] = {};
+#pragma unroll
+    for (int ks = 0; ks < kWgradK; ++ks) mma_bf16(sum, ones, bf[ks][0], bf[ks][1]);
+    accb[0] += sum[0];
+    accb[1] += sum[1];
+  }
+  // rows of a product: channel m & 3 of column m >> 2
+  float* out = a.partial + (size_t)blockIdx.x * (9 * 64 * 4 + 64);
+  const int g = lane >> 2, n = warp * 8 + 2 * (lane & 3);
+#pragma unroll
+  for (int ky = 0; ky < 3; ++ky) {
+    float* o = out + ((3 * ky + (g >> 2)) * 64 + n) * 4 + (g & 3);
+    o[0] = acc[ky][0];
+    o[4] = acc[ky][1];
+    if (g < 4) {
+      o = out + ((3 * ky + 2) * 64 + n) * 4 + g;
+      o[0] = acc[ky][2];
+      o[4] = acc[ky][3];
+    }
+  }
+  if (g == 0) {
+    out[9 * 64 * 4 + n] = accb[0];
+    out[9 * 64 * 4 + n + 1] = accb[1];
+  }
+}
+
 // Sum of the CTAs' partials into the master-layout gradients gw [3][3][cin][cout] and gb [cout] (only
 // the real channels): 32 neighbouring weights per CTA, eight warps taking every eighth partial each,
 // added in a fixed order.
@@ -447,7 +565,7 @@ __global__ void __launch_bounds__(256) wgrad_reduce_kernel(const float* __restri
 
 int wgrad_parts(int cin, int B, int Ho, int Wo) {
   const long tiles = (long)B * ((Wo + kWgradW - 1) / kWgradW) * ((Ho + kWgradH - 1) / kWgradH);
-  const int most = kWgradCtas * (cin == 16 ? 2 : 1);
+  const int most = kWgradCtas * (cin == 4 ? 4 : 1);
   return (int)(tiles < most ? tiles : most);
 }
 
@@ -461,8 +579,11 @@ cudaError_t launch_wgrad(int cin, int cout_pad, const WgradArgs& a, int cin_real
   const int parts = wgrad_parts(cin, a.B, a.Ho, a.Wo);
   if (parts <= 0) return cudaSuccess;
   cudaError_t e = cudaErrorInvalidValue;
-  if (cin == 16 && cout_pad == 64 && a.stride == 2) e = launch_wgrad_t<16, 4, 2>(a, parts, s);
-  else if (cin == 64 && cout_pad == 64 && a.stride == 2) e = launch_wgrad_t<64, 4, 2>(a, parts, s);
+  if (cin == 4 && cout_pad == 64 && a.stride == 2) {
+    wgrad_first_kernel<<<parts, kWgradThreads, 0, s>>>(a);
+    e = cudaGetLastError();
+  }
+  if (cin == 64 && cout_pad == 64 && a.stride == 2) e = launch_wgrad_t<64, 4, 2>(a, parts, s);
   else if (cin == 64 && cout_pad == 64 && a.stride == 1) e = launch_wgrad_t<64, 4, 1>(a, parts, s);
   else if (cin == 64 && cout_pad == 8 && a.stride == 1) e = launch_wgrad_t<64, 1, 1>(a, parts, s);
   if (e != cudaSuccess) return e;
@@ -529,8 +650,6 @@ cudaError_t launch_input(const uint16_t* depth, const uint32_t* rgba, long n_pix
   input_kernel<<<(unsigned)((n_pix + 255) / 256), 256, 0, s>>>(depth, rgba, n_pix, x);
   return cudaGetLastError();
 }
-
-
 
 // Targets: scene coordinate of each cell's centre pixel minus the origin; w = 1 if scored.  The scored
 // cells are counted into *scored (zeroed before).

@@ -28,7 +28,9 @@ struct ConvArgs {
 
 // Backward-weight sums (see wgrad_kernel)
 struct WgradArgs {
-  const bf16* in;     // layer input [B][Hi][Wi][CIN]
+  const bf16* in;     // layer input [B][Hi][Wi][64], or (the first layer) the images
+  const uint16_t* depth;  // [B][Hi][Wi] mm
+  const uint32_t* rgba;   // [B][Hi][Wi]
   const bf16* g;      // gradient of the pre-activation output [B][Ho][Wo][GS] (first N channels used)
   float* partial;     // [wgrad_parts][wgrad_partial_floats]
   int B, Hi, Wi, Ho, Wo, stride, GS;
@@ -68,7 +70,7 @@ constexpr int kRegCin[kRegLayers] = {4, 64, 64, 64, 64, 64, 64, 64};
 constexpr int kRegCout[kRegLayers] = {64, 64, 64, 64, 64, 64, 64, 4};
 constexpr int kRegCinPad[kRegLayers] = {16, 64, 64, 64, 64, 64, 64, 64};
 constexpr int kRegCoutPad[kRegLayers] = {64, 64, 64, 64, 64, 64, 64, 8};
-constexpr int kWgradCtas = 152;  // most CTAs (partial sums per weight) of a backward-weight launch; 16 channels: twice that
+constexpr int kWgradCtas = 152;  // most CTAs (partial sums per weight) of a backward-weight launch; first layer: four times that
 
 // Adam step of all parameters and the operands derived from them (see adam_kernel)
 struct AdamArgs {
@@ -82,7 +84,7 @@ struct AdamArgs {
 };
 
 cudaError_t launch_conv(int cin, int nt, const ConvArgs& a, int n_sms, cudaStream_t s);
-// Gradients gw [3][3][cin_real][cout_real] and gb [cout_real] of a layer.
+// Gradients gw [3][3][cin_real][cout_real] and gb [cout_real] of a layer (cin 4: the first, from the images).
 int wgrad_parts(int cin, int B, int Ho, int Wo);
 size_t wgrad_partial_floats(int cin, int cout_pad);
 cudaError_t launch_wgrad(int cin, int cout_pad, const WgradArgs& a, int cin_real, int cout_real, float* gw, float* gb,
