@@ -407,8 +407,8 @@ relo_status relo_ransac_round(const relo_forest* forest, const uint16_t* depth_d
  * over cells whose centre pixel has depth of rho(e) + 1/2 e^2 exp(-s) + 3/2 s, e = |y - y_hat|,
  * rho(e) = sqrt(e^2 + 1e-6 m^2); the gradient holds the error of the variance term fixed (the
  * coordinates follow rho alone).  Adam (0.9, 0.999, 1e-8).  Computed with BF16 tensor-core
- * convolutions accumulating in FP32 (FP32 master weights): the 64 -> 64-channel forward layers on
- * tcgen05 (TMA-fed, TMEM accumulators), the rest with mma.sync.
+ * convolutions accumulating in FP32 (FP32 master weights): forward and backward-data on tcgen05
+ * (TMA-fed, TMEM accumulators), backward-weight with mma.sync.
  * Parameters, flat FP32, per layer l: w [3][3][cin][cout] then b [cout], cin = 4, 64, ...,
  * cout = 64, ..., 4 (relo_regressor_param_count() values in all).  Images must have sides that
  * are multiples of 8.  Errors: RELO_EINVAL (sizes, null pointers, workspace), RELO_ENOMEM.

@@ -1466,7 +1466,7 @@ relo_status relo_ransac_round(const relo_forest* f, const uint16_t* depth, const
   RELO_CUDA(launch_compact(s.d_job, 1, s.chunks, cs));
   RELO_CUDA(launch_draw(s.d_job, 1, round, s.d_alive, cs));
   RELO_CUDA(launch_round(s.d_job, 1, round, s.d_alive, n_alive, n_alive, s.d_surv, (n_alive + 1) / 2,
-                         (n_alive + 1) / 2, p->batch, cs));
+                         (n_alive + 1) / 2, p->batch, cs, Schedule(), true));
   return RELO_OK;
 }
 
@@ -1581,7 +1581,9 @@ void reg_layout(char* base, int n, int W, int H, bool training, RegBuffers& b, s
     size_t part = 0;
     for (int l = 0; l < kRegLayers; ++l)
       part = std::max(part, wgrad_parts(kRegCin[l], n, Hs[l + 1], Ws[l + 1]) * wgrad_partial_floats(kRegCin[l], kRegCoutPad[l]));
-    b.partial = c.take<float>(part);
+    // (the padded input is read by the forward pass alone, and only on the mma.sync path)
+    const bool in_x = part * sizeof(float) <= (size_t)n * H * W * 16 * sizeof(bf16);
+    b.partial = in_x ? reinterpret_cast<float*>(b.x) : c.take<float>(part);
     b.loss = c.take<float>(1);
     b.loss_sums = c.take<float>(loss_blocks((int)cells));
     b.counters = c.take<int32_t>(2);

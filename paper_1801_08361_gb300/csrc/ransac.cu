@@ -205,10 +205,10 @@ __device__ __forceinline__ void horn_pose_group(double S_lane, const double cbar
 // Chained launches: a kernel of the sequence starts while the one before it runs its last CTAs, and
 // begins with chain_begin, which waits until that one has completed and its writes are visible; its own
 // successor may be launched from then on.  A lone attempt is up to fifty launches of 5 to 30 us, and the
-// gaps between them were a tenth of it (a house frame's RANSAC takes 848 us unchained, 784 chained).  Every thread calls chain_begin before anything else, so
-// a kernel never completes before those in front of it.  Data written by the kernel in front is read with
-// plain loads only (not __ldg, whose data may not change while a kernel is resident): hence no chaining
-// from the draws, whose records are read so.
+// gaps between them were a tenth of it (a house frame's RANSAC: 848 us unchained, 784 chained).  Every
+// thread calls chain_begin before anything else, so a kernel never completes before those in front of it.
+// Data written by the kernel in front is read with plain loads only (not __ldg, whose data may not change
+// while a kernel is resident): hence no chaining from the draws, whose records are read so.
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void chain_begin() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1457,13 +1457,13 @@ cudaError_t launch_draw(const RansacJob* jobs, int n_jobs, int round, const int3
 
 cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int32_t* alive_prefix_dev,
                          int total_alive, int max_alive, const int32_t* surv_prefix_dev, int total_surv, int max_surv,
-                         int B, cudaStream_t s, const Schedule& sched) {
+                         int B, cudaStream_t s, const Schedule& sched, bool after_draw) {
   if (total_alive <= 0) return cudaSuccess;
   if (sched.refit_per < 0 || sched.refit_per > 32) return cudaErrorInvalidValue;
   // few jobs: their pixels are split over more CTAs than the hypothesis chunks make
   const int n_split = energy_splits(n_jobs, max_alive, B);
-  // (round 0 follows the draws, which it reads with __ldg)
-  cudaError_t e = launch_chained(round > 0, energy_kernel, dim3((max_alive + 31) / 32, n_jobs, n_split), kRoundWarps * 32, 0, s,
+  // (round 0 follows the draws, which are read with __ldg)
+  cudaError_t e = launch_chained(round > 0 && !after_draw, energy_kernel, dim3((max_alive + 31) / 32, n_jobs, n_split), kRoundWarps * 32, 0, s,
                                  jobs, alive_prefix_dev, round);
   if (e == cudaSuccess && n_split > 1)
     e = launch_chained(true, sum_scores_kernel, dim3((max_alive * 8 + 255) / 256, n_jobs), 256, 0, s, jobs, alive_prefix_dev,

@@ -660,7 +660,7 @@ cudaError_t launch_draw(const RansacJob* jobs, int n_jobs, int round, const int3
 int round_launches(int n_jobs, int max_alive, int B);
 cudaError_t launch_round(const RansacJob* jobs, int n_jobs, int round, const int32_t* alive_prefix_dev,
                          int total_alive, int max_alive, const int32_t* surv_prefix_dev, int total_surv, int max_surv,
-                         int B, cudaStream_t s, const Schedule& sched = Schedule());
+                         int B, cudaStream_t s, const Schedule& sched = Schedule(), bool after_draw = false);
 cudaError_t launch_finalise(const RansacJob* jobs, int n_jobs, cudaStream_t s);
 
 // One persistent launch for a pass's search, fit, rounds and finalise (ransac.cu): items in
