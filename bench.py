@@ -66,26 +66,25 @@ ALG_BYTES_PER_PIXEL = {
     "learned_verify": 35.87,
 }
 # DRAM bytes (read + write) per attempt of the stage's main kernel: the ncu captures summarised in
-# profiles/attempt_dram_house_640x480_batch32.md, profiles/raycast_apron_house_640x480_batch32.md
-# and profiles/forest_kernel_house_640x480_batch32.md
+# profiles/kernels_house_640x480_batch32.md and (verification) profiles/raycast_apron_house_640x480_batch32.md
 # (32 attempts per launch, the current kernels)
 # divided by 32; a launch of A attempts is reported as A times that (attempts are independent, so
 # the traffic grows with their number; None: not captured for the current code).
 PROFILED_TRAFFIC_BYTES_PER_ATTEMPT = {
-    "query_raycast": (974674688 + 151929344) / 32,
-    "forest_eval": (101758464 + 64701440) / 32,
-    "forest_hypotheses": (161393152 + 7238400) / 32,
+    "query_raycast": (1062682368 + 148070912) / 32,
+    "forest_eval": (101005056 + 64423936) / 32,
+    "forest_hypotheses": (161174784 + 9449472) / 32,
     "forest_verify": (654187520 + 6215424) / 32,
 }
-# What limits each stage's main kernel (profiles/attempt_kernels_house_640x480_batch128.md,
-# profiles/forest_kernel_house_640x480_batch32.md and profiles/raycast_apron_house_640x480_batch32.md; the roofline fraction divides by DRAM
+# What limits each stage's main kernel (profiles/kernels_house_640x480_batch32.md,
+# profiles/attempt_kernels_house_640x480_batch128.md and profiles/raycast_apron_house_640x480_batch32.md; the roofline fraction divides by DRAM
 # bandwidth or an integer-issue peak; these kernels gather from L2 and are bound elsewhere).
 PROFILED_LIMITER = {
     "query_raycast": "instruction issue (74 % active at 63 % warps active; 23.5 of 32 lanes per instruction as rays "
                      "end at different steps); DRAM 17 % of peak, L2 hit 51 %",
-    "forest_eval": "instruction issue (65 % active at 97 % warps active, about 58 instructions per node "
-                   "visit) and dependent node and probe loads (L1 hit 23 %, L2 hit 98 %)",
-    "forest_hypotheses": "L2 throughput (63 %, L2 hit 98 %): four random 16-byte gathers per try",
+    "forest_eval": "instruction issue (74 % active at 98 % warps active, about 58 instructions per node "
+                   "visit), L1 data pipe 64 %, L2 hit 95 %",
+    "forest_hypotheses": "L1 data pipe (82 %, a gathered lane per cycle per SM): four random 16-byte gathers per try",
     "forest_verify": "instruction issue (74 % active at 61 % warps active; 23.2 of 32 lanes per instruction); "
                      "DRAM 11 % of peak, L2 hit 54 %",
 }
