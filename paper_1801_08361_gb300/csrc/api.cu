@@ -1034,9 +1034,10 @@ relo_status relo_create_forest(const void* nodes, int32_t T, int32_t D, const fl
         const size_t first = (size_t)1 << level;  // nodes above this level, and in it
         int4 nd = in_nodes[(size_t)t * n_int + first - 1 + p];
         const int kind = nd.z & 0xFF, c1 = (nd.z >> 8) & 0xFF, c2 = (nd.z >> 16) & 0xFF;
-        // planes 128 (1 + c); channel 3 reads plane b of a tiled image and is marked by bit 0
+        // planes 128 (1 + c); channel 3, which a tiled image does not hold, is marked by bit 0
         auto plane = [](int c) { return c == 3 ? 0x181 : 128 * (1 + c); };
         nd.z = kind == 0 ? 0 : plane(c1) | plane(c2) << 16;
+        if (kind == 1 && (c1 == 3 || c2 == 3)) f->reads_alpha = true;
         nd.w = std::min(std::max(nd.w, -65536), 65536);
         for (int* w : {&nd.x, &nd.y}) {
           const int lo = (int)(int16_t)(*w & 0xFFFF) * scale, hi = (int)(int16_t)((uint32_t)*w >> 16) * scale;
@@ -2323,11 +2324,11 @@ void layout_batch(const relo_attempt* at, int n, const relo_ransac_params& p, ch
       fill_ransac_job(r, a.forest_a->view, depth, leaves, a.intr, p, K, a.seed);
       carve_ransac(c, r, W, H, K, p.batch, r.n_rounds, T);
       // the query raycast also writes the image in tiles, which the forest reads; the valid-pixel table
-      // is written after the forest has run and may take its place
+      // is written after the forest has run and may take its place.  (A forest that reads alpha takes the
+      // depth and colour images: a tile holds depth, r, g and b.)
       const size_t tiled = tiled_values(W, H);
       uint16_t* image = tiled * sizeof(uint16_t) <= n_pix * r.nv * sizeof(uint4) ? (uint16_t*)r.table : c.take<uint16_t>(tiled);
-      h.query[i].tiled = image;
-      f.tiled = image;
+      if (!a.forest_a->reads_alpha) f.tiled = h.query[i].tiled = image;
       // one error word per attempt: a learned attempt's forest fallback shares the learned word
       r.err = iL[i] >= 0 ? b.d_errs + iL[i] : b.d_errs + nL + j;
       r.result = b.d_res_F + i;

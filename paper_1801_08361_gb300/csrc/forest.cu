@@ -97,7 +97,8 @@ __device__ __forceinline__ int probe(int x, int raw, const DepthDivisor& dv, int
 // 256 house images of five trees: 11.5 ms, 12.8 with pixels in rows and nodes a tree at a time; the L1 is
 // then at 64 % and the instructions bound it.  32 fragment views: 0.50 ms, 0.54 before.
 // Plane of a probe in a node's third word: its byte offset in a tile, 0 the depths, 128 (1 + c) channel c;
-// bit 0 marks channel 3, the alpha of the colour image, which a tiled image does not hold (it reads b).
+// bit 0 marks channel 3, the alpha of the colour image, which a tiled image does not hold: forests with
+// such a node read the colour image itself.
 constexpr unsigned kPlaneMask = 0x380u;
 __device__ __forceinline__ unsigned plane_shift(unsigned z) { return 8u * (((z & kPlaneMask) >> 7) - 1u + (z & 1u)); }
 

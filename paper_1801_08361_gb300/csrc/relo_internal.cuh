@@ -510,7 +510,8 @@ struct ForestJob {
   const int4* nodes;           // as ForestView
   const uint16_t* depth;
   const uint32_t* rgba;
-  const uint16_t* tiled;       // nullable: the same image in 8 x 8 tiles, row-major, each [depth, r, g, b][8][8] u16
+  const uint16_t* tiled;       // nullable (null for a forest that reads alpha): the same image in 8 x 8 tiles,
+                               // row-major, each [depth, r, g, b][8][8] u16
   uint16_t* leaves;            // [T][H][W]
   const int32_t* skip;         // when set and non-zero the job does nothing (fallback not needed)
   int32_t W, H;
@@ -818,6 +819,7 @@ struct relo_forest {
   void* d_n_modes;
   void* d_top;
   int32_t T, D, M;
+  bool reads_alpha;  // some node compares colour channel 3
   // training state
   relo_train_params train;
   bool training;

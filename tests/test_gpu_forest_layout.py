@@ -68,3 +68,26 @@ def test_tiled_images(room, room_training):
                 T, _, W, H = shapes[i]
                 d, c, lv = (x.cpu().numpy() for x in bt.attempt_images(k, W, H, trees=T))
                 assert np.array_equal(lv.view(np.uint16), oracle.forest_eval(nodes[i], d.view(np.uint16), c)), (i, rows)
+
+
+def test_batches_read_alpha(room, room_training):
+    """Forests whose nodes compare channel 3 (0 where a view's ray misses, 255 elsewhere), beside one that
+    has no such node."""
+    world, blocks = room
+    scene = B.Scene(blocks, 16)
+    shapes = [(5, 10, 150, 101, 4), (4, 9, 96, 72, 3), (8, 12, 47, 83, 4)]
+    qs = synth.query_poses(world, [f[1] for f in room_training], len(shapes), seed=12)
+    items, nodes = [], []
+    for i, (T, D, W, H, channels) in enumerate(shapes):
+        nodes.append(_nodes(T, D, 70 + i, channels))
+        f = B.Forest(nodes[i], np.zeros((T, 1 << D, 1, 12)), np.zeros((T, 1 << D)), max_modes=1)
+        items.append(dict(scene_b=scene, forest_a=f, scene_a=scene, intr=synth.Intrinsics.for_size(W, H), pose_b=qs[i],
+                          n_hyps=4, seed=i))
+    prm = B.ransac_params(n_hyps=4, batch=20, max_tries=5)
+    att = B.make_attempts(items)
+    bt = B.Batch(att, prm, torch.empty(B.batch_workspace_size(att, prm), dtype=torch.uint8, device=DEV))
+    bt.run(torch.zeros(len(items) * B.RESULT_BYTES, dtype=torch.uint8, device=DEV))
+    torch.cuda.synchronize()
+    for i, (T, _, W, H, _) in enumerate(shapes):
+        d, c, lv = (x.cpu().numpy() for x in bt.attempt_images(i, W, H, trees=T))
+        assert np.array_equal(lv.view(np.uint16), oracle.forest_eval(nodes[i], d.view(np.uint16), c)), i
