@@ -1117,40 +1117,44 @@ relo_status relo_forest_train_begin(relo_forest* f, const relo_train_params* p) 
 }  // extern "C"
 
 namespace {
-// The reservoirs of the training begun last, allocated (kept from an earlier training of the same
-// size) and zeroed on s.
-relo_status ready_reservoirs(relo_forest* f, cudaStream_t s) {
-  if (f->res_ready) return RELO_OK;
+// The reservoirs of the training begun last (kept from an earlier training of the same size).
+relo_status alloc_reservoirs(relo_forest* f) {
   const size_t L = (size_t)f->T << f->D, slots = L * f->train.capacity;
-  if (f->res_slots != slots) {
-    auto release = [f] {
-      relo::dev_free(f->res_samples);
-      relo::dev_free(f->res_count);
-      relo::dev_free(f->res_seen);
-      relo::dev_free(f->res_runs);
-      f->res_samples = nullptr;
-      f->res_count = nullptr;
-      f->res_seen = nullptr;
-      f->res_runs = nullptr;
-      f->res_slots = 0;
-    };
+  if (f->res_slots == slots) return RELO_OK;
+  auto release = [f] {
+    relo::dev_free(f->res_samples);
+    relo::dev_free(f->res_count);
+    relo::dev_free(f->res_seen);
+    relo::dev_free(f->res_runs);
+    f->res_samples = nullptr;
+    f->res_count = nullptr;
+    f->res_seen = nullptr;
+    f->res_runs = nullptr;
+    f->res_slots = 0;
+  };
+  release();
+  if (relo::dev_malloc((void**)&f->res_samples, slots * 3 * sizeof(float)) != cudaSuccess ||
+      relo::dev_malloc((void**)&f->res_count, L * sizeof(int32_t)) != cudaSuccess ||
+      relo::dev_malloc((void**)&f->res_seen, L * sizeof(int64_t)) != cudaSuccess ||
+      relo::dev_malloc((void**)&f->res_runs, 2 * L * sizeof(int32_t)) != cudaSuccess) {
+    cudaGetLastError();
     release();
-    if (relo::dev_malloc((void**)&f->res_samples, slots * 3 * sizeof(float)) != cudaSuccess ||
-        relo::dev_malloc((void**)&f->res_count, L * sizeof(int32_t)) != cudaSuccess ||
-        relo::dev_malloc((void**)&f->res_seen, L * sizeof(int64_t)) != cudaSuccess ||
-        relo::dev_malloc((void**)&f->res_runs, 2 * L * sizeof(int32_t)) != cudaSuccess) {
-      cudaGetLastError();
-      release();
-      return fail(RELO_ENOMEM, "reservoirs");
-    }
-    f->res_slots = slots;
+    return fail(RELO_ENOMEM, "reservoirs");
   }
-  RELO_CUDA(cudaMemsetAsync(f->res_samples, 0, slots * 3 * sizeof(float), s));
-  RELO_CUDA(cudaMemsetAsync(f->res_count, 0, L * sizeof(int32_t), s));
-  RELO_CUDA(cudaMemsetAsync(f->res_seen, 0, L * sizeof(int64_t), s));
-  RELO_CUDA(cudaMemsetAsync(f->res_runs, 0, 2 * L * sizeof(int32_t), s));
-  f->res_ready = true;
+  f->res_slots = slots;
   return RELO_OK;
+}
+
+// Zeroes a new training's reservoirs on s.  The caller sets res_ready once s has run this, so that a
+// later call on another stream never finds them ready before they are.
+cudaError_t zero_reservoirs(relo_forest* f, cudaStream_t s) {
+  if (f->res_ready) return cudaSuccess;
+  const size_t L = (size_t)f->T << f->D;
+  cudaError_t e = cudaMemsetAsync(f->res_samples, 0, f->res_slots * 3 * sizeof(float), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(f->res_count, 0, L * sizeof(int32_t), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(f->res_seen, 0, L * sizeof(int64_t), s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(f->res_runs, 0, 2 * L * sizeof(int32_t), s);
+  return e;
 }
 
 // Trees whose items are sorted together: the sort's buffers (16 bytes per grid pixel and tree) stay
@@ -1172,8 +1176,6 @@ relo_status relo_forest_train_frame(relo_forest* f, const relo_intrinsics* intr,
   const int gw = (W + S - 1) / S, gh = (H + S - 1) / S;
   const int64_t n = (int64_t)gw * gh;
   cudaStream_t s = (cudaStream_t)stream;
-  st = ready_reservoirs(f, s);
-  if (st) return st;
   ReservoirFrame r{};
   r.depth = depth;
   r.W = W;
@@ -1183,11 +1185,6 @@ relo_status relo_forest_train_frame(relo_forest* f, const relo_intrinsics* intr,
   r.D = f->D;
   r.per_block = (int)std::max<int64_t>(kSortItems, ((n + kSortBlocks - 1) / kSortBlocks + 255) / 256 * 256);
   r.blocks = (int)((n + r.per_block - 1) / r.per_block);
-  r.start = f->res_runs;
-  r.end = f->res_runs + ((size_t)T << f->D);
-  r.samples = f->res_samples;
-  r.count = f->res_count;
-  r.seen = f->res_seen;
   r.capacity = f->train.capacity;
   r.key0 = (uint32_t)(f->train.seed & 0xFFFFFFFFu);
   r.key1 = (uint32_t)(f->train.seed >> 32);
@@ -1216,10 +1213,18 @@ relo_status relo_forest_train_frame(relo_forest* f, const relo_intrinsics* intr,
     }
     f->scratch_bytes = need;
   }
+  st = alloc_reservoirs(f);
+  if (st) return st;
+  r.start = f->res_runs;
+  r.end = f->res_runs + ((size_t)T << f->D);
+  r.samples = f->res_samples;
+  r.count = f->res_count;
+  r.seen = f->res_seen;
   layout((char*)f->d_scratch);
   r.coords = coords;
   const ForestJob j = make_forest_job(f->view, depth, (const uint32_t*)rgba, leaves, W, H);
-  cudaError_t e = launch_forest_grid(j, S, s);
+  cudaError_t e = zero_reservoirs(f, s);
+  if (e == cudaSuccess) e = launch_forest_grid(j, S, s);
   if (e == cudaSuccess) e = launch_scene_coords(depth, W, H, S, intr->fx, intr->fy, intr->cx, intr->cy, pose, coords, s);
   for (int t = 0; e == cudaSuccess && t < T; t += step) {
     r.leaves = leaves + (size_t)n * t;
@@ -1227,8 +1232,10 @@ relo_status relo_forest_train_frame(relo_forest* f, const relo_intrinsics* intr,
     r.trees = std::min(step, T - t);
     e = launch_reservoirs(r, s);
   }
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  const cudaError_t done = cudaStreamSynchronize(s);  // after a failed launch too: nothing of this call stays in flight
+  if (e == cudaSuccess) e = done;
   if (e != cudaSuccess) return cuda_fail(e, "training frame");
+  f->res_ready = true;
   return RELO_OK;
 }
 
@@ -1249,17 +1256,20 @@ relo_status relo_forest_train_finish(relo_forest* f, relo_stream stream) {
   if (!f || !f->training) return fail(RELO_EINVAL, "training not begun");
   const size_t L = (size_t)f->T << f->D;
   cudaStream_t s = (cudaStream_t)stream;
-  const relo_status st = ready_reservoirs(f, s);
+  const relo_status st = alloc_reservoirs(f);
   if (st) return st;
-  cudaError_t e = cudaMemsetAsync(f->d_modes, 0, L * f->M * kModeFloats * sizeof(float), s);
+  cudaError_t e = zero_reservoirs(f, s);
+  if (e == cudaSuccess) e = cudaMemsetAsync(f->d_modes, 0, L * f->M * kModeFloats * sizeof(float), s);
   if (e == cudaSuccess)
     e = launch_mean_shift(f->res_samples, f->res_count, f->train.capacity, (int)L, (float)f->train.bandwidth,
                           (float)f->train.tol, f->train.max_iter, (float)f->train.merge_dist, (float)f->train.cov_floor,
                           f->M, (float*)f->d_modes, (uint8_t*)f->d_n_modes, s);
   if (e == cudaSuccess) e = launch_top_modes((const float*)f->d_modes, (const uint8_t*)f->d_n_modes, (int)L, f->M,
                                              (float4*)f->d_top, s);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  const cudaError_t done = cudaStreamSynchronize(s);
+  if (e == cudaSuccess) e = done;
   if (e != cudaSuccess) return cuda_fail(e, "mean shift");
+  f->res_ready = true;
   return RELO_OK;
 }
 

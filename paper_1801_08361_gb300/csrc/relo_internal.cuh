@@ -823,7 +823,8 @@ struct relo_forest {
   // training state
   relo_train_params train;
   bool training;
-  // reservoirs on the device, allocated and zeroed by the first frame after train_begin
+  // reservoirs on the device, allocated and zeroed by the first frame after train_begin (res_ready: that
+  // frame has run)
   bool res_ready;
   float* res_samples;   // [T][L][cap][3]
   int32_t* res_count;   // [T][L]

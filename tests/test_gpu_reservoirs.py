@@ -9,6 +9,7 @@ import torch
 import oracle
 from paper_1801_08361_gb300 import binding as B
 from paper_1801_08361_gb300 import synth
+from test_gpu_allocator import Counting
 
 pytestmark = pytest.mark.gpu
 DEV = torch.device("cuda:0")
@@ -49,3 +50,45 @@ def test_reservoirs_match_the_oracle(trees, depth, capacity, stride, W, H, flat)
         assert np.array_equal(samples, so)
         if flat:
             assert count[:, -1].min() == min(capacity, 2 * len(range(0, W, stride)) * len(range(0, H, stride)))
+
+
+class Limited(Counting):
+    limit = 0
+
+    def alloc(self, n):
+        return super().alloc(n) if n <= self.limit else 0
+
+
+@pytest.fixture
+def limited():
+    a = Limited()
+    yield a
+    B.set_allocator()
+
+
+def test_a_frame_without_room_leaves_nothing_behind(limited):
+    """Room for the reservoirs (4 KB) but not for the frame's scratch (16 bytes a pixel at least): the frame
+    fails with nothing allocated or under way, so the next one, on another stream, starts a training."""
+    W, H = 64, 48
+    nodes = synth.random_forest_nodes(2, 4, seed=9)
+    f = B.Forest(nodes, max_modes=4)
+    intr, pose = synth.Intrinsics.for_size(W, H, 12.0), synth.look_pose(np.array([1.0, 2.0, 1.5]), 0.3, -0.1)
+    (d, c), *_ = _frames(W, H, False, 3)
+    dd, cc = torch.from_numpy(d.view(np.int16)).to(DEV), torch.from_numpy(c).to(DEV)
+    torch.cuda.synchronize()
+    B.forest_train_begin(f, B.train_params(capacity=8, stride=1, seed=5))
+    limited.limit = 16 * W * H
+    B.set_allocator(limited.alloc, limited.free)
+    with pytest.raises(B.ReloError) as e:
+        B.forest_train_frame(f, intr, pose, dd, cc)
+    assert e.value.status == B.ENOMEM
+    assert not limited.live
+    samples, count = B.forest_train_reservoirs(f, 8)
+    assert not samples.any() and not count.any()
+    B.set_allocator()
+    B.forest_train_frame(f, intr, pose, dd, cc, torch.cuda.Stream())
+    want = oracle.Reservoirs(nodes, oracle.LeafParams(capacity=8, max_modes=4, seed=5, stride=1))
+    want.add_frame(intr, pose, d, c)
+    samples, count = B.forest_train_reservoirs(f, 8)
+    so, co = want.contents()
+    assert np.array_equal(count, co) and np.array_equal(samples, so)
