@@ -387,6 +387,7 @@ def run_ours(args):
         B.raycast_view(scene, intr, P, depth, rgba, noise_dev=nz)
         B.forest_train_frame(forest, intr, P, depth, rgba)
     B.forest_train_finish(forest)
+    B.forest_train_end(forest)
     del depth, rgba
 
     A = args.batch
@@ -842,6 +843,7 @@ def tiny_section(args, B, synth, torch, dev, stream, flush):
         B.raycast_view(scene, intr, P, depth, rgba, noise_dev=nz)
         B.forest_train_frame(forest, intr, P, depth, rgba)
     B.forest_train_finish(forest)
+    B.forest_train_end(forest)
     qs = synth.query_poses(world, train, TINY_ATTEMPTS, seed=31)
     prm = B.ransac_params(n_hyps=TINY.hypotheses[0], batch=TINY.batch_pixels, max_tries=TINY.max_tries)
     items = [dict(scene_b=scene, forest_a=forest, scene_a=scene, intr=intr, pose_b=qs[k], noise=None, seed=0)

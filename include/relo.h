@@ -268,9 +268,11 @@ relo_status relo_forest_eval(const relo_forest* forest, const uint16_t* depth_de
  * device and offers each pixel's scene coordinate P * backproject(depth) to its leaf's
  * reservoir (Algorithm R, capacity per leaf, Philox4x32-10 draws keyed by seed at counter
  * (3, tree * 2^depth + leaf, n_lo, n_hi) for the n-th offer, n from 0; the offer replaces
- * slot floor(word0 * (n+1) / 2^32) if that is below capacity).  The reservoirs live on the device
- * (12 bytes per leaf and slot), from the first frame until the forest is destroyed or a training of
- * another size begins (synchronous call).  relo_forest_train_finish runs mean shift on every
+ * slot floor(word0 * (n+1) / 2^32) if that is below capacity; synchronous call).  The reservoirs live
+ * on the device (12 bytes per leaf and slot and 20 per leaf), from the first frame until
+ * relo_forest_train_end, a training of another size or the forest's end.  A frame's scratch (per grid
+ * pixel 12 bytes and 2 a tree, and 16 a tree up to half a gigabyte in all or one tree's) is kept for the
+ * next frame; relo_forest_train_finish gives a scratch over 16 MB back.  It runs mean shift on every
  * leaf (Gaussian kernel of the given bandwidth from every sample, until the shift is below
  * tol or max_iter steps; a converged point joins the first mode whose opening point lies
  * within merge_dist; per mode: mean and covariance of its members + cov_floor I; keep the
@@ -286,6 +288,9 @@ relo_status relo_forest_train_begin(relo_forest* forest, const relo_train_params
 relo_status relo_forest_train_frame(relo_forest* forest, const relo_intrinsics* intr, const double pose_c2s[16],
                                     const uint16_t* depth_dev, const uint8_t* rgba_dev, relo_stream stream);
 relo_status relo_forest_train_finish(relo_forest* forest, relo_stream stream);
+/* Ends the training: its device memory goes back, and frames need a new begin; the modes stay.  Waits for
+ * the device when there is memory to give back.  Errors: RELO_EINVAL (null forest). */
+relo_status relo_forest_train_end(relo_forest* forest);
 /* Reservoir contents (host copies, synchronous): samples [T][2^D][capacity][3], count [T][2^D]. */
 relo_status relo_forest_train_reservoirs(const relo_forest* forest, float* samples_host, int32_t* count_host);
 

@@ -115,6 +115,7 @@ _SIGS = {
     "relo_forest_train_begin": (c_i32, [c_vp, ctypes.POINTER(TrainParams)]),
     "relo_forest_train_frame": (c_i32, [c_vp, ctypes.POINTER(Intrinsics), ctypes.POINTER(c_dbl), c_vp, c_vp, c_vp]),
     "relo_forest_train_finish": (c_i32, [c_vp, c_vp]),
+    "relo_forest_train_end": (c_i32, [c_vp]),
     "relo_forest_train_reservoirs": (c_i32, [c_vp, c_vp, c_vp]),
     "relo_ransac_workspace_size": (ctypes.c_size_t, [c_i32, c_i32, ctypes.POINTER(RansacParams)]),
     "relo_ransac_relocalise": (c_i32, [c_vp, c_vp, c_vp, ctypes.POINTER(Intrinsics), ctypes.POINTER(RansacParams),
@@ -454,6 +455,11 @@ def forest_train_frame(forest, intr, pose, depth_dev, rgba_dev, stream=None):
 
 def forest_train_finish(forest, stream=None):
     _check(lib().relo_forest_train_finish(forest.handle, _stream(stream)))
+
+
+def forest_train_end(forest):
+    """Give the training's device memory back (reservoirs of 12 bytes per leaf and slot); the modes stay."""
+    _check(lib().relo_forest_train_end(forest.handle))
 
 
 def forest_train_reservoirs(forest, capacity):

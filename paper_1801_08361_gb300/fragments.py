@@ -61,6 +61,7 @@ def build(dev, keep_blocks=()):
                     B.raycast_view(sc, intr, P, depth, rgba, noise_dev=nz)
                     B.forest_train_frame(fo, intr, P, depth, rgba)
             B.forest_train_finish(fo)
+            B.forest_train_end(fo)
             scenes.append(sc)
             forests.append(fo)
     return world, frags, scenes, forests, kept

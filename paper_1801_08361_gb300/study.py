@@ -72,6 +72,7 @@ def build_fragments(n_fragments, seed=3, train_per_room=12, capacity=1024, dev=N
                 B.raycast_view(f["scene"], intr, P, depth, rgba, noise_dev=nz)
                 B.forest_train_frame(f["forest"], intr, P, depth, rgba)
             B.forest_train_finish(f["forest"])
+            B.forest_train_end(f["forest"])
     return world, frags, intr
 
 

@@ -92,3 +92,36 @@ def test_a_frame_without_room_leaves_nothing_behind(limited):
     samples, count = B.forest_train_reservoirs(f, 8)
     so, co = want.contents()
     assert np.array_equal(count, co) and np.array_equal(samples, so)
+
+
+@pytest.mark.parametrize("W,H,kept", [(64, 48, 16 << 20), (700, 600, 0)])
+def test_training_gives_its_memory_back(limited, W, H, kept):
+    """finish gives a scratch of over 16 MB back (700 x 600 pixels take 12 + 2 * 18 bytes each), end the
+    reservoirs and the rest; reading and going on after finish are as before it, after end the training is over
+    and the modes stay."""
+    nodes = synth.random_forest_nodes(2, 4, seed=9)
+    intr, pose = synth.Intrinsics.for_size(W, H, 12.0), synth.look_pose(np.array([1.0, 2.0, 1.5]), 0.3, -0.1)
+    limited.limit = 1 << 30
+    B.set_allocator(limited.alloc, limited.free)
+    f = B.Forest(nodes, max_modes=4)
+    own = dict(limited.live)
+    want = oracle.Reservoirs(nodes, oracle.LeafParams(capacity=8, max_modes=4, seed=5, stride=1))
+    B.forest_train_begin(f, B.train_params(capacity=8, stride=1, seed=5))
+    for d, c in _frames(W, H, False, 3):
+        want.add_frame(intr, pose, d, c)
+        B.forest_train_frame(f, intr, pose, torch.from_numpy(d.view(np.int16)).to(DEV), torch.from_numpy(c).to(DEV))
+        B.forest_train_finish(f)
+        held = sum(n for q, (_, n) in limited.live.items() if q not in own)
+        assert held <= 2 * 16 * (12 * 8 + 20) + kept
+        samples, count = B.forest_train_reservoirs(f, 8)
+        so, co = want.contents()
+        assert np.array_equal(count, co) and np.array_equal(samples, so)
+    modes = f.get_modes()
+    B.forest_train_end(f)
+    assert limited.live == own
+    assert all(np.array_equal(a, b) for a, b in zip(f.get_modes(), modes)) and modes[1].any()
+    with pytest.raises(B.ReloError) as e:
+        B.forest_train_frame(f, intr, pose, torch.zeros((H, W), dtype=torch.int16, device=DEV),
+                             torch.zeros((H, W, 4), dtype=torch.uint8, device=DEV))
+    assert e.value.status == B.EINVAL
+    B.forest_train_end(f)
