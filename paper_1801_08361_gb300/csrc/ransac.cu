@@ -843,8 +843,9 @@ __global__ void draw_kernel(const RansacJob* __restrict__ jobs, const int32_t* _
 // (its record's mode ranges, then the modes), which is what bound the round kernels: the copies are
 // asynchronous into two slots per warp, so that the next pixel's modes arrive while this one is
 // scored, and the ranges are read a pixel earlier still.
-constexpr int kStageModes = 60;  // modes per warp slot (two slots of 8 warps fit 48 KB); a pixel with
-                                 // more is scored from global memory
+constexpr int kStageModes = 64;  // modes per warp slot (two slots of 8 warps take 48 KB, what a static array may);
+                                 // a pixel with more is scored from global memory, which takes two to three times
+                                 // as long (4 trees of 16 modes, 64 hypotheses, 500 pixels: 270 us staged, 731 not)
 
 struct ModeSlot {
   float4 m[kStageModes * 3];
@@ -1006,12 +1007,17 @@ __device__ __forceinline__ void for_staged_pixels(const RansacJob& job, const in
 // rounds (a job of two hypotheses has one).
 __device__ __forceinline__ bool split_scores(const RansacJob& job, int n_split) { return n_split > 1 && job.K > 2; }
 
+// Shared memory of the energies: the warps' mode slots, then (the pixels all scored) their sums.
+union EnergyShared {
+  ModeSlots slots[kRoundWarps];
+  float part[kRoundWarps][32];
+};
+
 // Energies of round r for hypotheses chunk * 32 .. + 31 of job jid.  n_split > 1: only the pixels of
 // part `split`, whose scores go to the job's score buffer [pixel][alive hypothesis] instead, for
 // sum_scores to add in the same order.
 __device__ __forceinline__ void energy_block(const RansacJob* __restrict__ jobs, const int32_t* __restrict__ alive_prefix,
-                                             int r, int chunk, int jid, int split, int n_split, ModeSlots* slots,
-                                             float (*part)[32]) {
+                                             int r, int chunk, int jid, int split, int n_split, EnergyShared& sh) {
   const int n_alive = alive_prefix[jid + 1] - alive_prefix[jid];
   if (chunk * 32 >= n_alive) return;
   const RansacJob& job = jobs[jid];
@@ -1029,7 +1035,7 @@ __device__ __forceinline__ void energy_block(const RansacJob* __restrict__ jobs,
   const int row0 = to_scores ? split * per : 0, row1 = to_scores ? min(rows, row0 + per) : rows;
   float* scores = reinterpret_cast<float*>(job.refit);
   for_staged_pixels(job, job.pix + (size_t)r * job.B * job.hs, job.hs, row0 * kRoundWarps + warp,
-                    min(row1 * kRoundWarps, job.B), kRoundWarps, slots[warp], lane,
+                    min(row1 * kRoundWarps, job.B), kRoundWarps, sh.slots[warp], lane,
                     [&](int i, float3 c, const ModeSlot& slot, int n_staged) {
                       const float3 x = apply(P, c);
                       const float best =
@@ -1043,14 +1049,15 @@ __device__ __forceinline__ void energy_block(const RansacJob* __restrict__ jobs,
                       }
                     });
   if (to_scores) return;
-  if (sub == 0) part[warp][lane >> g] = sum;
+  __syncthreads();  // the slots are read
+  if (sub == 0) sh.part[warp][lane >> g] = sum;
   __syncthreads();
   if (warp == 0 && chunk * 32 + lane < n_alive) {
     const int hl = alive_in(job, r)[chunk * 32 + lane];
     if (job.hyp_ok[hl]) {
       float e = 0.f;
 #pragma unroll
-      for (int w = 0; w < kRoundWarps; ++w) e += part[w][lane];
+      for (int w = 0; w < kRoundWarps; ++w) e += sh.part[w][lane];
       job.energy[hl] += (double)e;
     }
   }
@@ -1065,10 +1072,9 @@ __device__ __forceinline__ void energy_block(const RansacJob* __restrict__ jobs,
 #endif
 __global__ void RELO_ENERGY_BOUNDS energy_kernel(const RansacJob* __restrict__ jobs,
                                                                   const int32_t* __restrict__ alive_prefix, int r) {
-  __shared__ ModeSlots slots[kRoundWarps];
-  __shared__ float part[kRoundWarps][32];
+  __shared__ EnergyShared sh;
   chain_begin();
-  energy_block(jobs, alive_prefix, r, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, slots, part);
+  energy_block(jobs, alive_prefix, r, blockIdx.x, blockIdx.y, blockIdx.z, gridDim.z, sh);
 }
 
 // The energies of a split round from its per-pixel scores: eight lanes per hypothesis take the sums
@@ -1597,8 +1603,7 @@ __device__ __forceinline__ int ld_acquire_gpu(const int32_t* p) {
 constexpr int kPersistThreads = kRoundWarps * 32;
 static_assert(kPersistThreads == kPersistThreadsHost, "the host's item chunks match the CTA size");
 constexpr size_t kPersistSmem = 4096 * (sizeof(unsigned long long) + sizeof(int));  // the largest sort
-static_assert(sizeof(ModeSlots) * kRoundWarps + sizeof(float) * kRoundWarps * 32 <= kPersistSmem &&
-                  sizeof(RefineShared) <= kPersistSmem,
+static_assert(sizeof(EnergyShared) <= kPersistSmem && sizeof(RefineShared) <= kPersistSmem,
               "round stages fit the persistent kernel's shared memory");
 
 __global__ void __launch_bounds__(kPersistThreads, 2) persistent_kernel(PersistArgs a) {
@@ -1619,8 +1624,6 @@ __global__ void __launch_bounds__(kPersistThreads, 2) persistent_kernel(PersistA
   }
   __syncthreads();
   // phase 2: CTA items
-  ModeSlots* slots = reinterpret_cast<ModeSlots*>(psm);
-  float(*part)[32] = reinterpret_cast<float(*)[32]>(psm + kRoundWarps * sizeof(ModeSlots));
   for (;;) {
     if (threadIdx.x == 0) {
       const int it = atomicAdd(a.ctrl + 1, 1);
@@ -1661,7 +1664,8 @@ __global__ void __launch_bounds__(kPersistThreads, 2) persistent_kernel(PersistA
         draw_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.job);
         break;
       case kItemEnergy:
-        energy_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.sub, it.job, 0, 1, slots, part);
+        energy_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.sub, it.job, 0, 1,
+                     *reinterpret_cast<EnergyShared*>(psm));
         break;
       case kItemSelect:
         select_block(a.jobs, a.alive_prefix + (size_t)it.round * np, it.round, it.job,

@@ -2,8 +2,11 @@
 solves by 16 lanes or by one thread, one to 32 lanes per survivor) give the same results bit for bit:
 an attempt alone equals the same attempt among so many copies that no form for few jobs applies, at
 hypothesis counts around each form's edges and pixel counts that are no multiple of the warps."""
+import numpy as np
 import pytest
 import torch
+
+import oracle
 
 from paper_1801_08361_gb300 import binding as B
 from paper_1801_08361_gb300 import synth
@@ -31,3 +34,34 @@ def test_one_attempt_equals_many(room, room_training, room_forest, hyps, pixels)
         torch.cuda.synchronize()
         got.append(out.view(n, -1))
     assert (got[1] == got[0][0]).all()
+
+
+@pytest.mark.parametrize("counts", [(15, 15, 15, 15), (16, 15, 15, 15), (16, 16, 16, 16), (8,) * 8, (4,) * 16])
+@pytest.mark.parametrize("hyps,pixels", [(3, 17), (256, 40)])
+def test_pixels_of_up_to_64_modes(room_training, room_forest, counts, hyps, pixels):
+    """Scores from staged modes equal those read one by one: the same forest with further modes that never
+    win (a score below any other's) has more than 64 a pixel, which are not staged."""
+    intr, _, d, c = room_training[2]
+    T, D, M = len(counts), 10, 32
+    L = 1 << D
+    rng = np.random.default_rng(hyps + T)
+    trees = np.arange(T) % len(room_forest.modes)
+    modes = np.repeat(room_forest.modes[trees, :, :1], M, 2).astype(np.float32)  # each leaf's first mode, moved about
+    modes[:, :, 1:, :3] += rng.normal(0, 0.05, (T, L, M - 1, 3))
+    real = oracle.forest_eval(room_forest.nodes, d, c)
+    prm = B.ransac_params(n_hyps=hyps, batch=pixels, max_tries=2000, seed=5)
+    ws = torch.empty(B.ransac_workspace_size(intr.width, intr.height, prm), dtype=torch.uint8, device=DEV)
+    du, lu = (torch.from_numpy(np.ascontiguousarray(a, np.uint16).view(np.int16)).to(DEV) for a in (d, real[trees]))
+    nodes = synth.random_forest_nodes(T, D, seed=3)
+    got = []
+    for extra in (0, 65 - sum(counts)):
+        m, n = modes.copy(), np.zeros((T, L), np.uint8)
+        for t, k in enumerate(counts):
+            n[t] = np.where(room_forest.n_modes[trees[t]] > 0, k + (extra if t == 0 else 0), 0)
+            m[t, :, k:, 9] = -1e30
+        res = torch.zeros(B.RESULT_BYTES, dtype=torch.uint8, device=DEV)
+        B.ransac_relocalise(B.Forest(nodes, m, n, max_modes=M), du, lu, intr, prm, ws, res)
+        torch.cuda.synchronize()
+        got.append(res)
+    assert hyps == 3 or B.result_from_bytes(got[0])["status"] == 0  # (three draws may all fail)
+    assert torch.equal(got[0], got[1])
