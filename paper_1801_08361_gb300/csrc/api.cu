@@ -1579,7 +1579,7 @@ void reg_sizes(int W, int H, int* Hs, int* Ws) {
 }
 
 struct RegBuffers {
-  bf16* x = nullptr;                  // [n][H][W][16]
+  bf16* x = nullptr;                  // [H][W][16] an image's padded input (mma.sync path alone)
   bf16* act[kRegLayers] = {};         // act[l] = input of layer l (l >= 1): [n][H_l][W_l][64]
   float* head = nullptr;              // [n][Hc][Wc][8]
   float4* tgt = nullptr;              // [n][Hc][Wc]
@@ -1597,7 +1597,13 @@ void reg_layout(char* base, int n, int W, int H, bool training, RegBuffers& b, s
   Carver c{base, start};
   int Hs[kRegLayers + 1], Ws[kRegLayers + 1];
   reg_sizes(W, H, Hs, Ws);
-  b.x = c.take<bf16>((size_t)n * H * W * 16);
+  size_t part = 0;
+  if (training)
+    for (int l = 0; l < kRegLayers; ++l)
+      part = std::max(part, wgrad_parts(kRegCin[l], n, Hs[l + 1], Ws[l + 1]) * wgrad_partial_floats(kRegCin[l], kRegCoutPad[l]));
+  // the padded input is read by the forward pass alone, so the partial sums share its space
+  b.x = reinterpret_cast<bf16*>(c.take<char>(std::max((size_t)H * W * 16 * sizeof(bf16), part * sizeof(float))));
+  b.partial = reinterpret_cast<float*>(b.x);
   for (int l = 1; l < kRegLayers; ++l) b.act[l] = c.take<bf16>((size_t)n * Hs[l] * Ws[l] * 64);
   const size_t cells = (size_t)n * Hs[kRegLayers] * Ws[kRegLayers];
   b.head = c.take<float>(cells * 8);
@@ -1605,12 +1611,6 @@ void reg_layout(char* base, int n, int W, int H, bool training, RegBuffers& b, s
     b.tgt = c.take<float4>(cells);
     b.ghead = c.take<bf16>(cells * 16);
     for (int l = 0; l < kRegLayers - 1; ++l) b.gpre[l] = c.take<bf16>((size_t)n * Hs[l + 1] * Ws[l + 1] * 64);
-    size_t part = 0;
-    for (int l = 0; l < kRegLayers; ++l)
-      part = std::max(part, wgrad_parts(kRegCin[l], n, Hs[l + 1], Ws[l + 1]) * wgrad_partial_floats(kRegCin[l], kRegCoutPad[l]));
-    // (the padded input is read by the forward pass alone, and only on the mma.sync path)
-    const bool in_x = part * sizeof(float) <= (size_t)n * H * W * 16 * sizeof(bf16);
-    b.partial = in_x ? reinterpret_cast<float*>(b.x) : c.take<float>(part);
     b.loss = c.take<float>(1);
     b.loss_sums = c.take<float>(loss_blocks((int)cells));
     b.counters = c.take<int32_t>(2);
@@ -1623,41 +1623,47 @@ relo_status reg_forward(relo_regressor* r, const RegBuffers& b, const uint16_t* 
                         int W, int H, cudaStream_t s) {
   int Hs[kRegLayers + 1], Ws[kRegLayers + 1];
   reg_sizes(W, H, Hs, Ws);
-  // the tcgen05 first layer reads the images themselves
-  if (!g_conv_tcgen05.load()) RELO_CUDA(launch_input(depth, (const uint32_t*)rgba, (long)n * H * W, b.x, s));
+  const bool tc = g_conv_tcgen05.load();
   RELO_CUDA(cudaMemsetAsync(r->d_status, 0, sizeof(int32_t), s));
   for (int l = 0; l < kRegLayers; ++l) {
-    if (l == 0 && g_conv_tcgen05.load()) {
+    if (l == 0 && tc) {
+      // from the images themselves
       RELO_CUDA(launch_conv_first(depth, (const uint32_t*)rgba, n, H, W, r->d_wk[0], r->d_bias[0], b.act[1], Hs[1], Ws[1],
                                   r->d_status, r->n_sms, s, g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
       continue;
     }
-    if (kRegCoutPad[l] == 64 && g_conv_tcgen05.load()) {
+    if (kRegCoutPad[l] == 64 && tc) {
       // every layer but the head on the tcgen05 tensor cores (TMA-fed implicit GEMM)
       RELO_CUDA(launch_conv_tc(kRegCinPad[l], b.act[l], n, Hs[l], Ws[l], r->d_wk[l], r->d_bias[l],
                                nullptr, b.act[l + 1], Hs[l + 1], Ws[l + 1], kRegStride[l], 1, 1, r->d_status, r->n_sms,
                                s, g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
       continue;
     }
-    if (l == kRegLayers - 1 && g_conv_tcgen05.load()) {
+    if (l == kRegLayers - 1 && tc) {
       RELO_CUDA(launch_conv_head(b.act[l], n, Hs[l], Ws[l], r->d_wk[l], r->d_bias[l], b.head, r->d_status, r->n_sms, s,
                                  g_conv_timeout_ns.load(), g_conv_stall_tile.load()));
       continue;
     }
     ConvArgs a{};
-    a.in = l == 0 ? b.x : b.act[l];
+    a.in = l > 0 ? b.act[l] : b.x;
     a.w = r->d_wk[l];
     a.bias = r->d_bias[l];
     a.out = l < kRegLayers - 1 ? b.act[l + 1] : nullptr;
     a.out_f32 = l == kRegLayers - 1 ? b.head : nullptr;
-    a.B = n;
+    a.B = l > 0 ? n : 1;
     a.Hi = Hs[l];
     a.Wi = Ws[l];
     a.Ho = Hs[l + 1];
     a.Wo = Ws[l + 1];
     a.stride = kRegStride[l];
     a.relu = l < kRegLayers - 1;
-    RELO_CUDA(launch_conv(kRegCinPad[l], kRegCoutPad[l] / 8, a, r->n_sms, s));
+    for (int i = 0; l == 0 && i < n; ++i) {  // an image at a time through the padded input
+      const size_t px = (size_t)i * H * W;
+      RELO_CUDA(launch_input(depth + px, (const uint32_t*)rgba + px, (long)H * W, b.x, s));
+      a.out = b.act[1] + (size_t)i * Hs[1] * Ws[1] * 64;
+      RELO_CUDA(launch_conv(kRegCinPad[0], kRegCoutPad[0] / 8, a, r->n_sms, s));
+    }
+    if (l > 0) RELO_CUDA(launch_conv(kRegCinPad[l], kRegCoutPad[l] / 8, a, r->n_sms, s));
   }
   return RELO_OK;
 }

@@ -67,3 +67,12 @@ def test_gradients_match_the_oracle(params, W, H, n):  # noqa: F811
     lo, want = _oracle_gradients(view, params, bf16_storage=True)
     assert abs(reg_loss - lo) <= 1e-2 * abs(lo)
     assert min(_cosines(_unflat(grads, params), want)) >= 0.99
+
+
+@pytest.mark.parametrize("n,W,H", [(1, 64, 48), (16, 160, 120), (64, 640, 480)])
+def test_workspaces_hold_one_padded_image(n, W, H):
+    """Activations of 64 channels at 1/2, 1/4 and (six times) 1/8 of the size and the head's 32 bytes a cell; the
+    padded input of the mma.sync path, 32 bytes a pixel, of one image; 256 bytes of alignment per buffer."""
+    px = W * H
+    forward = 128 * n * (px // 4 + px // 16 + 5 * px // 64) + 32 * n * px // 64
+    assert B.regressor_workspace_size(n, W, H, False) <= forward + 32 * px + 16 * 256
