@@ -1668,6 +1668,9 @@ relo_status reg_forward(relo_regressor* r, const RegBuffers& b, const uint16_t* 
   return RELO_OK;
 }
 
+// Kernels that reg_forward launches.
+int forward_launches(int n) { return g_conv_tcgen05.load() ? kRegLayers : kRegLayers - 1 + 2 * n; }
+
 relo_status reg_backward(relo_regressor* r, const RegBuffers& b, const uint16_t* depth, const uint8_t* rgba, int n, int W,
                          int H, cudaStream_t s) {
   int Hs[kRegLayers + 1], Ws[kRegLayers + 1];
@@ -2440,7 +2443,7 @@ relo_status issue_batch(relo_batch* b, relo_pose_result* results, cudaStream_t s
     relo_status st = reg_forward(b->reg, b->regbuf, b->depth_L, (const uint8_t*)b->rgba_L, b->nL, b->lW, b->lH, s);
     if (st) return st;
     RELO_CUDA(launch_cell_forest(b->cells, s));
-    L += 1 + kRegLayers + 1;
+    L += forward_launches(b->nL) + 1;
   }
   RELO_CUDA(mark(b, 2, s, capturing));
   const bool ev = b->timing;
@@ -2576,7 +2579,7 @@ relo_status relo_batch_attempt_images(const relo_batch* b, int32_t k, const uint
 int32_t relo_batch_launch_count(const relo_batch* b) {
   if (!b) return 0;
   int L = 2 + 1;  // result init + query raycast, merge
-  if (b->nL > 0) L += 1 + kRegLayers + 1 + 2 + pass_launches(b->passL, b->sched);
+  if (b->nL > 0) L += forward_launches(b->nL) + 1 + 2 + pass_launches(b->passL, b->sched);
   if (b->nF > 0) L += forest_launches(b->nF) + 2 + pass_launches(b->passF, b->sched);
   return L;
 }
