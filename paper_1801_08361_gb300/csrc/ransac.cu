@@ -799,9 +799,9 @@ cudaError_t launch_hypotheses(const RansacJob* jobs, int n_jobs, int total_hyps,
   // warps resident at once against the hypotheses: share each hypothesis among 16 or 4 warps while
   // that keeps to about one and a half rounds of them
   const int slots = sms * ctas * kSearchWarps;
-  if (total_hyps * 16 <= RELO_SEARCH_WIDE * slots / 2)
+  if (total_hyps <= RELO_SEARCH_WIDE * slots / 32)
     search_shared_kernel<16><<<std::min(total_hyps, std::max(1, slots / 16)), 512, 0, s>>>(jobs, n_jobs, total_hyps, counter);
-  else if (total_hyps * 4 <= RELO_SEARCH_SHARED * slots / 2)
+  else if (total_hyps <= RELO_SEARCH_SHARED * slots / 8)
     search_shared_kernel<4><<<std::min(total_hyps, std::max(1, slots / 4)), 128, 0, s>>>(jobs, n_jobs, total_hyps, counter);
   else
     search_kernel<<<std::min(sms * ctas, (total_hyps + kSearchWarps - 1) / kSearchWarps), kSearchWarps * 32, 0, s>>>(
