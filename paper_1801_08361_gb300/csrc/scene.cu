@@ -272,8 +272,10 @@ constexpr int kTile = 16;
 #endif
 
 // kFew: launches of at most kFewTiles CTAs an SM, which are resident together however many registers a
-// thread takes: 64 of them, so nothing spills in the march, whose latency such a launch waits for.
-// A house view of 300 x 220 (266 CTAs): 73 us for the call, 75 with the spills.
+// thread takes: 64 of them, so nothing spills in the march, whose latency such a launch waits for.  Views
+// of 160 x 120 to 400 x 300, device time with and without: room 52.4 / 53.9 us at 320 x 240, house 60.5 / 61.9
+// (1.5 to 3.4 % over the sizes, repeats within 0.1 %), a scene without its apron copy 101 / 104, through the
+// hash alone 237 / 258.  Not growing scenes, whose five CTAs an SM leave 48: 121.6 / 120.6.
 constexpr int kFewTiles = 4;
 
 template <bool kColour, bool kCompare, bool kTiled, int kMode, bool kFew>
@@ -422,10 +424,11 @@ cudaError_t launch_raycast(const RayJob* jobs_dev, int n_jobs, const RayJob* sin
   auto launch = [&](auto few) {
     constexpr bool kFew = decltype(few)::value;
     if (mode == kSceneApron) launch_raycast_t<kSceneApron, kFew>(jobs_dev, n_jobs, one, total_tiles, with_colour, tiled, compare, s, w);
-    else if (mode == kSceneCells) launch_raycast_t<kSceneCells, kFew>(jobs_dev, n_jobs, one, total_tiles, with_colour, tiled, compare, s, w);
     else launch_raycast_t<kSceneAny, kFew>(jobs_dev, n_jobs, one, total_tiles, with_colour, tiled, compare, s, w);
   };
-  if (total_tiles <= kFewTiles * sms) launch(std::true_type{});
+  if (mode == kSceneCells)
+    launch_raycast_t<kSceneCells, false>(jobs_dev, n_jobs, one, total_tiles, with_colour, tiled, compare, s, w);
+  else if (total_tiles <= kFewTiles * sms) launch(std::true_type{});
   else launch(std::false_type{});
   return cudaGetLastError();
 }
