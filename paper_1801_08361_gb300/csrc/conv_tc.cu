@@ -41,9 +41,9 @@ constexpr int kTcM = 128, kTcN = 64;
 constexpr int kTcAccCols = 64;              // FP32 columns of one accumulator
 constexpr int kTcTmemCols = 2 * kTcAccCols;
 
-// Per input-channel count CIN (64: the inner layers; 16: the first layer, its 4 channels padded):
-// a pixel row is CIN x 2 bytes, which is also the swizzle span of the operand layout (128 B or 32 B;
-// 8-row atoms of 1024 B or 256 B).
+// Per input-channel count CIN (64: the strided layers but the first; 16: the head's backward-data pass, whose
+// gradients' 4 channels are padded): a pixel row is CIN x 2 bytes, which is also the swizzle span of the
+// operand layout (128 B or 32 B; 8-row atoms of 1024 B or 256 B).
 template <int CIN>
 struct TcShape {
   static constexpr int kRowBytes = CIN * 2;

@@ -507,10 +507,11 @@ __device__ __forceinline__ int try_status(const RansacJob& job, const TryDraw& d
 // Each warp step evaluates 64 tries, two per lane (tries base + lane and base + 32 + lane, whose loads
 // are issued together), and keeps the first one not failing in try order, settling guard-band tries in
 // FP64 in order.  What bounds it is the L1: a gather takes about one cycle per lane, four a try (84 % of
-// the data pipe's peak over a batch).  Tried and slower: queueing the tries that pass their first pair
-// for a dense second stage (house batch 19.2 -> 21.3 ms with the fits and compaction), and testing first
-// pairs from 16-bit position codes in the table, two gathers a try, with such a queue for the one in six
-// that those let through (18.2 ms at best, its second stage a chain of six dependent loads).
+// the data pipe's peak over a batch).  Tried: queueing the tries that pass their first pair for a dense
+// second stage (slower: house batch 19.2 -> 21.3 ms with the fits and compaction).  Testing first pairs
+// from 16-bit position codes in the table, two gathers a try, with such a queue for the one in six that
+// those let through, was faster at four CTAs an SM (18.2 ms of that 19.2, 2 % of the batch; 21.2 ms at
+// five, its second stage a chain of six dependent loads): not kept for a gain that small and a larger table.
 constexpr int kSearchWarps = 4;
 
 // first try of mask (bits = lanes) that passes, settling guard-band statuses in FP64; -1 if none

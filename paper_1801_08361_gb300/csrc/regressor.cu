@@ -225,8 +225,9 @@ cudaError_t launch_conv(int cin, int nt, const ConvArgs& a, int n_sms, cudaStrea
 // added to the sums of all taps, in registers (144 a thread at 64 x 64 channels), by rounded FP32
 // additions -- the tensor core's own additions drop bits, which a chain over hundreds of tiles shows --
 // and one partial per CTA is left to sum.
-// The bias is one more product, with a row of ones.  16 views of 640 x 480: 0.38 ms with the sums for
-// all layers; bound by mma.sync (288 products a scheduler and tile of 64 channels, 17 cycles each).
+// The bias is one more product, with a row of ones.  16 views of 640 x 480: 0.31 ms with the sums for
+// all layers, the first's (wgrad_first_kernel) among them; bound by mma.sync (288 products a scheduler and
+// tile of 64 channels, 17 cycles each).
 // ---------------------------------------------------------------------------------------------
 __device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const bf16* p) {
   const unsigned a = (unsigned)__cvta_generic_to_shared(p);

@@ -70,7 +70,9 @@ constexpr int kRegCin[kRegLayers] = {4, 64, 64, 64, 64, 64, 64, 64};
 constexpr int kRegCout[kRegLayers] = {64, 64, 64, 64, 64, 64, 64, 4};
 constexpr int kRegCinPad[kRegLayers] = {16, 64, 64, 64, 64, 64, 64, 64};
 constexpr int kRegCoutPad[kRegLayers] = {64, 64, 64, 64, 64, 64, 64, 8};
-constexpr int kWgradCtas = 152;  // most CTAs (partial sums per weight) of a backward-weight launch; first layer: four times that
+// Most CTAs (partial sums per weight) of a backward-weight launch, one an SM; first layer: four times that.  A
+// constant, since the order of the sums, so the gradients' bits, and the workspace's size follow it.
+constexpr int kWgradCtas = 152;
 
 // Adam step of all parameters and the operands derived from them (see adam_kernel)
 struct AdamArgs {

@@ -249,7 +249,7 @@ __device__ __forceinline__ void quaternion_pose(double w, double x, double y, do
 // of the error, so two are usual, and what remains is the residual's own rounding: that of FP64
 // rotations.  About 100 FP64 operations where the rotations take 700 a sweep and five sweeps, on a pipe
 // that takes 16 cycles or more a warp.  False (the caller takes horn_jacobi): a relative gap under 5e-4
-// (beyond, the residual's rounding would pass for a step; about one in a thousand random triples),
+// (beyond, the residual's rounding would pass for a step; 0.4 to 1 % of a room's kept triples),
 // no convergence, or entries FP32 cannot hold (zeros, infinities, NaN).
 __device__ __forceinline__ bool horn_refined(const double S_in[9], double (&q)[4]) {
   int top = 0;
